@@ -7,20 +7,31 @@
 // this library's answer for many small fragments.
 //
 // Work items are (fragment, chunk of rows), handed out by a device counter in
-// the order of decreasing fragment size. A block walks its chunk in tiles of
-// THREADS x ITEMS rows: per row the filter column, join key and aggregate inputs
-// load together, then the key's home bucket (one sector: keys, build rows and,
-// when the dimension was built with its group column copied, the group keys),
-// else the group key gathered from the build column at the build row; the
-// aggregates go into the fragment's dense accumulators (group key - group_lo
-// indexes them):
+// the order of decreasing fragment size. Every warp of a block walks its own runs of
+// 128 rows of the chunk: it reads the filter column alone (4 consecutive rows per
+// lane, one vector load) and appends the passing rows to a queue in shared memory;
+// whenever the queue holds 32 x ITEMS rows the warp takes them off, every lane with
+// ITEMS rows: their join keys, then their home buckets (one sector: keys, build rows
+// and, when the dimension was built with its group column copied, the group keys;
+// else the group key is gathered from the build column at the build row) with the
+// aggregate inputs loading beside them; the aggregates go into the fragment's dense
+// accumulators (group key - group_lo indexes them):
 //   * shared mode (small key ranges): block arrays in shared memory, cleared per
 //     work item and added into the fragment's global arrays at its end;
 //   * direct mode: 64-bit reductions straight into the global arrays.
-// Rows of one warp that share lane 0's group are summed with a butterfly first.
 // The emit kernel compacts each fragment's occupied slots into its output in
 // key order (single pass, per-fragment bounded look-back).
+//
+// What bounds it: the lookups' dependent round trips (filter, key, bucket, the next
+// bucket for one key in eight) at 32 warps per SM, then DRAM (49 % busy): 512
+// fragments, 388M rows, 28 B per row of columns and 2.4 GB of tables. Measured on
+// that batch: every row looked up in place 12.8 ms; passing rows queued and looked up
+// by full warps 6.0 ms; the next run's columns prefetched into L2, the items' walks
+// merged and small block arrays 3.8 ms (3.1 TB/s). Blocks of 512 threads with 2 rows
+// in flight per thread (two per SM, 64 registers): 3.8 ms; 256 x 2 4.0 ms, 512 x 4
+// (one per SM, 128 registers) 4.3 ms.
 #include <algorithm>
+#include <type_traits>
 #include <vector>
 
 #include "px_common.cuh"
@@ -29,7 +40,11 @@
 namespace px {
 namespace {
 
-constexpr size_t kSmemAccBudget = 96 * 1024;  // shared-mode block accumulators
+// Shared-mode block accumulators. Direct mode above: 64M rows over 1M-key tables, 3
+// aggregates: 4000 groups take 0.89 ms direct and 1.28 ms with 96 KB block arrays
+// (two such blocks leave the SM no L1 for the table); 1000 groups 0.82 ms shared.
+constexpr size_t kSmemAccBudget = 24 * 1024;
+constexpr uint64_t kRepSlots = 1024;               // shared-mode slots with their replicas, at most
 constexpr int kEmitThreads = 256;
 constexpr int kEmitItems = 8;
 constexpr int kEmitTile = kEmitThreads * kEmitItems;
@@ -44,7 +59,12 @@ struct FragDev {
     // aggregate k reads column pa[k] (width wa[k]) and, for SUM_MUL, pb[k] (wb[k])
     const void* pa[PX_FRAG_MAX_AGGS];
     const void* pb[PX_FRAG_MAX_AGGS];
+    int32_t same[PX_FRAG_MAX_AGGS];  // an earlier SUM of the column pa[k], whose value is reused, or -1
     int32_t op[PX_FRAG_MAX_AGGS], wa[PX_FRAG_MAX_AGGS], wb[PX_FRAG_MAX_AGGS];
+    // the distinct columns a row is read from (filter, key, aggregate inputs)
+    int32_t nstream;
+    int32_t stream_w[PX_FRAG_MAX_COLS + 2];
+    const void* stream[PX_FRAG_MAX_COLS + 2];
     int32_t filter_w, naggs, group_w, count_agg;  // count_agg: a COUNT aggregate, or -1
     TableView t;
     int64_t nbuild;
@@ -52,6 +72,8 @@ struct FragDev {
     int64_t group_lo;
     uint32_t D;      // dense slots
     int32_t shared;  // 1: block accumulators in shared memory
+    uint32_t rep_shift;  // shared mode: 1 << rep_shift replicas of every slot, side by side
+    uint32_t reserved;
     int64_t chunk;   // rows per work item
     unsigned long long* acc;  // [naggs][D]
     uint8_t* occ;             // [D] occupancy flags (only without COUNT)
@@ -97,6 +119,11 @@ __device__ __forceinline__ int find_frag(const int64_t* start, int n, int64_t x)
 
 __device__ __forceinline__ int64_t load_w(const void* p, int w, int64_t i) { return load_int(p, w, i); }
 
+// Starts a copy of [p, p + bytes) into L2 (both multiples of 16).
+__device__ __forceinline__ void prefetch_l2(const void* p, uint32_t bytes) {
+    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
+}
+
 // Adds x (mod 2^64) to a 64-bit value held as 32-bit words lo/hi in shared memory.
 __device__ __forceinline__ void add_split(uint32_t* lo, uint32_t* hi, uint64_t x) {
     const uint32_t xl = static_cast<uint32_t>(x), xh = static_cast<uint32_t>(x >> 32);
@@ -105,115 +132,256 @@ __device__ __forceinline__ void add_split(uint32_t* lo, uint32_t* hi, uint64_t x
     if (add_hi) red_add_shared(hi, add_hi);
 }
 
-// Build row of `key` (not kEmpty) in an unsegmented unique table, or -1; *pay
-// receives the payload value copied beside the key (meaningful when the table
-// holds one).
-__device__ __forceinline__ int32_t probe_row(const TableView& t, uint32_t nb, int64_t key, int32_t* pay) {
-    const Bucket* bp = t.bk + home_bucket(static_cast<uint64_t>(key), nb);
-    for (uint32_t round = 0; round < nb; ++round) {
-        const BucketRegs v = load_bucket(bp);
-        bool end;
-        const int l = bucket_find(v, key, &end);
-        if (l >= 0) {
-            *pay = bucket_pay(v, l);
-            return bucket_row(v, l);
+constexpr int kFilterRows = 4;                  // consecutive rows a lane filters at a time
+constexpr int kWarpRows = 32 * kFilterRows;     // rows a warp filters at a time
+constexpr uint32_t kNone = 0xffffffffu;         // no dense slot
+
+// Rows a warp's queue holds at most: one short of a full take, plus one filter step.
+template <int ITEMS>
+constexpr int kQueue = 32 * ITEMS - 1 + kWarpRows;
+
+// Bit j of the result: row r + j passes lo <= col < hi. A full run of kFilterRows
+// rows below r1 is one aligned vector load (r is a multiple of kFilterRows and the
+// column is 16-byte aligned).
+template <typename T>
+__device__ __forceinline__ uint32_t filter_rows(const T* col, int64_t lo, int64_t hi, int64_t r, int64_t r1) {
+    T v[kFilterRows];
+    uint32_t ok = 0;
+    if (r + kFilterRows <= r1) {
+        if (sizeof(T) == 8) {
+            const longlong2 x = *reinterpret_cast<const longlong2*>(col + r);
+            const longlong2 y = *reinterpret_cast<const longlong2*>(col + r + 2);
+            v[0] = static_cast<T>(x.x);
+            v[1] = static_cast<T>(x.y);
+            v[2] = static_cast<T>(y.x);
+            v[3] = static_cast<T>(y.y);
+        } else if (sizeof(T) == 4) {
+            const int4 x = *reinterpret_cast<const int4*>(col + r);
+            v[0] = static_cast<T>(x.x);
+            v[1] = static_cast<T>(x.y);
+            v[2] = static_cast<T>(x.z);
+            v[3] = static_cast<T>(x.w);
+        } else {
+            const char4 x = *reinterpret_cast<const char4*>(col + r);
+            v[0] = static_cast<T>(x.x);
+            v[1] = static_cast<T>(x.y);
+            v[2] = static_cast<T>(x.z);
+            v[3] = static_cast<T>(x.w);
         }
-        if (end) return -1;
-        bp = bp + 1 == t.bk + nb ? t.bk : bp + 1;
+#pragma unroll
+        for (int j = 0; j < kFilterRows; ++j)
+            ok |= (static_cast<int64_t>(v[j]) >= lo && static_cast<int64_t>(v[j]) < hi ? 1u : 0u) << j;
+    } else {
+#pragma unroll
+        for (int j = 0; j < kFilterRows; ++j)
+            if (r + j < r1) {
+                const int64_t x = static_cast<int64_t>(col[r + j]);
+                ok |= (x >= lo && x < hi ? 1u : 0u) << j;
+            }
     }
-    return -1;
+    return ok;
 }
 
-// Rows [r0, r1) of fragment f. SHARED: accumulate into the block arrays lo/hi
-// ([naggs][D] each) and occupancy bits; else reduce into the global arrays.
-template <int THREADS, int ITEMS, int NA, bool SHARED>
+// Rows [r0, r1) of fragment f (r0 a multiple of kFilterRows). SHARED: accumulate
+// into the block arrays lo/hi ([naggs][D][replicas] each) and occupancy bits; else
+// reduce into the global arrays. `queue`: this warp's kQueue<ITEMS> entries.
+// Only rows that pass the filter touch the key, value and table memory, and every
+// lane of a lookup holds one: with the lookups predicated in place a filter that
+// keeps 30 % of the rows left two lanes of three idle through them (ncu: 19.5
+// threads per instruction).
+// W8: every aggregated column of the batch is 8 bytes wide (no width switches).
+template <int THREADS, int ITEMS, int NA, bool W8, bool SHARED>
 __device__ void frag_rows(const FragDev& f, int64_t r0, int64_t r1, uint32_t* s_lo, uint32_t* s_hi,
-                          uint32_t* s_occ, int32_t* status) {
+                          uint32_t* s_occ, uint32_t* queue, int32_t* status) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t nb = static_cast<uint32_t>(table_buckets(f.t.hdr->nbuild, 1));
     // the group column copied into the table at build time: read with the key
     const bool group_in_table = f.t.hdr->pay_src == f.group && f.t.hdr->pay_w == f.group_w;
     const int naggs = f.naggs;
-    for (int64_t tb = r0; tb < r1; tb += THREADS * ITEMS) {
+    const uint32_t lt = lanemask_lt();
+    const uint32_t rep = SHARED ? static_cast<uint32_t>(lane) & ((1u << f.rep_shift) - 1) : 0;
+    uint32_t held = 0;  // rows in the queue
+
+    // Takes the last `n` (1..32 * ITEMS) rows off the queue and aggregates them.
+    auto take = [&](uint32_t n) {
+        uint32_t row[ITEMS];
         int64_t key[ITEMS], v[NA][ITEMS];
-        bool pass[ITEMS];
+        BucketRegs bv[ITEMS];
+        uint32_t hb[ITEMS];
 #pragma unroll
         for (int i = 0; i < ITEMS; ++i) {
-            const int64_t r = tb + warp * (32 * ITEMS) + i * 32 + lane;
-            const bool valid = r < r1;
-            bool p = valid;
-            if (f.filter && valid) {
-                const int64_t x = load_w(f.filter, f.filter_w, r);
-                p = x >= f.lo && x < f.hi;
-            }
-            pass[i] = p;
-            key[i] = valid ? f.key[r] : kEmpty;
+            const uint32_t e = 32 * i + lane;
+            row[i] = e < n ? queue[held - n + e] : kNone;
+        }
+        __syncwarp();  // the entries are read: the next append may overwrite them
+        held -= n;
 #pragma unroll
-            for (int a = 0; a < NA; ++a) {
-                if (a >= naggs) break;
-                int64_t x = 1;
-                if (f.op[a] != PX_COUNT && valid) {
-                    x = load_w(f.pa[a], f.wa[a], r);
-                    if (f.op[a] == PX_SUM_MUL)
-                        x = static_cast<int64_t>(static_cast<uint64_t>(x) *
-                                                 static_cast<uint64_t>(load_w(f.pb[a], f.wb[a], r)));
-                }
-                v[a][i] = x;
+        for (int i = 0; i < ITEMS; ++i) key[i] = row[i] != kNone ? f.key[r0 + row[i]] : kEmpty;
+#pragma unroll
+        for (int i = 0; i < ITEMS; ++i) {
+            hb[i] = home_bucket(static_cast<uint64_t>(key[i]), nb);
+            bv[i] = load_bucket(f.t.bk + hb[i]);  // hb < nb: inside the table
+        }
+#pragma unroll
+        for (int a = 0; a < NA; ++a) {
+            if (a >= naggs) break;
+            if (f.op[a] == PX_COUNT) continue;
+            const int same = f.same[a];
+            if (same >= 0) {
+#pragma unroll
+                for (int b = 0; b < a; ++b)
+                    if (same == b) {
+#pragma unroll
+                        for (int i = 0; i < ITEMS; ++i) v[a][i] = v[b][i];
+                    }
+            } else {
+#pragma unroll
+                for (int i = 0; i < ITEMS; ++i)
+                    v[a][i] = row[i] != kNone ? load_w(f.pa[a], W8 ? 8 : f.wa[a], r0 + row[i]) : 0;
+            }
+            if (f.op[a] == PX_SUM_MUL) {
+#pragma unroll
+                for (int i = 0; i < ITEMS; ++i)
+                    if (row[i] != kNone)
+                        v[a][i] = static_cast<int64_t>(static_cast<uint64_t>(v[a][i]) *
+                                                       static_cast<uint64_t>(load_w(f.pb[a], W8 ? 8 : f.wb[a], r0 + row[i])));
             }
         }
-        uint32_t slot[ITEMS];  // dense slot of the row's group, or 0xffffffff
+        // The match of every item; the keys displaced past their home bucket (about one
+        // in eight, so some lane of nearly every warp) then walk on together, one round
+        // trip for all of the warp's items.
+        int32_t mrow[ITEMS], mpay[ITEMS];
+        uint32_t pend = 0;
 #pragma unroll
         for (int i = 0; i < ITEMS; ++i) {
-            slot[i] = 0xffffffffu;
-            if (!pass[i] || key[i] == kEmpty) continue;
-            int32_t pay = 0;
-            const int32_t br = probe_row(f.t, nb, key[i], &pay);
-            if (br < 0) continue;
-            const int64_t gk = group_in_table ? static_cast<int64_t>(pay) : load_w(f.group, f.group_w, br);
+            mrow[i] = -1;
+            mpay[i] = 0;
+            if (key[i] == kEmpty) continue;
+            bool end;
+            const int l = bucket_find(bv[i], key[i], &end);
+            if (l >= 0) {
+                mrow[i] = bucket_row(bv[i], l);
+                mpay[i] = bucket_pay(bv[i], l);
+            } else if (!end) {
+                pend |= 1u << i;
+            }
+        }
+        for (uint32_t round = 1; round < nb && pend; ++round) {
+#pragma unroll
+            for (int i = 0; i < ITEMS; ++i)
+                if ((pend >> i) & 1u) {
+                    hb[i] = hb[i] + 1 == nb ? 0 : hb[i] + 1;
+                    bv[i] = load_bucket(f.t.bk + hb[i]);
+                }
+#pragma unroll
+            for (int i = 0; i < ITEMS; ++i)
+                if ((pend >> i) & 1u) {
+                    bool end;
+                    const int l = bucket_find(bv[i], key[i], &end);
+                    if (l >= 0) {
+                        mrow[i] = bucket_row(bv[i], l);
+                        mpay[i] = bucket_pay(bv[i], l);
+                    }
+                    if (l >= 0 || end) pend &= ~(1u << i);
+                }
+        }
+        __syncwarp();
+        uint32_t slot[ITEMS];  // dense slot of the row's group, or kNone
+#pragma unroll
+        for (int i = 0; i < ITEMS; ++i) {
+            slot[i] = kNone;
+            if (mrow[i] < 0) continue;
+            const int64_t gk = group_in_table ? static_cast<int64_t>(mpay[i]) : load_w(f.group, f.group_w, mrow[i]);
             const uint64_t d = static_cast<uint64_t>(gk - f.group_lo);
             if (d < f.D) slot[i] = static_cast<uint32_t>(d);
             else set_status(status, PX_ERR_UNSUPPORTED);
         }
 #pragma unroll
         for (int i = 0; i < ITEMS; ++i) {
-            // Rows sharing lane 0's slot: one butterfly sum, applied once by lane 0.
+            // Rows sharing lane 0's slot: summed across the warp, applied once by lane 0
+            // (not where every lane has a replica of its own).
             uint32_t apply = slot[i];
-            const uint32_t c0 = __shfl_sync(FULL, slot[i], 0);
-            const uint32_t mm = __ballot_sync(FULL, slot[i] == c0);
-            if (c0 != 0xffffffffu && __popc(mm) >= kMajority) {
-                const bool in = (mm >> lane) & 1u;
+            uint32_t cnt = 1;
+            if (!SHARED || f.rep_shift < 5) {
+                const uint32_t c0 = __shfl_sync(FULL, slot[i], 0);
+                const uint32_t mm = __ballot_sync(FULL, slot[i] == c0);
+                if (c0 != kNone && __popc(mm) >= kMajority) {
+                    const bool in = (mm >> lane) & 1u;
 #pragma unroll
-                for (int a = 0; a < NA; ++a) {
-                    if (a >= naggs) break;
-                    const int64_t x = warp_sum(in ? v[a][i] : int64_t(0));
-                    if (lane == 0) v[a][i] = x;
+                    for (int a = 0; a < NA; ++a) {
+                        if (a >= naggs) break;
+                        if (f.op[a] == PX_COUNT) continue;
+                        const uint64_t x = warp_sum_u64(in ? static_cast<uint64_t>(v[a][i]) : 0);
+                        if (lane == 0) v[a][i] = static_cast<int64_t>(x);
+                    }
+                    if (lane == 0) cnt = __popc(mm);
+                    else if (in) apply = kNone;
                 }
-                if (in && lane != 0) apply = 0xffffffffu;
             }
-            if (apply == 0xffffffffu) continue;
+            if (apply == kNone) continue;
             if (SHARED) {
 #pragma unroll
                 for (int a = 0; a < NA; ++a) {
                     if (a >= naggs) break;
-                    const size_t o = static_cast<size_t>(a) * f.D + apply;
-                    add_split(&s_lo[o], &s_hi[o], static_cast<uint64_t>(v[a][i]));
+                    const uint32_t o = ((static_cast<uint32_t>(a) * f.D + apply) << f.rep_shift) + rep;
+                    // a work item counts fewer than 2^32 rows
+                    if (f.op[a] == PX_COUNT) red_add_shared(&s_lo[o], cnt);
+                    else add_split(&s_lo[o], &s_hi[o], static_cast<uint64_t>(v[a][i]));
                 }
                 if (f.count_agg < 0) red_or_shared(&s_occ[apply / 32], 1u << (apply % 32));
             } else {
 #pragma unroll
                 for (int a = 0; a < NA; ++a) {
                     if (a >= naggs) break;
-                    red_add_global(&f.acc[static_cast<size_t>(a) * f.D + apply], static_cast<unsigned long long>(v[a][i]));
+                    red_add_global(&f.acc[static_cast<size_t>(a) * f.D + apply],
+                                   f.op[a] == PX_COUNT ? cnt : static_cast<unsigned long long>(v[a][i]));
                 }
                 if (f.count_agg < 0) f.occ[apply] = 1;  // every writer stores the same value
             }
         }
+    };
+
+    for (int64_t tb = r0 + warp * kWarpRows;; tb += THREADS * kFilterRows) {
+        const bool more = tb < r1;
+        if (more) {
+            // The next run's columns start on their way to L2 while this one is
+            // aggregated (one bulk prefetch per column, lanes 0..ncols+1).
+            const int64_t nt = tb + THREADS * kFilterRows;
+            if (lane < f.nstream && nt < r1) {
+                const int64_t w = f.stream_w[lane];
+                const int64_t bytes = ((r1 - nt < kWarpRows ? r1 - nt : kWarpRows) * w) & ~int64_t(15);
+                if (bytes) prefetch_l2(static_cast<const char*>(f.stream[lane]) + nt * w, static_cast<uint32_t>(bytes));
+            }
+            const int64_t r = tb + kFilterRows * lane;
+            uint32_t ok;
+            if (!f.filter) {
+                ok = r + kFilterRows <= r1 ? (1u << kFilterRows) - 1 : (r < r1 ? (1u << (r1 - r)) - 1 : 0);
+            } else if (f.filter_w == 4) {
+                ok = filter_rows(static_cast<const int32_t*>(f.filter), f.lo, f.hi, r, r1);
+            } else if (f.filter_w == 8) {
+                ok = filter_rows(static_cast<const int64_t*>(f.filter), f.lo, f.hi, r, r1);
+            } else {
+                ok = filter_rows(static_cast<const int8_t*>(f.filter), f.lo, f.hi, r, r1);
+            }
+            const uint32_t rel = static_cast<uint32_t>(r - r0);
+#pragma unroll
+            for (int j = 0; j < kFilterRows; ++j) {
+                const bool p = (ok >> j) & 1u;
+                const uint32_t m = __ballot_sync(FULL, p);
+                if (p) queue[held + __popc(m & lt)] = rel + j;
+                held += __popc(m);
+            }
+            __syncwarp();
+        }
+        // Full takes while rows are left to filter, whatever is held at the end.
+        while (held >= (more ? 32u * ITEMS : 1u)) take(held < 32u * ITEMS ? held : 32u * ITEMS);
+        if (!more) break;
     }
 }
 
 // Persistent fused kernel: (fragment, chunk) work items from a device counter.
-template <int THREADS, int ITEMS, int NA>
-__global__ void __launch_bounds__(THREADS)
+template <int THREADS, int ITEMS, int NA, bool W8>
+__global__ void __launch_bounds__(THREADS, (ITEMS > 2 ? 512 : 1024) / THREADS)
 frag_kernel(const PlanHeader* __restrict__ ph, const int64_t* __restrict__ item_start, const FragDev* __restrict__ fd,
             unsigned long long* counter, int32_t* status) {
     extern __shared__ __align__(16) unsigned char smem[];
@@ -223,6 +391,8 @@ frag_kernel(const PlanHeader* __restrict__ ph, const int64_t* __restrict__ item_
     // reductions' memory clobbers would otherwise reload its fields from global
     // memory after every update.
     __shared__ __align__(16) FragDev s_f;
+    __shared__ uint32_t s_queue[THREADS / 32][kQueue<ITEMS>];
+    uint32_t* queue = s_queue[threadIdx.x >> 5];
     const int n = ph->nfrags;
     const int64_t nitems = ph->nitems;
     for (;;) {
@@ -250,29 +420,33 @@ frag_kernel(const PlanHeader* __restrict__ ph, const int64_t* __restrict__ item_
         const int64_t r0 = (item - item_start[p]) * f.chunk;
         const int64_t r1 = r0 + f.chunk < f.nrows ? r0 + f.chunk : f.nrows;
         if (!f.shared) {
-            frag_rows<THREADS, ITEMS, NA, false>(f, r0, r1, nullptr, nullptr, nullptr, status);
+            frag_rows<THREADS, ITEMS, NA, W8, false>(f, r0, r1, nullptr, nullptr, nullptr, queue, status);
             continue;
         }
         const uint32_t D = f.D;
         const int naggs = f.naggs;
+        const uint32_t rs = f.rep_shift;
+        const uint32_t slots = (naggs * D) << rs;
         uint32_t* s_lo = reinterpret_cast<uint32_t*>(smem);
-        uint32_t* s_hi = s_lo + static_cast<size_t>(naggs) * D;
-        uint32_t* s_occ = s_hi + static_cast<size_t>(naggs) * D;
-        const uint32_t words = 2 * naggs * D + (f.count_agg < 0 ? (D + 31) / 32 : 0);
+        uint32_t* s_hi = s_lo + slots;
+        uint32_t* s_occ = s_hi + slots;
+        const uint32_t words = 2 * slots + (f.count_agg < 0 ? (D + 31) / 32 : 0);
         for (uint32_t w = threadIdx.x; w < words; w += THREADS) s_lo[w] = 0;
         __syncthreads();
-        frag_rows<THREADS, ITEMS, NA, true>(f, r0, r1, s_lo, s_hi, s_occ, status);
+        frag_rows<THREADS, ITEMS, NA, W8, true>(f, r0, r1, s_lo, s_hi, s_occ, queue, status);
         __syncthreads();
-        for (uint32_t d = threadIdx.x; d < D; d += THREADS) {
-            bool occ = f.count_agg < 0 && ((s_occ[d / 32] >> (d % 32)) & 1u);
-            for (int a = 0; a < naggs; ++a) {
-                const size_t o = static_cast<size_t>(a) * D + d;
-                const uint64_t x = (static_cast<uint64_t>(s_hi[o]) << 32) | s_lo[o];
-                if (x) red_add_global(&f.acc[o], x);
-                if (a == f.count_agg) occ = x != 0;
+        const uint32_t reps = 1u << rs;
+        for (uint32_t o = threadIdx.x; o < naggs * D; o += THREADS) {
+            uint64_t x = 0;
+            for (uint32_t k = 0; k < reps; ++k) {
+                const uint32_t w = (o << rs) + ((k + threadIdx.x) & (reps - 1));  // banks spread over the threads
+                x += (static_cast<uint64_t>(s_hi[w]) << 32) | s_lo[w];
             }
-            if (occ && f.count_agg < 0) f.occ[d] = 1;
+            if (x) red_add_global(&f.acc[o], x);
         }
+        if (f.count_agg < 0)
+            for (uint32_t d = threadIdx.x; d < D; d += THREADS)
+                if ((s_occ[d / 32] >> (d % 32)) & 1u) f.occ[d] = 1;
         // The next item's clear waits for every thread's flush at the loop top.
     }
 }
@@ -319,19 +493,29 @@ frag_emit_kernel(const PlanHeader* __restrict__ ph, const int64_t* __restrict__ 
         }
     }
     __syncthreads();
-    int64_t pos = s_excl + s_warp[warp];
+    // Every item's value of an aggregate is loaded before any is stored: the stores
+    // would otherwise hold back the next loads, one memory round trip per item (22
+    // tiles of six fragments: 15.8 us for this kernel).
     const uint32_t ltm = lanemask_lt();
+    int64_t q[kEmitItems];  // output row, or -1
+    int64_t pos = s_excl + s_warp[warp];
 #pragma unroll
     for (int i = 0; i < kEmitItems; ++i) {
-        if (mask[i] & (1u << lane)) {
-            const int64_t e = base + i * 32 + lane;
-            const int64_t q = pos + __popc(mask[i] & ltm);
-            if (q < f.max_groups) {
-                store_int(f.out_keys, f.group_w, q, f.group_lo + e);
-                for (int a = 0; a < f.naggs; ++a) f.out_aggs[a][q] = static_cast<int64_t>(f.acc[a * D + e]);
-            }
-        }
+        q[i] = pos + __popc(mask[i] & ltm);
+        if (!((mask[i] >> lane) & 1u) || q[i] >= f.max_groups) q[i] = -1;
         pos += __popc(mask[i]);
+        if (q[i] >= 0) store_int(f.out_keys, f.group_w, q[i], f.group_lo + base + i * 32 + lane);
+    }
+    for (int a = 0; a < f.naggs; ++a) {
+        const unsigned long long* acc = f.acc + a * D + base + lane;
+        int64_t* out = f.out_aggs[a];
+        unsigned long long v[kEmitItems];
+#pragma unroll
+        for (int i = 0; i < kEmitItems; ++i)
+            if (q[i] >= 0) v[i] = acc[i * 32];
+#pragma unroll
+        for (int i = 0; i < kEmitItems; ++i)
+            if (q[i] >= 0) out[q[i]] = static_cast<int64_t>(v[i]);
     }
 }
 
@@ -404,10 +588,10 @@ px_status check_fragment(const px_fragment& f, int32_t i) {
     return PX_OK;
 }
 
-template <int THREADS, int ITEMS, int NA>
+template <int THREADS, int ITEMS, int NA, bool W8>
 px_status launch_frag_na(const PlanHeader* ph, const int64_t* item_start, const FragDev* fd,
                          unsigned long long* counter, int32_t* status, size_t smem, int bps, cudaStream_t st) {
-    auto kernel = frag_kernel<THREADS, ITEMS, NA>;
+    auto kernel = frag_kernel<THREADS, ITEMS, NA, W8>;
     if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)) !=
         cudaSuccess)
         return check_launch("px_fragments_run attribute");
@@ -421,15 +605,15 @@ px_status launch_frag_na(const PlanHeader* ph, const int64_t* item_start, const 
 }
 
 // NA: the batch's largest aggregate count (at least 1), a compile-time bound.
-template <int THREADS, int ITEMS>
+template <int THREADS, int ITEMS, bool W8>
 px_status launch_frag(int na, const PlanHeader* ph, const int64_t* item_start, const FragDev* fd,
                       unsigned long long* counter, int32_t* status, size_t smem, int bps, cudaStream_t st) {
     switch (na) {
         case 0:
-        case 1: return launch_frag_na<THREADS, ITEMS, 1>(ph, item_start, fd, counter, status, smem, bps, st);
-        case 2: return launch_frag_na<THREADS, ITEMS, 2>(ph, item_start, fd, counter, status, smem, bps, st);
-        case 3: return launch_frag_na<THREADS, ITEMS, 3>(ph, item_start, fd, counter, status, smem, bps, st);
-        default: return launch_frag_na<THREADS, ITEMS, 4>(ph, item_start, fd, counter, status, smem, bps, st);
+        case 1: return launch_frag_na<THREADS, ITEMS, 1, W8>(ph, item_start, fd, counter, status, smem, bps, st);
+        case 2: return launch_frag_na<THREADS, ITEMS, 2, W8>(ph, item_start, fd, counter, status, smem, bps, st);
+        case 3: return launch_frag_na<THREADS, ITEMS, 3, W8>(ph, item_start, fd, counter, status, smem, bps, st);
+        default: return launch_frag_na<THREADS, ITEMS, 4, W8>(ph, item_start, fd, counter, status, smem, bps, st);
     }
 }
 
@@ -457,7 +641,7 @@ px_status px_fragments_run(const px_fragment* frags, int32_t nfrags, const px_fr
         const px_status s = check_fragment(frags[i], i);
         if (s != PX_OK) return s;
     }
-    px_fragments_config c = {256, 2, 0, 8};
+    px_fragments_config c = {512, 2, 0, 2};
     if (cfg) c = *cfg;
     if ((c.threads != 256 && c.threads != 512) || (c.items != 2 && c.items != 4) || c.blocks_per_sm < 1 ||
         c.blocks_per_sm > 8 || c.chunk_rows < 0 || c.chunk_rows % (static_cast<int64_t>(c.threads) * c.items) != 0)
@@ -466,7 +650,7 @@ px_status px_fragments_run(const px_fragment* frags, int32_t nfrags, const px_fr
         // Rows per work item from the batch: about four items per block of the
         // persistent grid, so a small batch still spreads over every SM, within
         // [one tile, 65536 rows].
-        const int64_t tile = static_cast<int64_t>(c.threads) * c.items;
+        const int64_t tile = static_cast<int64_t>(c.threads) * kFilterRows;
         int64_t rows = 0;
         for (int32_t i = 0; i < nfrags; ++i) rows += frags[i].nrows;
         const int64_t want = cdiv(rows, 4 * static_cast<int64_t>(sm_count()) * c.blocks_per_sm);
@@ -504,6 +688,7 @@ px_status px_fragments_run(const px_fragment* frags, int32_t nfrags, const px_fr
         sto += frag_state_bytes(frags[i]);
     }
     size_t smem = 0;
+    bool w8 = true;  // every aggregated column is 8 bytes wide
     int64_t items = 0, emits = 0;
     for (int32_t k = 0; k < nfrags; ++k) {
         const int32_t i = order[k];
@@ -524,12 +709,32 @@ px_status px_fragments_run(const px_fragment* frags, int32_t nfrags, const px_fr
             if (g.op != PX_COUNT) {
                 d.pa[a] = f.cols[g.a].data;
                 d.wa[a] = f.cols[g.a].type;
+                w8 = w8 && d.wa[a] == 8;
             }
+            d.same[a] = -1;
+            for (int e = 0; e < a && g.op != PX_COUNT; ++e)
+                if (f.aggs[e].op == PX_SUM && f.aggs[e].a == g.a) d.same[a] = e;
             if (g.op == PX_SUM_MUL) {
                 d.pb[a] = f.cols[g.b].data;
                 d.wb[a] = f.cols[g.b].type;
+                w8 = w8 && d.wb[a] == 8;
             }
             if (g.op == PX_COUNT && d.count_agg < 0) d.count_agg = a;
+        }
+        if (f.filter.data) {
+            d.stream[d.nstream] = f.filter.data;
+            d.stream_w[d.nstream++] = f.filter.type;
+        }
+        d.stream[d.nstream] = f.key.data;
+        d.stream_w[d.nstream++] = 8;
+        for (int k = 0; k < f.ncols; ++k) {
+            bool read = false;
+            for (int a = 0; a < f.naggs; ++a)
+                read |= (f.aggs[a].op != PX_COUNT && f.aggs[a].a == k) || (f.aggs[a].op == PX_SUM_MUL && f.aggs[a].b == k);
+            if (read) {
+                d.stream[d.nstream] = f.cols[k].data;
+                d.stream_w[d.nstream++] = f.cols[k].type;
+            }
         }
         d.t = table_view(const_cast<void*>(f.d_table), 1);
         d.nbuild = f.nbuild;
@@ -544,7 +749,13 @@ px_status px_fragments_run(const px_fragment* frags, int32_t nfrags, const px_fr
         d.chunk = c.chunk_rows;
         if (d.shared) {
             d.chunk = std::max<int64_t>(c.chunk_rows, cdiv(4 * static_cast<int64_t>(d.D), tile) * tile);
-            smem = std::max(smem, sbytes);
+            // Replicas of every slot while they stay few enough to clear and flush per
+            // item: lanes with the same group then add to different banks.
+            while (d.rep_shift < 5 && (static_cast<uint64_t>(d.D) << (d.rep_shift + 1)) <= kRepSlots &&
+                   static_cast<int64_t>((static_cast<uint64_t>(d.D) << (d.rep_shift + 1)) * 8) <= d.chunk)
+                ++d.rep_shift;
+            smem = std::max(smem, (8 * static_cast<size_t>(f.naggs) * d.D << d.rep_shift) +
+                                      (d.count_agg < 0 ? (d.D + 31) / 32 * 4 : 0));
         }
         d.acc = reinterpret_cast<unsigned long long*>(ws + L.acc + acc_off[i]);
         d.occ = d.count_agg < 0 ? reinterpret_cast<uint8_t*>(ws + L.acc + acc_off[i]) + 8 * static_cast<size_t>(f.naggs) * d.D
@@ -579,14 +790,17 @@ px_status px_fragments_run(const px_fragment* frags, int32_t nfrags, const px_fr
     if (items > 0) {
         int na = 0;
         for (int32_t i = 0; i < nfrags; ++i) na = std::max(na, frags[i].naggs);
-        if (c.threads == 256 && c.items == 2)
-            s = launch_frag<256, 2>(na, d_ph, d_items, d_fd, counters, status, smem, c.blocks_per_sm, st);
-        else if (c.threads == 256)
-            s = launch_frag<256, 4>(na, d_ph, d_items, d_fd, counters, status, smem, c.blocks_per_sm, st);
-        else if (c.items == 2)
-            s = launch_frag<512, 2>(na, d_ph, d_items, d_fd, counters, status, smem, c.blocks_per_sm, st);
-        else
-            s = launch_frag<512, 4>(na, d_ph, d_items, d_fd, counters, status, smem, c.blocks_per_sm, st);
+        const auto go = [&](auto threads, auto per_thread) {
+            constexpr int T = decltype(threads)::value, I = decltype(per_thread)::value;
+            return w8 ? launch_frag<T, I, true>(na, d_ph, d_items, d_fd, counters, status, smem, c.blocks_per_sm, st)
+                      : launch_frag<T, I, false>(na, d_ph, d_items, d_fd, counters, status, smem, c.blocks_per_sm, st);
+        };
+        const std::integral_constant<int, 256> t256;
+        const std::integral_constant<int, 512> t512;
+        const std::integral_constant<int, 2> i2;
+        const std::integral_constant<int, 4> i4;
+        if (c.threads == 256) s = c.items == 2 ? go(t256, i2) : go(t256, i4);
+        else s = c.items == 2 ? go(t512, i2) : go(t512, i4);
         if (s != PX_OK) return s;
     }
     frag_emit_kernel<<<static_cast<unsigned>(emits), kEmitThreads, 0, st>>>(d_ph, d_emits, d_fd, counters + 1, status);

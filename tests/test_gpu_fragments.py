@@ -148,3 +148,41 @@ def test_fragments_bad_arguments_are_rejected(px):
     f = _frag(px, d, 4)
     with pytest.raises(px.PxError):
         px.FragmentBatch([f], config=(128, 4, 512, 1)).run()
+
+
+# Edges of the filter step (4 rows per lane, 128 per warp, 2048 per block), of the
+# shared-mode replicas (1024 slots with their replicas: 32 replicas up to 32 groups,
+# one from 513 on) and of shared against direct mode (24 KB of accumulators), with
+# every filter and value width; the hot case gives every row one group.
+@pytest.mark.parametrize("ftype", [None, np.int8, np.int32, np.int64])
+@pytest.mark.parametrize("nf,ngroups", [(1, 1), (3, 2), (127, 1), (129, 33), (2047, 32), (6151, 512), (2049, 513),
+                                        (9001, 1024), (40_003, 1025), (40_003, 2000)])
+@pytest.mark.parametrize("vtype,cfg", [(np.int64, None), (np.int32, (512, 4, 0, 1)), (np.int8, (256, 2, 512, 2))])
+def test_fragments_edges_of_filter_replicas_and_modes(px, ftype, nf, ngroups, vtype, cfg):
+    g = pxdata.rng(nf * 7 + ngroups)
+    nb = 2 * ngroups + 3
+    pk = (g.permutation(nb) * 3 - nb).astype(np.int64)  # negative keys too; two probe keys of three miss
+    attr = (g.integers(0, ngroups, nb) - 5).astype(np.int32)
+    key = g.integers(-nb - 3, 2 * nb + 3, nf).astype(np.int64)
+    if nf == 127:
+        key[:] = pk[0]
+    a, b = pxdata.random_column(g, nf, vtype), pxdata.random_column(g, nf, np.int64)
+    table = px.px_join_build([dev(pk), dev(attr)], 0, unique=True, pay_col=1)
+    sel, lo, hi = np.arange(nf, dtype=np.int32), 0, 0
+    f = {"key": dev(key), "cols": [dev(a), dev(b) if vtype == np.int64 else dev(a)], "table": table,
+         "aggs": [(px.PX_SUM, 0, None), (px.PX_COUNT, None, None), (px.PX_SUM_MUL, 0, 1)], "group": dev(attr),
+         "group_lo": -5, "group_hi": ngroups - 6, "max_groups": ngroups}
+    if ftype is not None:
+        col = pxdata.random_column(g, nf, ftype)
+        lo, hi = int(np.iinfo(ftype).min // 4), int(np.iinfo(ftype).max // 2)
+        f.update(filter=dev(col), lo=lo, hi=hi)
+        sel = oracle.filter(col, lo, hi)
+    fb = px.FragmentBatch([f], config=cfg)
+    res = fb.run()[0]
+    torch.cuda.synchronize()
+    assert fb.ws.status() == px.PX_OK
+    pr, br, _ = oracle.join(pk, key, sel=sel)
+    av, bv = a.astype(np.int64), (b if vtype == np.int64 else a).astype(np.int64)
+    want = oracle.groupby([attr[br]], [(oracle.SUM, av[pr], None), (oracle.COUNT, None, None),
+                                       (oracle.SUM_MUL, av[pr], bv[pr])])
+    _check(res, want)
