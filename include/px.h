@@ -164,7 +164,7 @@ px_status px_filter(const px_col* col, int64_t nrows, const int64_t* d_nrows,
  * array (it keeps the last call's contents; each call writes every count it reads
  * before reading it), so calls whose GPU work may overlap (other streams, other
  * threads) race and must be serialised by the caller. */
-#define PX_FILTER_NOALLOC_MAX_ROWS 134217728LL /* 65536 tiles of 2048 rows */
+#define PX_FILTER_NOALLOC_MAX_ROWS 134217728LL /* 2^27 */
 px_status px_filter_noalloc(const px_col* col, int64_t nrows, const int64_t* d_nrows,
                             int64_t lo, int64_t hi, int32_t* d_sel, int64_t* d_nsel,
                             int32_t* d_status, void* stream);

@@ -267,6 +267,11 @@ __device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint32_t by
         : "memory");
 }
 
+// Starts a copy of [p, p + bytes) into L2 (both multiples of 16).
+__device__ __forceinline__ void prefetch_l2(const void* p, uint32_t bytes) {
+    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
+}
+
 // ------------------------------------------- programmatic dependent launch --
 // A kernel launched with launch_after() may start while the kernel before it on the
 // stream is still running (once every block of that one has called

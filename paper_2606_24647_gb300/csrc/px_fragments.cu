@@ -119,11 +119,6 @@ __device__ __forceinline__ int find_frag(const int64_t* start, int n, int64_t x)
 
 __device__ __forceinline__ int64_t load_w(const void* p, int w, int64_t i) { return load_int(p, w, i); }
 
-// Starts a copy of [p, p + bytes) into L2 (both multiples of 16).
-__device__ __forceinline__ void prefetch_l2(const void* p, uint32_t bytes) {
-    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
-}
-
 // Adds x (mod 2^64) to a 64-bit value held as 32-bit words lo/hi in shared memory.
 __device__ __forceinline__ void add_split(uint32_t* lo, uint32_t* hi, uint64_t x) {
     const uint32_t xl = static_cast<uint32_t>(x), xh = static_cast<uint32_t>(x >> 32);

@@ -524,3 +524,29 @@ def test_groupby_sum_count_wide_key_range(px, kt, vt):
             if not segmented:
                 want = oracle.groupby([keys], o_aggs)
             assert_groups_equal(res, want, 1, segmented=segmented)
+
+
+# Edges of the filter's tiles (4 warps of 256 rows, of 1024 rows once a tile per block
+# of the 256-row ones no longer holds the column: 1.9M rows on 152 SMs; more than one
+# tile per block past 7.5M): row counts around them, every width, bounds at and beyond
+# the type's range, device row counts.
+@pytest.mark.parametrize("dtype", [np.int8, np.int32, np.int64])
+@pytest.mark.parametrize("n", [1, 31, 255, 1023, 1024, 1025, 4097, 65_537, 2_000_003, 9_000_001])
+def test_filter_edges_of_steps_and_bounds(px, dtype, n):
+    g = pxdata.rng(n)
+    info = np.iinfo(dtype)
+    col = pxdata.random_column(g, n, dtype)
+    col[:: max(1, n // 7)] = info.max
+    col[n // 2] = info.min
+    d = dev(col)
+    bounds = [(info.min, info.max), (int(info.min) // 3, int(info.max) // 2), (int(info.max), 2**63 - 1),
+              (-(2**63), int(info.min)), (-(2**63), 2**63 - 1), (5, 5), (7, -7)]
+    for lo, hi in bounds if n < 10**6 else bounds[1:2]:
+        for rows in (None, n - 1 if n > 1 else 0):
+            want = oracle.filter(col if rows is None else col[:rows], int(lo), int(hi))
+            sel, nsel = px.px_filter(d, int(lo), int(hi), sel=torch.full((n,), -9, dtype=torch.int32, device="cuda"),
+                                     d_nrows=None if rows is None else dev(np.array([rows], np.int64)))
+            m = count(nsel)
+            assert m == want.size
+            np.testing.assert_array_equal(host(sel, m), want)
+            assert bool((sel[m:] == -9).all())
