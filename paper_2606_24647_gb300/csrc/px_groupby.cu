@@ -3,22 +3,19 @@
 //
 // Group key: the key columns (and the segment id) packed into one 64-bit code,
 // each key biased by its sign bit so the code orders like the signed tuple.
-// Each block is persistent over a contiguous range of positions, which it walks
-// segment by segment. Per segment it aggregates into a block-local table and
-// merges that table into the global result when the segment ends (codes of a
-// finished segment never recur in the block's range, so the table starts empty
-// for the next one). The block-local table is either
-//   * dense: when the caller's key-range statistic makes the key space small,
-//     shared-memory arrays indexed by the key offset, replicated per warp when
-//     they fit (fewer same-address atomics); rows outside the range take the
-//     global path; or
-//   * hashed: an open-addressing shared-memory table (code -> accumulators);
-//     codes that find no room within a few probes take the global path.
-// Rows of one warp with equal codes are first combined with shuffles (peers from
-// match_any), so a hot key costs one shared-memory update per warp, not 32.
-// The global table lives in the workspace: slots are claimed with a CAS on a
-// state word (empty -> claimed -> published), take the next output row from a
-// counter, and accumulate with 64-bit reductions straight into the output columns.
+// Blocks are persistent over contiguous ranges of positions, which they walk segment
+// by segment. With a key-range statistic that makes the key space small, a block
+// aggregates into dense shared-memory arrays indexed by the key offset, replicated per
+// warp when they fit (fewer same-address atomics), and merges them into the global
+// result when the segment ends; rows outside the range take the claim table: slots of
+// a table in the workspace claimed with a CAS on a state word (empty -> claimed ->
+// published), each taking the next output row, accumulated with 64-bit reductions
+// straight into the output columns.
+// Without such a statistic: groupby_hash_kernel, an open-addressing table of keys and
+// accumulators in the workspace with a small block-local cache in front of it, and
+// hash_emit_kernel, which writes its groups out.
+// Rows of one warp with lane 0's group are first combined across the warp, so a hot
+// key costs one update per warp, not 32.
 // All arithmetic is mod 2^64. Every thread loads all of its rows' inputs for a
 // tile before aggregating any of them, so each thread keeps many loads in flight.
 #include <algorithm>
@@ -33,7 +30,6 @@ constexpr int kThreads = 1024;
 constexpr int kWarps = kThreads / 32;
 constexpr int kItems = 4;
 constexpr int kTile = kThreads * kItems;
-constexpr int kSmemProbes = 8;
 constexpr int kMajority = 6;  // smallest group worth a warp reduction
 constexpr size_t kSmemBudget = 192 * 1024;
 
@@ -170,48 +166,9 @@ __device__ __forceinline__ void global_add(const GTable& g, const Spec& sp, uint
         red_add_global(reinterpret_cast<unsigned long long*>(&sp.agg_out[a][gi]), static_cast<unsigned long long>(v[a]));
 }
 
-// Slot of `code` in the block's hash table, inserting it if absent; -1 if no
-// room within kSmemProbes probes.
-__device__ __forceinline__ int smem_slot(uint32_t* s_state, unsigned long long* s_key, uint32_t smask, uint64_t code,
-                                         int32_t* status) {
-    uint32_t s = static_cast<uint32_t>(fmix64(code)) & smask;
-    for (int probe = 0; probe < kSmemProbes; ++probe) {
-        volatile uint32_t* vs = &s_state[s];
-        uint32_t st = *vs;
-        if (st == 0) {
-            st = atomicCAS(&s_state[s], 0u, 1u);
-            if (st == 0) {
-                s_key[s] = code;
-                __threadfence_block();
-                *vs = 2u;
-                return static_cast<int>(s);
-            }
-        }
-        uint32_t spins = 0;
-        while (st == 1) {
-            if (++spins > kSpinLimit) {
-                set_status(status, PX_ERR_TIMEOUT);
-                return -1;
-            }
-            st = *vs;
-        }
-        __threadfence_block();
-        if (static_cast<volatile unsigned long long*>(s_key)[s] == code) return static_cast<int>(s);
-        s = (s + 1) & smask;
-    }
-    return -1;
-}
-
 struct Smem {
-    // dense: replicas of rep_bytes each (see Spec)
-    unsigned char* rep0;
+    unsigned char* rep0;  // replicas of rep_bytes each (see Spec)
     uint32_t occ_words;
-    // hashed: low words [naggs][S], high words [naggs][S], key[S], state[S]
-    uint32_t* h_lo;
-    uint32_t* h_hi;
-    unsigned long long* h_key;
-    uint32_t* h_state;
-    uint32_t S;
 };
 
 // A replica holds each 64-bit sum as two 32-bit words, low words [n64][D] then
@@ -246,14 +203,9 @@ __device__ __forceinline__ uint32_t* rep_occ(const Spec& sp, const Smem& m, int 
 }
 
 __device__ __forceinline__ void clear_block_table(const Spec& sp, const Smem& m) {
-    if (sp.dense) {
-        uint32_t* w = reinterpret_cast<uint32_t*>(m.rep0);
-        const uint32_t nw = static_cast<uint32_t>(sp.reps) * sp.rep_bytes / 4;
-        for (uint32_t i = threadIdx.x; i < nw; i += kThreads) w[i] = 0;
-    } else {
-        for (uint32_t s = threadIdx.x; s < m.S; s += kThreads) m.h_state[s] = 0;
-        for (uint32_t s = threadIdx.x; s < m.S * sp.naggs; s += kThreads) m.h_lo[s] = m.h_hi[s] = 0;
-    }
+    uint32_t* w = reinterpret_cast<uint32_t*>(m.rep0);
+    const uint32_t nw = static_cast<uint32_t>(sp.reps) * sp.rep_bytes / 4;
+    for (uint32_t i = threadIdx.x; i < nw; i += kThreads) w[i] = 0;
 }
 
 // Merge the block table (segment q) into the global table and clear it.
@@ -265,8 +217,8 @@ __device__ void flush_block_table(const Spec& sp, const Smem& m, int q, const GT
     // while the rest of the block waits at the barrier. With many slots the thread
     // per slot keeps every thread busy and wins (a warp sum costs ~12 thread-slot
     // steps).
-    const bool warp_flush = sp.dense && (sp.D + kWarps - 1) / kWarps * 12 <
-                                            (sp.D + kThreads - 1) / kThreads * static_cast<uint32_t>(sp.reps);
+    const bool warp_flush = (sp.D + kWarps - 1) / kWarps * 12 <
+                            (sp.D + kThreads - 1) / kThreads * static_cast<uint32_t>(sp.reps);
     if (warp_flush) {
         const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
         for (uint32_t d = warp; d < sp.D; d += kWarps) {
@@ -310,7 +262,7 @@ __device__ void flush_block_table(const Spec& sp, const Smem& m, int q, const GT
         if (sp.count_agg < 0)
             for (uint32_t i = threadIdx.x; i < sp.reps * m.occ_words; i += kThreads)
                 rep_occ(sp, m, i / m.occ_words)[i % m.occ_words] = 0;
-    } else if (sp.dense) {
+    } else {
         for (uint32_t d = threadIdx.x; d < sp.D; d += kThreads) {
             uint64_t v[PX_MAX_AGGS];
             bool occ = false;
@@ -351,19 +303,6 @@ __device__ void flush_block_table(const Spec& sp, const Smem& m, int q, const GT
         if (sp.count_agg < 0)
             for (uint32_t i = threadIdx.x; i < sp.reps * m.occ_words; i += kThreads)
                 rep_occ(sp, m, i / m.occ_words)[i % m.occ_words] = 0;
-    } else {
-        for (uint32_t s = threadIdx.x; s < m.S; s += kThreads) {
-            if (m.h_state[s] == 2) {
-                uint64_t v[PX_MAX_AGGS];
-                for (int a = 0; a < sp.naggs; ++a) {
-                    const size_t o = static_cast<size_t>(a) * m.S + s;
-                    v[a] = (static_cast<uint64_t>(m.h_hi[o]) << 32) | m.h_lo[o];
-                    m.h_lo[o] = m.h_hi[o] = 0;
-                }
-                global_add(g, sp, m.h_key[s], v, max_groups, out_seg, status);
-            }
-            m.h_state[s] = 0;
-        }
     }
     __syncthreads();
 }
@@ -372,13 +311,14 @@ constexpr uint32_t kIdxNone = 0xffffffffu;   // no row at this item
 constexpr uint32_t kIdxOutside = 0xfffffffeu;  // key outside the dense range
 
 // v[i] = column value at row[i] (sign-extended), 0 where row[i] < 0. One type
-// switch per column, then kItems independent loads.
-template <typename T>
-__device__ __forceinline__ void load_col_t(const void* p, const int32_t* row, int64_t* v) {
+// switch per column, then ITEMS independent loads.
+template <typename T, int ITEMS>
+__device__ __forceinline__ void load_col_t(const void* p, const int32_t (&row)[ITEMS], int64_t* v) {
 #pragma unroll
-    for (int i = 0; i < kItems; ++i) v[i] = row[i] >= 0 ? static_cast<int64_t>(static_cast<const T*>(p)[row[i]]) : 0;
+    for (int i = 0; i < ITEMS; ++i) v[i] = row[i] >= 0 ? static_cast<int64_t>(static_cast<const T*>(p)[row[i]]) : 0;
 }
-__device__ __forceinline__ void load_col(const void* p, int w, const int32_t* row, int64_t* v) {
+template <int ITEMS>
+__device__ __forceinline__ void load_col(const void* p, int w, const int32_t (&row)[ITEMS], int64_t* v) {
     if (w == 8) load_col_t<int64_t>(p, row, v);
     else if (w == 4) load_col_t<int32_t>(p, row, v);
     else load_col_t<int8_t>(p, row, v);
@@ -574,108 +514,357 @@ __device__ void aggregate_range_dense(const Spec& sp, const Smem& m, const int32
     }
 }
 
-// Hash-mode aggregation of positions [a0, a1) of segment q into the block's
-// shared-memory hash table; codes that find no room go to the global table. NA:
-// number of aggregates when known at compile time (0..4), or PX_MAX_AGGS.
+// ---------------------------------------------------------------- hash mode ----
+// The table of groups, in the workspace: buckets of four slots (one 32-byte sector of
+// keys), at least two slots per possible group, and one slot more for the code whose
+// stored form would read as empty. Keys hold ~code, 0 where empty; a slot's
+// accumulators sit together. A key is set once, by a CAS, and nothing else is published
+// with it: accumulators start at zero (cleared with the keys before the call), so no
+// row ever waits for another. A code takes the first empty slot from its home bucket
+// on, so a lookup mostly reads one sector and ends at the first empty slot.
+struct HTable {
+    unsigned long long* emitted;  // the emit's counter (see hash_emit_kernel), zero between calls
+    unsigned long long* key;  // [slots + 1], 32-byte aligned
+    unsigned long long* acc;  // [slots + 1] << shift
+    uint32_t slots;           // a power of two
+    int32_t shift;
+};
+
+constexpr int kHashThreads = 512;
+constexpr int kHashItems = 4;  // rows a thread loads at a time
+constexpr int kHashTile = kHashThreads * kHashItems;
+constexpr int kHashBlocksPerSm = 2;
+constexpr size_t kCacheBudget = 64 * 1024;  // the block-local cache
+constexpr int kHashMajority = 12;           // smallest group worth a warp reduction here
+constexpr uint32_t kNoSlot = 0xffffffffu;
+constexpr uint32_t kBucketSlots = 4;
+
+struct KeyBucket {
+    unsigned long long k[kBucketSlots];
+};
+
+// The keys of a bucket as L2 holds them (no L1: another SM's insert must not stay hidden
+// behind a stale line). A key that reads 0 may have been set since; its CAS tells.
+__device__ __forceinline__ KeyBucket load_keys(const HTable& h, uint32_t bucket) {
+    KeyBucket b;
+    asm volatile("ld.relaxed.gpu.global.v4.u64 {%0, %1, %2, %3}, [%4];"
+                 : "=l"(b.k[0]), "=l"(b.k[1]), "=l"(b.k[2]), "=l"(b.k[3])
+                 : "l"(h.key + static_cast<size_t>(bucket) * kBucketSlots)
+                 : "memory");
+    return b;
+}
+
+// The slot of `inv` in the bucket whose keys are `b`, set there if the bucket has room;
+// kNoSlot if it is full of other keys.
+__device__ __forceinline__ uint32_t bucket_slot(const HTable& h, uint32_t bucket, const KeyBucket& b,
+                                                unsigned long long inv) {
+    uint32_t at = kNoSlot, empty = kBucketSlots;
+#pragma unroll
+    for (int j = kBucketSlots - 1; j >= 0; --j) {
+        if (b.k[j] == inv) at = bucket * kBucketSlots + j;
+        if (b.k[j] == 0) empty = j;
+    }
+    if (at == kNoSlot)
+        for (uint32_t j = empty; j < kBucketSlots; ++j) {
+            const unsigned long long old = atomicCAS(&h.key[bucket * kBucketSlots + j], 0ull, inv);
+            if (old == 0 || old == inv) {
+                at = bucket * kBucketSlots + j;
+                break;
+            }
+        }
+    return at;
+}
+
+// The slot of `inv` from bucket `bucket` on (its first bucket was full); kNoSlot where
+// the table is full.
+__device__ __noinline__ uint32_t hash_walk(const HTable& h, uint32_t bucket, unsigned long long inv) {
+    const uint32_t last = h.slots / kBucketSlots - 1;
+    for (uint32_t round = 0; round < last; ++round) {
+        bucket = (bucket + 1) & last;
+        const uint32_t at = bucket_slot(h, bucket, load_keys(h, bucket), inv);
+        if (at != kNoSlot) return at;
+    }
+    return kNoSlot;
+}
+
+// Two neighbouring 64-bit words of shared memory, read anew.
+__device__ __forceinline__ ulonglong2 ld_shared_pair(const unsigned long long* p) {
+    ulonglong2 v;
+    asm volatile("ld.volatile.shared.v2.u64 {%0, %1}, [%2];" : "=l"(v.x), "=l"(v.y) : "r"(smem_u32(p)) : "memory");
+    return v;
+}
+
+// Takes an empty slot of the cache pair at `c` for `inv` (or finds it set meanwhile);
+// kNoSlot if other codes took both.
+__device__ __forceinline__ uint32_t cache_claim(unsigned long long* c_key, uint32_t c, unsigned long long inv) {
+    for (uint32_t j = c; j < c + 2; ++j) {
+        const unsigned long long old = atomicCAS(&c_key[j], 0ull, inv);
+        if (old == 0 || old == inv) return j;
+    }
+    return kNoSlot;
+}
+
+// GROUP BY without a usable statistic. Each row's code is hashed once; the high hash
+// bits name two slots of a block-local cache in shared memory, taken by whichever
+// codes come first (a hot code comes early and then costs shared-memory adds only),
+// the low bits a slot of the table in the workspace, where the rows the cache does not
+// hold are added with 64-bit reductions. NA: number of aggregates when known at compile
+// time (0..4), or PX_MAX_AGGS.
+// Bound by the 64-bit reductions' L2 traffic where most rows go to the table (L2 81 %
+// busy), else by the latency of the dependent steps at 1024 threads per SM. Measured,
+// 10M rows, int64 keys, SUM + SUM_MUL + COUNT (240 MB), against block tables of 4096
+// slots probed 8 deep in front of a claimed and published table: 100,000 groups 1465 ->
+// 207 us, Zipf(1.1) 1209 -> 153; 3000 groups 833 -> 152; 1M groups 1469 -> 353; 100
+// groups 97 -> 94. A cache slot pair is read with one 16-byte load and a bucket with
+// one 32-byte load; single-slot probing took 408 us at 100,000 groups.
 template <int NA>
-__device__ void aggregate_range(const Spec& sp, const Smem& m, const int32_t* __restrict__ sel, int64_t a0, int64_t a1,
-                                int q, const GTable& g, int64_t max_groups, int32_t* out_seg, int32_t* status) {
+__global__ void __launch_bounds__(kHashThreads, kHashBlocksPerSm)
+groupby_hash_kernel(Spec sp, const int32_t* __restrict__ sel, const int64_t* __restrict__ d_n, int64_t ncap,
+                    const int64_t* __restrict__ d_seg, HTable h, uint32_t cache_slots, int32_t* status) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    const uint32_t C = cache_slots;
+    unsigned long long* c_key = reinterpret_cast<unsigned long long*>(smem);  // [C], ~code or 0
+    uint32_t* c_lo = reinterpret_cast<uint32_t*>(c_key + C);                  // [naggs][C]
+    uint32_t* c_hi = c_lo + static_cast<size_t>(sp.naggs) * C;                // [naggs][C]
     const int tid = threadIdx.x, lane = tid & 31;
-    for (int64_t tb = a0; tb < a1; tb += kTile) {
-        int32_t row[kItems];
-#pragma unroll
-        for (int i = 0; i < kItems; ++i) {
-            const int64_t j = tb + i * kThreads + tid;
-            row[i] = j < a1 ? (sel ? sel[j] : static_cast<int32_t>(j)) : -1;
-        }
-        uint64_t code[kItems];
-        {
-            int64_t k0[kItems], k1[kItems];
-            load_col(sp.key_in[0], sp.key_w[0], row, k0);
-            if (sp.nkeys > 1) load_col(sp.key_in[1], sp.key_w[1], row, k1);
-#pragma unroll
-            for (int i = 0; i < kItems; ++i) code[i] = compose(sp, k0[i], sp.nkeys > 1 ? k1[i] : 0, q);
-        }
-        int64_t v[NA > 0 ? NA : 1][kItems];
-#pragma unroll
-        for (int a = 0; a < NA; ++a) {
-            if (a >= sp.naggs) break;
-            if (sp.op[a] == PX_COUNT) {
-#pragma unroll
-                for (int i = 0; i < kItems; ++i) v[a][i] = 1;
-            } else {
-                load_col(sp.a_in[a], sp.a_w[a], row, v[a]);
-                if (sp.op[a] == PX_SUM_MUL) {
-                    int64_t y[kItems];
-                    load_col(sp.b_in[a], sp.b_w[a], row, y);
-#pragma unroll
-                    for (int i = 0; i < kItems; ++i)
-                        v[a][i] = static_cast<int64_t>(static_cast<uint64_t>(v[a][i]) * static_cast<uint64_t>(y[i]));
-                }
+    for (uint32_t w = tid; w < C * (2 + 2 * sp.naggs); w += kHashThreads) reinterpret_cast<uint32_t*>(smem)[w] = 0;
+    __syncthreads();
+    const int64_t n = actual_rows(d_n, ncap);
+    const int64_t chunk = cdiv(cdiv(n, gridDim.x), kHashTile) * kHashTile;
+    const int64_t cb = static_cast<int64_t>(blockIdx.x) * chunk;
+    const int64_t ce = n < cb + chunk ? n : cb + chunk;
+    int64_t pos = cb;
+    while (pos < ce) {
+        int q = 0;
+        int64_t qend = ce;
+        if (sp.nsegs > 1) {
+            q = seg_of(d_seg, sp.nsegs, pos);
+            if (q + 1 < sp.nsegs) {
+                const int64_t e = d_seg[q + 1];
+                if (e > pos && e < ce) qend = e;
             }
         }
+        for (int64_t tb = pos; tb < qend; tb += kHashTile) {
+            int32_t row[kHashItems];
 #pragma unroll
-        for (int i = 0; i < kItems; ++i) {
-            const bool valid = row[i] >= 0;
-            // Hot keys: lane 0's code shared by >= kMajority lanes is summed across
-            // the warp and applied once by lane 0.
-            bool lead = valid;
-            const uint64_t c0 = __shfl_sync(FULL, code[i], 0);
-            const uint32_t mm = __ballot_sync(FULL, valid && code[i] == c0);
-            if ((mm & 1u) && __popc(mm) >= kMajority) {
-                const bool in = (mm >> lane) & 1u;
+            for (int i = 0; i < kHashItems; ++i) {
+                const int64_t j = tb + i * kHashThreads + tid;
+                row[i] = j < qend ? (sel ? sel[j] : static_cast<int32_t>(j)) : -1;
+            }
+            unsigned long long inv[kHashItems];  // ~code
+            uint32_t bucket[kHashItems], cslot[kHashItems];  // home bucket; cache slot pair
+            {
+                int64_t k0[kHashItems], k1[kHashItems];
+                load_col(sp.key_in[0], sp.key_w[0], row, k0);
+                if (sp.nkeys > 1) load_col(sp.key_in[1], sp.key_w[1], row, k1);
+#pragma unroll
+                for (int i = 0; i < kHashItems; ++i) {
+                    const uint64_t code = compose(sp, k0[i], sp.nkeys > 1 ? k1[i] : 0, q);
+                    const uint64_t hash = fmix64(code);
+                    inv[i] = ~code;
+                    bucket[i] = static_cast<uint32_t>(hash) & (h.slots / kBucketSlots - 1);
+                    cslot[i] = static_cast<uint32_t>(hash >> 32) & (C - 2);
+                }
+            }
+            int64_t v[NA > 0 ? NA : 1][kHashItems];
+#pragma unroll
+            for (int a = 0; a < NA; ++a) {
+                if (a >= sp.naggs) break;
+                if (sp.op[a] == PX_COUNT) {
+#pragma unroll
+                    for (int i = 0; i < kHashItems; ++i) v[a][i] = 1;
+                } else {
+                    load_col(sp.a_in[a], sp.a_w[a], row, v[a]);
+                    if (sp.op[a] == PX_SUM_MUL) {
+                        int64_t y[kHashItems];
+                        load_col(sp.b_in[a], sp.b_w[a], row, y);
+#pragma unroll
+                        for (int i = 0; i < kHashItems; ++i)
+                            v[a][i] = static_cast<int64_t>(static_cast<uint64_t>(v[a][i]) * static_cast<uint64_t>(y[i]));
+                    }
+                }
+            }
+            bool lead[kHashItems];  // the lane applies the item
+#pragma unroll
+            for (int i = 0; i < kHashItems; ++i) {
+                lead[i] = row[i] >= 0;
+                // Hot keys: lane 0's code shared by >= kHashMajority lanes is summed across
+                // the warp and applied once by lane 0.
+                const unsigned long long c0 = __shfl_sync(FULL, inv[i], 0);
+                const uint32_t mm = __ballot_sync(FULL, lead[i] && inv[i] == c0);
+                if ((mm & 1u) && __popc(mm) >= kHashMajority) {
+                    const bool in = (mm >> lane) & 1u;
+#pragma unroll
+                    for (int a = 0; a < NA; ++a) {
+                        if (a >= sp.naggs) break;
+                        const int64_t x = sp.op[a] == PX_COUNT
+                                              ? static_cast<int64_t>(__popc(mm))
+                                              : static_cast<int64_t>(warp_sum_u64(in ? static_cast<uint64_t>(v[a][i]) : 0));
+                        if (lane == 0) v[a][i] = x;
+                    }
+                    lead[i] = lead[i] && (!in || lane == 0);
+                }
+            }
+            // One row of a thread at a time (two rows' round trips together: the registers
+            // spill, 251 us at 100,000 groups).
+#pragma unroll
+            for (int i = 0; i < kHashItems; ++i) {
+                // The cache: either slot of the pair, or an empty one of the two.
+                const ulonglong2 ck = ld_shared_pair(c_key + cslot[i]);
+                uint32_t c = kNoSlot;
+                bool pend = false;  // for the table
+                if (lead[i]) {
+                    if (inv[i] != 0) {
+                        if (ck.x == inv[i]) c = cslot[i];
+                        else if (ck.y == inv[i]) c = cslot[i] + 1;
+                        else if (ck.x == 0 || ck.y == 0) c = cache_claim(c_key, cslot[i], inv[i]);
+                    }
+                    pend = c == kNoSlot;
+                }
 #pragma unroll
                 for (int a = 0; a < NA; ++a) {
                     if (a >= sp.naggs) break;
-                    const int64_t x = sp.op[a] == PX_COUNT
-                                          ? static_cast<int64_t>(__popc(mm))
-                                          : static_cast<int64_t>(warp_sum_u64(in ? static_cast<uint64_t>(v[a][i]) : 0));
-                    if (lane == 0) v[a][i] = x;
+                    uint32_t* lo = c_lo + static_cast<uint32_t>(a) * C;
+                    if (sp.op[a] == PX_COUNT) {  // a block counts fewer than 2^32 rows
+                        if (c != kNoSlot) red_add_shared(&lo[c], static_cast<uint32_t>(v[a][i]));
+                    } else if (c != kNoSlot) {
+                        add_split_atomic(&lo[c], c_hi + static_cast<uint32_t>(a) * C + c, static_cast<uint64_t>(v[a][i]));
+                    }
                 }
-                lead = valid && (!in || lane == 0);
-            }
-            if (!lead) continue;
-            const int s = smem_slot(m.h_state, m.h_key, m.S - 1, code[i], status);
-            if (s >= 0) {
+                KeyBucket kb;
+                if (pend) kb = load_keys(h, bucket[i]);
+                if (pend) {
+                    uint32_t slot;
+                    if (inv[i] == 0) {  // the code that reads as empty has a slot of its own
+                        slot = h.slots;
+                        h.key[slot] = 1;  // every writer stores the same value
+                    } else {
+                        slot = bucket_slot(h, bucket[i], kb, inv[i]);
+                        if (slot == kNoSlot) slot = hash_walk(h, bucket[i], inv[i]);
+                    }
+                    if (slot == kNoSlot) {
+                        set_status(status, PX_ERR_CAPACITY);
+                    } else {
+                        unsigned long long* acc = h.acc + (static_cast<size_t>(slot) << h.shift);
 #pragma unroll
-                for (int a = 0; a < NA; ++a) {
-                    if (a >= sp.naggs) break;
-                    const size_t o = static_cast<size_t>(a) * m.S + s;
-                    add_split_atomic(&m.h_lo[o], &m.h_hi[o], static_cast<uint64_t>(v[a][i]));
+                        for (int a = 0; a < NA; ++a) {
+                            if (a >= sp.naggs) break;
+                            red_add_global(acc + a, static_cast<unsigned long long>(v[a][i]));
+                        }
+                    }
                 }
-            } else {
-                uint64_t full[PX_MAX_AGGS];
-#pragma unroll
-                for (int a = 0; a < NA; ++a) full[a] = static_cast<uint64_t>(v[a][i]);
-                global_add(g, sp, code[i], full, max_groups, out_seg, status);
             }
         }
+        // The cache into the table, then cleared: a next segment's codes are other codes.
+        __syncthreads();
+        for (uint32_t c = tid; c < C; c += kHashThreads) {
+            const unsigned long long ci = c_key[c];
+            if (ci == 0) continue;
+            const uint32_t home = static_cast<uint32_t>(fmix64(~ci)) & (h.slots / kBucketSlots - 1);
+            uint32_t slot = bucket_slot(h, home, load_keys(h, home), ci);
+            if (slot == kNoSlot) slot = hash_walk(h, home, ci);
+            if (slot == kNoSlot) set_status(status, PX_ERR_CAPACITY);
+            for (int a = 0; a < sp.naggs; ++a) {
+                const uint32_t o = static_cast<uint32_t>(a) * C + c;
+                const uint64_t x = (static_cast<uint64_t>(c_hi[o]) << 32) | c_lo[o];
+                if (x && slot != kNoSlot) red_add_global(h.acc + (static_cast<size_t>(slot) << h.shift) + a, x);
+                c_lo[o] = c_hi[o] = 0;
+            }
+            c_key[c] = 0;
+        }
+        __syncthreads();
+        pos = qend;
     }
 }
 
-// Modes: kHashed, kDenseBlock (block arrays) and kDenseDirect (rows straight into
-// the dense global array). MODE must agree with sp.dense / sp.direct: the modes are
-// separate kernels so each gets its own register allocation.
-constexpr int kHashed = 0, kDenseBlock = 1, kDenseDirect = 2;
+constexpr int kEmitThreads = 256;
+constexpr int kEmitItems = 8;
+constexpr int kEmitTile = kEmitThreads * kEmitItems;
+constexpr int kEmitWarps = kEmitThreads / 32;
+
+// Writes the table's groups out, in no particular order: each block takes its tile's
+// output rows with one add to *h.emitted, whose low bits count groups and whose high
+// bits count blocks; the last block writes the total and clears it.
+constexpr int kEmittedBits = 40;
+__global__ void __launch_bounds__(kEmitThreads)
+hash_emit_kernel(Spec sp, HTable h, int64_t max_groups, int32_t* __restrict__ out_seg, int64_t* __restrict__ d_ngroups,
+                 int32_t* status) {
+    __shared__ int32_t s_warp[kEmitWarps];
+    __shared__ int64_t s_base;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    wait_prior();  // the table
+    const int64_t nslots = static_cast<int64_t>(h.slots) + 1;
+    const int64_t base = static_cast<int64_t>(blockIdx.x) * kEmitTile + warp * (32 * kEmitItems) + lane;
+    unsigned long long key[kEmitItems];
+#pragma unroll
+    for (int i = 0; i < kEmitItems; ++i) key[i] = base + i * 32 < nslots ? h.key[base + i * 32] : 0;
+    uint32_t mask[kEmitItems];
+    int32_t cnt = 0;
+#pragma unroll
+    for (int i = 0; i < kEmitItems; ++i) {
+        mask[i] = __ballot_sync(FULL, key[i] != 0);
+        cnt += __popc(mask[i]);
+    }
+    if (lane == 0) s_warp[warp] = cnt;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        int32_t total = 0;
+        for (int w = 0; w < kEmitWarps; ++w) {
+            const int32_t c = s_warp[w];
+            s_warp[w] = total;
+            total += c;
+        }
+        const unsigned long long old =
+            atomicAdd(h.emitted, (1ull << kEmittedBits) | static_cast<unsigned long long>(total));
+        s_base = static_cast<int64_t>(old & ((1ull << kEmittedBits) - 1));
+        if ((old >> kEmittedBits) == gridDim.x - 1) {
+            *h.emitted = 0;
+            *d_ngroups = s_base + total;
+            if (s_base + total > max_groups) set_status(status, PX_ERR_CAPACITY);
+        }
+    }
+    __syncthreads();
+    const uint32_t lt = lanemask_lt();
+    int64_t p[kEmitItems];  // output row, or -1
+    int64_t pos = s_base + s_warp[warp];
+#pragma unroll
+    for (int i = 0; i < kEmitItems; ++i) {
+        p[i] = pos + __popc(mask[i] & lt);
+        if (key[i] == 0 || p[i] >= max_groups) p[i] = -1;
+        pos += __popc(mask[i]);
+        if (p[i] >= 0) {
+            const uint64_t code = base + i * 32 == nslots - 1 ? ~0ull : ~key[i];
+            write_group(sp, code, static_cast<int32_t>(p[i]), out_seg);
+        }
+    }
+    for (int a = 0; a < sp.naggs; ++a) {
+        const unsigned long long* acc = h.acc + (static_cast<size_t>(base) << h.shift) + a;
+        int64_t* out = sp.agg_out[a];
+        unsigned long long v[kEmitItems];
+#pragma unroll
+        for (int i = 0; i < kEmitItems; ++i)
+            if (p[i] >= 0) v[i] = acc[static_cast<size_t>(i) * 32 << h.shift];
+#pragma unroll
+        for (int i = 0; i < kEmitItems; ++i)
+            if (p[i] >= 0) out[p[i]] = static_cast<int64_t>(v[i]);
+    }
+}
+
+// Dense modes: kDenseBlock (block arrays) and kDenseDirect (rows straight into the
+// dense global array). MODE must agree with sp.direct: the modes are separate kernels
+// so each gets its own register allocation.
+constexpr int kDenseBlock = 1, kDenseDirect = 2;
 
 template <int NA, int MODE, bool PROBE = false>
 __global__ void __launch_bounds__(kThreads)
 groupby_kernel(Spec sp, const int32_t* __restrict__ sel, const int64_t* __restrict__ d_n, int64_t ncap,
                const int64_t* __restrict__ d_seg, GTable g, int64_t max_groups, int32_t* __restrict__ out_seg,
-               int32_t* status, uint32_t hash_slots) {
+               int32_t* status) {
     extern __shared__ __align__(16) unsigned char smem[];
     Smem m = {};
     if (MODE == kDenseBlock) {
         m.rep0 = smem;
         m.occ_words = (sp.D + 31) / 32;
-    } else if (MODE == kHashed) {
-        m.S = hash_slots;
-        m.h_lo = reinterpret_cast<uint32_t*>(smem);
-        m.h_hi = m.h_lo + static_cast<size_t>(sp.naggs) * hash_slots;
-        m.h_key = reinterpret_cast<unsigned long long*>(m.h_hi + static_cast<size_t>(sp.naggs) * hash_slots);
-        m.h_state = reinterpret_cast<uint32_t*>(m.h_key + hash_slots);
-    }
-    if (MODE != kDenseDirect) {
         clear_block_table(sp, m);
         __syncthreads();
     }
@@ -707,10 +896,7 @@ groupby_kernel(Spec sp, const int32_t* __restrict__ sel, const int64_t* __restri
         if (MODE == kDenseDirect) {
             aggregate_range_dense<NA, true, PROBE>(sp, m, sel, pos, qend, q, g, max_groups, out_seg, status);
         } else {
-            if (MODE == kDenseBlock)
-                aggregate_range_dense<NA, false, PROBE>(sp, m, sel, pos, qend, q, g, max_groups, out_seg, status);
-            else
-                aggregate_range<NA>(sp, m, sel, pos, qend, q, g, max_groups, out_seg, status);
+            aggregate_range_dense<NA, false, PROBE>(sp, m, sel, pos, qend, q, g, max_groups, out_seg, status);
             flush_block_table(sp, m, q, g, max_groups, out_seg, status);
         }
         pos = qend;
@@ -1031,11 +1217,6 @@ px_status launch_probe_sum_count(const Spec& sp, int32_t sum_slot, int32_t cnt_s
     return check_launch("px_join_probe_agg sum-count");
 }
 
-constexpr int kEmitThreads = 256;
-constexpr int kEmitItems = 8;
-constexpr int kEmitTile = kEmitThreads * kEmitItems;
-constexpr int kEmitWarps = kEmitThreads / 32;
-
 // Writes the occupied entries of the dense global array as output groups, in
 // (segment, key) order, after the groups the hash path claimed (rows whose keys
 // fell outside the key range). Single pass with a bounded look-back.
@@ -1106,11 +1287,21 @@ uint32_t gtable_slots(int64_t max_groups) {
     return static_cast<uint32_t>(G);
 }
 
-uint32_t hash_slots(int naggs) {
-    uint32_t s = 8192;
-    while (s > 64 && static_cast<size_t>(s) * (12 + 8 * static_cast<size_t>(naggs)) > kSmemBudget) s >>= 1;
+// Slots of the hash mode's block-local cache: keys and split accumulators.
+uint32_t cache_slots(int naggs) {
+    uint32_t s = 4096;
+    while (s * (8 + 8 * static_cast<size_t>(naggs)) > kCacheBudget) s >>= 1;
     return s;
 }
+
+// log2 of a table slot's accumulators, rounded up to a power of two.
+int acc_shift(int naggs) { return naggs <= 1 ? 0 : (naggs == 2 ? 1 : (naggs <= 4 ? 2 : 3)); }
+
+// The table of the hash mode: slots, and bytes with naggs accumulators each.
+size_t htable_bytes(uint32_t slots, int naggs) {
+    return align_up(8 * (static_cast<size_t>(slots) + 1), 256) + (8 * (static_cast<size_t>(slots) + 1) << acc_shift(naggs));
+}
+constexpr size_t kEmittedBytes = 256;  // the emit's counter, before the table
 
 int num_sms() {
     int dev = 0, n = 0;
@@ -1122,7 +1313,7 @@ int num_sms() {
 template <int NA, int MODE, bool PROBE = false>
 px_status launch_mode(const Spec& sp, size_t smem, const int32_t* sel, const int64_t* d_n, int64_t ncap,
                       const int64_t* d_seg, const GTable& g, int64_t max_groups, int32_t* out_seg, int32_t* status,
-                      uint32_t hslots, cudaStream_t st) {
+                      cudaStream_t st) {
     auto kernel = groupby_kernel<NA, MODE, PROBE>;
     cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
     int per_sm = 0;
@@ -1135,36 +1326,33 @@ px_status launch_mode(const Spec& sp, size_t smem, const int32_t* sel, const int
     const int64_t grid = std::max<int64_t>(
         1, std::min<int64_t>(cdiv(ncap, min_rows), static_cast<int64_t>(num_sms()) * std::max(1, per_sm)));
     kernel<<<static_cast<unsigned>(grid), kThreads, smem, st>>>(sp, sel, d_n, ncap, d_seg, g, max_groups, out_seg,
-                                                                status, hslots);
+                                                                status);
     note_launch();
     return check_launch("px_groupby_agg");
 }
 
-// Fused probe: dense modes only (the caller guarantees sp.dense).
+// The dense modes (sp.dense), fused with the probe or not.
 template <int NA>
-px_status launch_probe(const Spec& sp, size_t smem, const int32_t* sel, const int64_t* d_n, int64_t ncap,
+px_status launch_dense(const Spec& sp, size_t smem, const int32_t* sel, const int64_t* d_n, int64_t ncap,
                        const int64_t* d_seg, const GTable& g, int64_t max_groups, int32_t* out_seg, int32_t* status,
-                       uint32_t hslots, cudaStream_t st) {
-    if (sp.direct)
-        return launch_mode<NA, kDenseDirect, true>(sp, smem, sel, d_n, ncap, d_seg, g, max_groups, out_seg, status,
-                                                   hslots, st);
-    return launch_mode<NA, kDenseBlock, true>(sp, smem, sel, d_n, ncap, d_seg, g, max_groups, out_seg, status, hslots,
-                                              st);
+                       cudaStream_t st) {
+    const auto go = [&](auto launch) { return launch(sp, smem, sel, d_n, ncap, d_seg, g, max_groups, out_seg, status, st); };
+    if (sp.probe_fk)
+        return sp.direct ? go(launch_mode<NA, kDenseDirect, true>) : go(launch_mode<NA, kDenseBlock, true>);
+    return sp.direct ? go(launch_mode<NA, kDenseDirect, false>) : go(launch_mode<NA, kDenseBlock, false>);
 }
 
 template <int NA>
-px_status launch(const Spec& sp, size_t smem, const int32_t* sel, const int64_t* d_n, int64_t ncap,
-                 const int64_t* d_seg, const GTable& g, int64_t max_groups, int32_t* out_seg, int32_t* status,
-                 uint32_t hslots, cudaStream_t st) {
-    if (sp.probe_fk)
-        return launch_probe<NA>(sp, smem, sel, d_n, ncap, d_seg, g, max_groups, out_seg, status, hslots, st);
-    if (sp.direct)
-        return launch_mode<NA, kDenseDirect>(sp, smem, sel, d_n, ncap, d_seg, g, max_groups, out_seg, status, hslots,
-                                             st);
-    if (sp.dense)
-        return launch_mode<NA, kDenseBlock>(sp, smem, sel, d_n, ncap, d_seg, g, max_groups, out_seg, status, hslots,
-                                            st);
-    return launch_mode<NA, kHashed>(sp, smem, sel, d_n, ncap, d_seg, g, max_groups, out_seg, status, hslots, st);
+px_status launch_hash(const Spec& sp, const int32_t* sel, const int64_t* d_n, int64_t ncap, const int64_t* d_seg,
+                      const HTable& h, int32_t* status, cudaStream_t st) {
+    auto kernel = groupby_hash_kernel<NA>;
+    const uint32_t C = cache_slots(sp.naggs);
+    const size_t smem = static_cast<size_t>(C) * (8 + 8 * static_cast<size_t>(sp.naggs));
+    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+    const int64_t grid = std::min<int64_t>(cdiv(ncap, kHashTile), static_cast<int64_t>(num_sms()) * kHashBlocksPerSm);
+    kernel<<<static_cast<unsigned>(grid), kHashThreads, smem, st>>>(sp, sel, d_n, ncap, d_seg, h, C, status);
+    note_launch();
+    return check_launch("px_groupby_agg hash");
 }
 
 }  // namespace
@@ -1174,8 +1362,10 @@ using namespace px;
 
 extern "C" {
 
-// Workspace: [header][group counter][hash table: state, key, gidx (G slots)]
-// [dense global: acc (PX_MAX_AGGS x max_groups), occupancy flags (1 byte each)][emit scan scratch].
+// Workspace, dense modes: [header][group counter][claim table: state, key, gidx (G
+// slots)][dense global: acc (PX_MAX_AGGS x max_groups), occupancy flags (1 byte each)]
+// [emit scan scratch]; hash mode: [header][emit counter][table: keys, accumulators (G + 1
+// slots)].
 struct WsLayout {
     size_t counter, state, key, gidx, dg_acc, dg_occ, emit_scan, total;
 };
@@ -1192,7 +1382,8 @@ WsLayout ws_layout(int64_t max_groups) {
     L.dg_acc = L.gidx + align_up(4 * G, 256);
     L.dg_occ = L.dg_acc + align_up(8 * PX_MAX_AGGS * M, 256);
     L.emit_scan = L.dg_occ + align_up(M, 256);
-    L.total = L.emit_scan + scan_scratch_bytes(cdiv(static_cast<int64_t>(M), kEmitTile));
+    L.total = std::max(L.emit_scan + scan_scratch_bytes(cdiv(static_cast<int64_t>(M), kEmitTile)),
+                       kWsScratch + kEmittedBytes + htable_bytes(static_cast<uint32_t>(G), PX_MAX_AGGS));
     return L;
 }
 
@@ -1359,10 +1550,40 @@ static px_status groupby_impl(const px_batch* in, const int32_t* key_cols, int32
         sp.group_w = probe->group->type;
         sp.nbuild = probe->nbuild;
     }
-    const uint32_t hslots = hash_slots(naggs);
-    if (!sp.dense) smem = static_cast<size_t>(hslots) * (12 + 8 * static_cast<size_t>(naggs));
-
     cudaStream_t st = static_cast<cudaStream_t>(stream);
+    int32_t* status = &static_cast<WsHeader*>(d_ws)->status;
+    const int64_t ncap = in->nrows;
+    if (!sp.dense) {
+        // Hash mode. The table has two slots for every possible group; a stream of
+        // calls keeps one table, so its size must not depend on a call's rows.
+        const uint32_t slots = gtable_slots(streaming ? max_groups : std::max<int64_t>(1, std::min(max_groups, ncap)));
+        char* base = static_cast<char*>(d_ws) + kWsScratch;
+        HTable h;
+        h.emitted = reinterpret_cast<unsigned long long*>(base);
+        h.key = reinterpret_cast<unsigned long long*>(base + kEmittedBytes);
+        h.acc = reinterpret_cast<unsigned long long*>(base + kEmittedBytes +
+                                                      align_up(8 * (static_cast<size_t>(slots) + 1), 256));
+        h.slots = slots;
+        h.shift = acc_shift(naggs);
+        if (!accumulate) cudaMemsetAsync(base, 0, kEmittedBytes + htable_bytes(slots, naggs), st);
+        if (ncap > 0) {
+            const int64_t* d_n = d_sel ? d_nsel : in->d_nrows;
+            const auto go = [&](auto launch) { return launch(sp, d_sel, d_n, ncap, d_seg, h, status, st); };
+            switch (naggs) {
+                case 0: s = go(launch_hash<0>); break;
+                case 1: s = go(launch_hash<1>); break;
+                case 2: s = go(launch_hash<2>); break;
+                case 3: s = go(launch_hash<3>); break;
+                case 4: s = go(launch_hash<4>); break;
+                default: s = go(launch_hash<PX_MAX_AGGS>); break;
+            }
+            if (s != PX_OK) return s;
+        }
+        launch_after(hash_emit_kernel, dim3(static_cast<unsigned>(cdiv(static_cast<int64_t>(slots) + 1, kEmitTile))),
+                     dim3(kEmitThreads), 0, st, sp, h, max_groups, d_out_seg, d_ngroups, status);
+        note_launch();
+        return check_launch("px_groupby_agg hash emit");
+    }
     const uint32_t G = gtable_slots(max_groups);
     const WsLayout L = ws_layout(max_groups);
     char* ws = static_cast<char*>(d_ws);
@@ -1388,8 +1609,6 @@ static px_status groupby_impl(const px_batch* in, const int32_t* key_cols, int32
             }
         }
     }
-    const int64_t ncap = in->nrows;
-    int32_t* status = &static_cast<WsHeader*>(d_ws)->status;
     // The lean kernel of the SUM + COUNT shape (see groupby_sum_count_kernel):
     // one key of 4 or 8 bytes, a dense block mode with one replica of a dense
     // global result, no selection, not fused with a probe.
@@ -1431,16 +1650,16 @@ static px_status groupby_impl(const px_batch* in, const int32_t* key_cols, int32
         if (s != PX_OK) return s;
     } else if (ncap > 0) {
         const int64_t* d_n = d_sel ? d_nsel : in->d_nrows;
+        const auto go = [&](auto launch) {
+            return launch(sp, smem, d_sel, d_n, ncap, d_seg, g, max_groups, d_out_seg, status, st);
+        };
         switch (naggs) {
-            case 0: s = launch<0>(sp, smem, d_sel, d_n, ncap, d_seg, g, max_groups, d_out_seg, status, hslots, st); break;
-            case 1: s = launch<1>(sp, smem, d_sel, d_n, ncap, d_seg, g, max_groups, d_out_seg, status, hslots, st); break;
-            case 2: s = launch<2>(sp, smem, d_sel, d_n, ncap, d_seg, g, max_groups, d_out_seg, status, hslots, st); break;
-            case 3: s = launch<3>(sp, smem, d_sel, d_n, ncap, d_seg, g, max_groups, d_out_seg, status, hslots, st); break;
-            case 4: s = launch<4>(sp, smem, d_sel, d_n, ncap, d_seg, g, max_groups, d_out_seg, status, hslots, st); break;
-            default:
-                s = launch<PX_MAX_AGGS>(sp, smem, d_sel, d_n, ncap, d_seg, g, max_groups, d_out_seg, status, hslots,
-                                        st);
-                break;
+            case 0: s = go(launch_dense<0>); break;
+            case 1: s = go(launch_dense<1>); break;
+            case 2: s = go(launch_dense<2>); break;
+            case 3: s = go(launch_dense<3>); break;
+            case 4: s = go(launch_dense<4>); break;
+            default: s = go(launch_dense<PX_MAX_AGGS>); break;
         }
         if (s != PX_OK) return s;
     }

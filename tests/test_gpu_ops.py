@@ -550,3 +550,52 @@ def test_filter_edges_of_steps_and_bounds(px, dtype, n):
             assert m == want.size
             np.testing.assert_array_equal(host(sel, m), want)
             assert bool((sel[m:] == -9).all())
+
+
+# Hash mode (no statistic): row counts around a block's tile (1024 rows), aggregate
+# counts at each accumulator stride, groups within and far past the block cache, keys at
+# both ends of int64 (the largest reads as an empty slot), with and without segments.
+@pytest.mark.parametrize("n,dom", [(1, 1), (1023, 7), (1024, 2000), (1025, 100_000), (50_001, 3), (300_007, 5000),
+                                   (700_001, 10**9)])
+@pytest.mark.parametrize("naggs", [0, 1, 2, 3, 5, 8])
+def test_groupby_hash_edges(px, n, dom, naggs):
+    g = pxdata.rng(n + naggs)
+    k = pxdata.random_column(g, n, np.int64, -dom, dom) * 3_000_000_019
+    k[::5] = np.iinfo(np.int64).max
+    k[1::7] = np.iinfo(np.int64).min
+    a, b = pxdata.random_column(g, n, np.int64), pxdata.random_column(g, n, np.int32)
+    ops = [("SUM", 1, None), ("COUNT", None, None), ("SUM_MUL", 1, 2), ("SUM", 2, None), ("COUNT", None, None),
+           ("SUM_MUL", 2, 2), ("SUM", 1, None), ("SUM", 2, None)][:naggs]
+    cols = [k, a, b]
+    aggs = [(getattr(px, "PX_" + o), x, y) for o, x, y in ops]
+    oaggs = [(getattr(oracle, o), None if x is None else cols[x], None if y is None else cols[y]) for o, x, y in ops]
+    want = oracle.groupby([k], oaggs)
+    ws = px.Workspace(256)
+    res = _gb(px, cols, [0], aggs, max(1, want["ngroups"]), ws=ws)
+    assert_groups_equal(res, want, 1)
+    k32 = (k % 2**31 - 2**30).astype(np.int32)  # segments need key bits to spare
+    seg = np.array([0, n // 3, n // 3, n // 2, n], np.int64)
+    want = oracle.groupby([k32], oaggs, seg=seg)
+    res = _gb(px, [k32, a, b], [0], aggs, max(1, want["ngroups"]), seg=dev(seg), ws=ws)
+    assert_groups_equal(res, want, 1, segmented=True)
+    assert ws.status() == px.PX_OK
+
+
+def test_groupby_hash_stream_keeps_its_table(px):
+    # calls of one stream, one of them empty, each reporting into another count, the
+    # last one's row count read from the word its group count goes to
+    g = pxdata.rng(77)
+    n = 20_000
+    k, a = pxdata.random_column(g, n, np.int64, 0, 3000), pxdata.random_column(g, n, np.int64)
+    aggs = [(px.PX_SUM, 1, None), (px.PX_COUNT, None, None)]
+    out = [torch.zeros(4000, dtype=torch.int64, device="cuda") for _ in range(3)]
+    ws = px.Workspace(256).ensure(px.load().px_groupby_ws_bytes(n, 4000))
+    counts = []
+    for i, (lo, hi) in enumerate([(0, 0), (0, 5000), (5000, 5000), (5000, n)]):
+        ng = dev(np.array([n - 5000 if i == 3 else -1], np.int64))
+        res = px.px_groupby_agg([dev(k[lo:hi]), dev(a[lo:hi])], [0], aggs, max_groups=4000, out=out, ws=ws, ngroups=ng,
+                                d_nrows=ng if i == 3 else None, flags=px.PX_AGG_ACCUMULATE if i else px.PX_AGG_STREAM)
+        counts.append(count(ng))
+    assert counts[:3] == [0, np.unique(k[:5000]).size, np.unique(k[:5000]).size]
+    assert ws.status() == px.PX_OK
+    assert_groups_equal(res, oracle.groupby([k], [(oracle.SUM, a, None), (oracle.COUNT, None, None)]), 1)
