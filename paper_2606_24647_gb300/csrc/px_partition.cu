@@ -12,12 +12,19 @@
 //                offsets[q] = start of (q, tile 0).
 //   3. scatter - stages the tile of every column into shared memory with one TMA
 //                bulk copy per column (all in flight together, completed on an
-//                mbarrier; plain loads for gathers through a selection and for a
-//                ragged last tile), ranks rows stably inside the tile with a warp
-//                multi-split (one ballot per partition-id bit gives the lanes with
-//                the same partition) and per-warp counters, then per column moves
-//                the values into partition order in shared memory and writes each
-//                partition's run contiguously, so the stores coalesce.
+//                mbarrier; plain loads for a ragged last tile), ranks rows stably
+//                inside the tile with a warp multi-split (one ballot per partition-id
+//                bit gives the lanes with the same partition) and per-warp counters,
+//                then per column moves the values into partition order in shared
+//                memory and writes each partition's run contiguously, so the stores
+//                coalesce.
+//      direct  - the scatter for rows read through a selection and for many
+//                partitions: the same ranking, but each column goes from global
+//                memory through registers into one partition-ordered buffer, the
+//                next column's loads in flight while this one is written. Through a
+//                selection of 98 % of 20M 30-byte rows: 8 partitions 428 -> 330 us,
+//                64 473 -> 355 us (staging loaded every row number once per column and
+//                held tiles to 1024 rows).
 // The key column is read twice (hist and scatter); every other column once; every
 // column written once.
 #include <algorithm>
@@ -28,10 +35,9 @@
 namespace px {
 namespace {
 
+constexpr size_t kStageBudget = 48 * 1024;  // raw tile staging bytes (all columns)
 constexpr int kThreads = 256;
 constexpr int kWarps = kThreads / 32;
-constexpr size_t kStageBudget = 48 * 1024;  // raw tile staging bytes (all columns)
-constexpr int kOffRegs = (PX_MAX_PARTS + kThreads - 1) / kThreads;  // partitions per thread, at most
 
 constexpr int kScanThreads = 256;
 constexpr int kScanItems = 32;  // 8192 counts per scan tile: a short look-back chain
@@ -240,8 +246,118 @@ __device__ __forceinline__ void stage_plain(const T* in, T* staged, const int32_
     }
 }
 
-// NBITS: bits of the largest partition id (nparts - 1), so the multi-split below
-// is unrolled: one ballot per id bit, plus one for the valid rows of a ragged tile.
+// Consecutive partitions a thread turns into tile positions: as many as cover every
+// partition, and two for up to 64, which then stay within one warp.
+template <int NBITS>
+constexpr int kPer = NBITS > 8 ? (1 << NBITS) / kThreads : (NBITS == 6 ? 2 : 1);
+
+// From the partition of every row (pidv, nparts past a ragged tile's end) to its
+// position in the tile's partition order (posv), and the output row of the position
+// each thread writes (dest[k]: position threadIdx.x + k * kThreads, -1 past the tile).
+// my_off: the tile's output start in each of the thread's partitions. s_whist:
+// kWarps x (nparts + 1) counters, zero on entry; s_delta: nparts; s_dest: the tile's
+// rows; s_part: kWarps. NBITS: bits of the largest partition id (nparts - 1), so the
+// multi-split is unrolled: one ballot per id bit, plus one for the valid rows of a
+// ragged tile. FT: a full tile, where every position holds a row (no per-row checks).
+// Holds barriers: call from all threads, the counters' clearing behind the first.
+template <int ITEMS, int NBITS, bool FT>
+__device__ __forceinline__ void rank_tile(const uint32_t* pidv, int32_t* posv, int32_t* dest,
+                                          const int32_t (&my_off)[kPer<NBITS>], int32_t* s_whist, int32_t* s_delta,
+                                          int32_t* s_dest, int32_t* s_part, uint32_t nparts, int tile_rows) {
+    constexpr int PER = kPer<NBITS>;
+    const int np1 = static_cast<int>(nparts) + 1;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    // The stable rank inside the warp's run: the lanes with the same partition id come
+    // from one ballot per id bit (multi-split); a per-warp counter row carries ranks
+    // across the thread's items.
+    int32_t* wh = s_whist + warp * np1;
+    const uint32_t lt = lanemask_lt();
+#pragma unroll
+    for (int i = 0; i < ITEMS; ++i) {
+        // A row past a ragged tile's end has p = nparts and is in no valid row's
+        // peer set; it never updates a counter (it is not its own peers' leader).
+        const uint32_t p = pidv[i];
+        uint32_t peers = FT ? FULL : __ballot_sync(FULL, p < nparts);
+#pragma unroll
+        for (int b = 0; b < NBITS; ++b) {
+            const bool bit = (p >> b) & 1u;
+            const uint32_t bal = __ballot_sync(FULL, bit);
+            peers &= bit ? bal : ~bal;
+        }
+        const int32_t base = wh[p];
+        __syncwarp();
+        if (lane == __ffs(peers) - 1) wh[p] = base + __popc(peers);
+        __syncwarp();
+        posv[i] = base + __popc(peers & lt);
+    }
+    __syncthreads();
+    // Every thread takes its PER partitions (one warp walking all of them while the
+    // others wait: 256 partitions, 20M x 20 B rows 341 us, now 273; 1024: 835, now
+    // 615): the start of each partition's run in the tile (block scan of the
+    // partitions' counts) plus each warp's start inside the run (scan of the warps'
+    // counters) turn s_whist[w][q] into the tile position of warp w's first row of
+    // partition q, and s_delta[q] into the shift from a tile position in partition q's
+    // run to its output row.
+    {
+        int32_t run[PER], sum = 0;
+#pragma unroll
+        for (int r = 0; r < PER; ++r) {
+            const int q = tid * PER + r;
+            run[r] = 0;
+            if (q < static_cast<int>(nparts))
+                for (int w = 0; w < kWarps; ++w) run[r] += s_whist[w * np1 + q];
+            sum += run[r];
+        }
+        int32_t at = 0;
+        if (warp * 32 * PER < static_cast<int>(nparts)) at = warp_incl_scan(sum);
+        if (nparts > 32 * PER) {  // more than one warp's partitions
+            if (lane == 31) s_part[warp] = at;
+            __syncthreads();
+            const int32_t before = lane < warp ? s_part[lane] : 0;
+            at += static_cast<int32_t>(__reduce_add_sync(FULL, static_cast<uint32_t>(before)));
+        }
+        at -= sum;
+#pragma unroll
+        for (int r = 0; r < PER; ++r) {
+            const int q = tid * PER + r;
+            if (q < static_cast<int>(nparts)) {
+                s_delta[q] = my_off[r] - at;
+                for (int w = 0; w < kWarps; ++w) {
+                    const int32_t c = s_whist[w * np1 + q];
+                    s_whist[w * np1 + q] = at;
+                    at += c;
+                }
+            }
+        }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < ITEMS; ++i) {
+        if (FT || pidv[i] < nparts) {
+            posv[i] += wh[pidv[i]];
+            s_dest[posv[i]] = posv[i] + s_delta[pidv[i]];
+        }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < ITEMS; ++k) {
+        const int jj = tid + k * kThreads;
+        dest[k] = FT || jj < tile_rows ? s_dest[jj] : -1;
+    }
+}
+
+// The tile's output start in each of this thread's partitions (one strided load each).
+template <int NBITS>
+__device__ __forceinline__ void load_offs(int32_t (&my_off)[kPer<NBITS>], const int32_t* __restrict__ offs,
+                                          uint32_t nparts, int64_t ntiles, int64_t tile) {
+#pragma unroll
+    for (int r = 0; r < kPer<NBITS>; ++r) {
+        const int q = threadIdx.x * kPer<NBITS> + r;
+        my_off[r] = q < static_cast<int>(nparts) ? offs[static_cast<int64_t>(q) * ntiles + tile] : 0;
+    }
+}
+
+// NBITS: see rank_tile.
 template <int ITEMS, int NBITS>
 __global__ void __launch_bounds__(kThreads, ITEMS >= 8 ? 3 : 4)
 part_scatter_kernel(Cols cols, int32_t key_col, const int32_t* __restrict__ sel,
@@ -260,6 +376,8 @@ part_scatter_kernel(Cols cols, int32_t key_col, const int32_t* __restrict__ sel,
     int32_t* s_whist = s_delta + np1p;                                             // kWarps x np1
     // partition ids from the histogram pass (T bytes), when it wrote them
     uint8_t* s_pid = smem + ((stage_bytes + T * 12 + 16 + (np1p + kWarps * np1) * 4 + 15) & ~15u);
+
+    __shared__ int32_t s_part[kWarps];  // rank_tile's
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int64_t tile = blockIdx.x;
@@ -288,14 +406,9 @@ part_scatter_kernel(Cols cols, int32_t key_col, const int32_t* __restrict__ sel,
         }
     }
     wait_prior();  // the scan's offsets, and the histogram's ids before it
-    // This tile's output start in each partition (one strided load per partition),
-    // requested now so its latency hides behind the staging of the tile.
-    int32_t my_off[kOffRegs];
-#pragma unroll
-    for (int r = 0; r < kOffRegs; ++r) {
-        const int q = tid + r * kThreads;
-        my_off[r] = q < static_cast<int>(nparts) ? offs[static_cast<int64_t>(q) * ntiles + tile] : 0;
-    }
+    // Requested now so their latency hides behind the staging of the tile.
+    int32_t my_off[kPer<NBITS>];
+    load_offs<NBITS>(my_off, offs, nparts, ntiles, tile);
     if (bulk) {
         if (tid == 0 && pid_in) bulk_g2s(s_pid, pid_in + tbase, static_cast<uint32_t>(T), bar);
         if (!mbar_wait(bar, 0) && lane == 0) set_status(status, PX_ERR_TIMEOUT);
@@ -320,9 +433,6 @@ part_scatter_kernel(Cols cols, int32_t key_col, const int32_t* __restrict__ sel,
     // The rest runs specialised for a full tile (every position a row) or not.
     auto finish = [&](auto full_tile) {
         constexpr bool FT = decltype(full_tile)::value;
-        // Partition of every row, then its stable rank inside the warp's run: the lanes
-        // with the same partition id come from one ballot per id bit (multi-split); a
-        // per-warp counter row carries ranks across the thread's items.
         const int64_t* keys = reinterpret_cast<const int64_t*>(stage + cols.stage_off[key_col]);
         uint32_t pidv[ITEMS];
         int32_t posv[ITEMS];
@@ -332,72 +442,8 @@ part_scatter_kernel(Cols cols, int32_t key_col, const int32_t* __restrict__ sel,
             pidv[i] = FT || lp < tile_rows ? (pid_in ? static_cast<uint32_t>(s_pid[lp]) : part_of(keys[lp], seed, nparts))
                                            : nparts;
         }
-        int32_t* wh = s_whist + warp * np1;
-        const uint32_t lt = lanemask_lt();
-#pragma unroll
-        for (int i = 0; i < ITEMS; ++i) {
-            // A row past a ragged tile's end has p = nparts and is in no valid row's
-            // peer set; it never updates a counter (it is not its own peers' leader).
-            const uint32_t p = pidv[i];
-            uint32_t peers = FT ? FULL : __ballot_sync(FULL, p < nparts);
-#pragma unroll
-            for (int b = 0; b < NBITS; ++b) {
-                const bool bit = (p >> b) & 1u;
-                const uint32_t bal = __ballot_sync(FULL, bit);
-                peers &= bit ? bal : ~bal;
-            }
-            const int32_t base = wh[p];
-            __syncwarp();
-            if (lane == __ffs(peers) - 1) wh[p] = base + __popc(peers);
-            __syncwarp();
-            posv[i] = base + __popc(peers & lt);
-        }
-#pragma unroll
-        for (int r = 0; r < kOffRegs; ++r) {
-            const int q = tid + r * kThreads;
-            if (q < static_cast<int>(nparts)) s_delta[q] = my_off[r];
-        }
-        __syncthreads();
-        // Warp 0, 32 partitions at a time: the start of each partition's run in the tile
-        // (warp scan of the partitions' counts) plus each warp's start inside the run
-        // (scan of the warps' counters) turn s_whist[w][q] into the tile position of
-        // warp w's first row of partition q, and s_delta[q] into the shift from a tile
-        // position in partition q's run to its output row.
-        if (warp == 0) {
-            int32_t carry = 0;
-            for (int base = 0; base < static_cast<int>(nparts); base += 32) {
-                const int q = base + lane;
-                int32_t run = 0;
-                if (q < static_cast<int>(nparts))
-                    for (int w = 0; w < kWarps; ++w) run += s_whist[w * np1 + q];
-                const int32_t incl = warp_incl_scan(run);
-                if (q < static_cast<int>(nparts)) {
-                    int32_t at = carry + incl - run;
-                    s_delta[q] -= at;
-                    for (int w = 0; w < kWarps; ++w) {
-                        const int32_t c = s_whist[w * np1 + q];
-                        s_whist[w * np1 + q] = at;
-                        at += c;
-                    }
-                }
-                carry += __shfl_sync(FULL, incl, 31);
-            }
-        }
-        __syncthreads();
-#pragma unroll
-        for (int i = 0; i < ITEMS; ++i) {
-            if (FT || pidv[i] < nparts) {
-                posv[i] += wh[pidv[i]];
-                s_dest[posv[i]] = posv[i] + s_delta[pidv[i]];
-            }
-        }
-        __syncthreads();
         int32_t dest[ITEMS];
-#pragma unroll
-        for (int k = 0; k < ITEMS; ++k) {
-            const int jj = tid + k * kThreads;
-            dest[k] = FT || jj < tile_rows ? s_dest[jj] : -1;
-        }
+        rank_tile<ITEMS, NBITS, FT>(pidv, posv, dest, my_off, s_whist, s_delta, s_dest, s_part, nparts, tile_rows);
 
         // Column phases, one barrier each: phase k writes column order[k-1] to global
         // memory from its partition-ordered buffer while moving column order[k] into
@@ -432,11 +478,111 @@ part_scatter_kernel(Cols cols, int32_t key_col, const int32_t* __restrict__ sel,
     else finish(std::false_type{});
 }
 
+// The values of one column at this thread's rows of the tile, sign-extended.
+template <typename T, int ITEMS, bool FT>
+__device__ __forceinline__ void gather_t(const void* in, const int32_t* row, int64_t* v) {
+#pragma unroll
+    for (int i = 0; i < ITEMS; ++i)
+        if (FT || row[i] >= 0) v[i] = static_cast<int64_t>(static_cast<const T*>(in)[row[i]]);
+}
+template <int ITEMS, bool FT>
+__device__ __forceinline__ void gather_rows(const void* in, int w, const int32_t* row, int64_t* v) {
+    if (w == 8) gather_t<int64_t, ITEMS, FT>(in, row, v);
+    else if (w == 4) gather_t<int32_t, ITEMS, FT>(in, row, v);
+    else gather_t<int8_t, ITEMS, FT>(in, row, v);
+}
+template <typename T, int ITEMS, bool FT>
+__device__ __forceinline__ void place_t(void* buf, const int32_t* row, const int32_t* posv, const int64_t* v) {
+#pragma unroll
+    for (int i = 0; i < ITEMS; ++i)
+        if (FT || row[i] >= 0) static_cast<T*>(buf)[posv[i]] = static_cast<T>(v[i]);
+}
+
+// The scatter without staging: every thread keeps its rows' values of one column in
+// registers and moves them into partition order in one shared-memory buffer, loading
+// the next column's before it writes this one out. For rows read through a selection
+// (a row number loaded once serves every column) and for rows too wide to stage whole
+// tiles of 2048.
+template <int ITEMS, int NBITS>
+__global__ void __launch_bounds__(kThreads, ITEMS >= 8 ? 3 : 4)
+part_direct_kernel(Cols cols, int32_t key_col, const int32_t* __restrict__ sel, const int64_t* __restrict__ d_nsel,
+                   int64_t ncap, uint64_t seed, uint32_t nparts, const int32_t* __restrict__ offs, int64_t ntiles,
+                   const uint8_t* __restrict__ pid_in) {
+    constexpr int T = kThreads * ITEMS;
+    extern __shared__ __align__(16) unsigned char smem[];
+    int32_t* s_dest = reinterpret_cast<int32_t*>(smem + T * 8);  // after the buffer of T 8-byte values
+    const int np1 = static_cast<int>(nparts) + 1;
+    int32_t* s_delta = s_dest + T;
+    int32_t* s_whist = s_delta + np1;
+    __shared__ int32_t s_part[kWarps];
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int64_t tile = blockIdx.x;
+    const int64_t n = actual_rows(d_nsel, ncap);
+    const int64_t tbase = tile * T;
+    const int64_t rem = n - tbase;
+    const int tile_rows = rem <= 0 ? 0 : (rem < T ? static_cast<int>(rem) : T);
+    for (int k = tid; k < kWarps * np1; k += kThreads) s_whist[k] = 0;
+
+    auto run = [&](auto full_tile) {
+        constexpr bool FT = decltype(full_tile)::value;
+        // Row numbers and the first column come from earlier calls: loaded before the
+        // wait for the scan.
+        int32_t row[ITEMS];
+        int64_t v[ITEMS];
+#pragma unroll
+        for (int i = 0; i < ITEMS; ++i) {
+            const int lp = local_pos<ITEMS>(warp, i, lane);
+            row[i] = FT || lp < tile_rows ? (sel ? sel[tbase + lp] : static_cast<int32_t>(tbase + lp)) : -1;
+        }
+        gather_rows<ITEMS, FT>(cols.in[cols.order[0]], cols.width[cols.order[0]], row, v);
+        wait_prior();  // the scan's offsets, and the histogram's ids before it
+        int32_t my_off[kPer<NBITS>];
+        load_offs<NBITS>(my_off, offs, nparts, ntiles, tile);
+        int32_t posv[ITEMS], dest[ITEMS];
+        {
+            uint32_t pidv[ITEMS];
+            if (pid_in) {
+#pragma unroll
+                for (int i = 0; i < ITEMS; ++i)
+                    pidv[i] = FT || row[i] >= 0 ? pid_in[tbase + local_pos<ITEMS>(warp, i, lane)] : nparts;
+            } else {
+                const int64_t* keys = static_cast<const int64_t*>(cols.in[key_col]);
+#pragma unroll
+                for (int i = 0; i < ITEMS; ++i)
+                    pidv[i] = FT || row[i] >= 0 ? part_of(keys[row[i]], seed, nparts) : nparts;
+            }
+            __syncthreads();  // the counters are clear
+            rank_tile<ITEMS, NBITS, FT>(pidv, posv, dest, my_off, s_whist, s_delta, s_dest, s_part, nparts, tile_rows);
+        }
+        for (int k = 0; k < cols.ncols; ++k) {
+            const int c = cols.order[k], w = cols.width[c];
+            if (w == 8) place_t<int64_t, ITEMS, FT>(smem, row, posv, v);
+            else if (w == 4) place_t<int32_t, ITEMS, FT>(smem, row, posv, v);
+            else place_t<int8_t, ITEMS, FT>(smem, row, posv, v);
+            __syncthreads();
+            if (k + 1 < cols.ncols) gather_rows<ITEMS, FT>(cols.in[cols.order[k + 1]], cols.width[cols.order[k + 1]], row, v);
+            if (w == 8) store_col<int64_t, ITEMS, FT>(smem, dest, cols.out[c]);
+            else if (w == 4) store_col<int32_t, ITEMS, FT>(smem, dest, cols.out[c]);
+            else store_col<int8_t, ITEMS, FT>(smem, dest, cols.out[c]);
+            __syncthreads();  // the buffer is free
+        }
+    };
+    if (tile_rows == T) run(std::true_type{});
+    else run(std::false_type{});
+}
+
+int id_bits(int32_t nparts) { return nparts <= 1 ? 0 : 32 - __builtin_clz(static_cast<unsigned>(nparts - 1)); }
+
 size_t scatter_smem_bytes(int items, uint32_t stage_bytes, int32_t nparts) {
     const size_t T = static_cast<size_t>(kThreads) * items;
     const size_t np1 = static_cast<size_t>(nparts) + 1;
     const size_t np1p = (np1 + 3) & ~static_cast<size_t>(3);
     return align_up(stage_bytes + T * 12 + 16 + np1p * 4 + kWarps * np1 * 4, size_t(16)) + T;  // + ids
+}
+
+size_t direct_smem_bytes(int items, int32_t nparts) {
+    const size_t np1 = static_cast<size_t>(nparts) + 1;
+    return static_cast<size_t>(kThreads) * items * 12 + np1 * 4 + kWarps * np1 * 4;
 }
 
 // Workspace: count matrix, offset matrix (partition-major, P x tiles int32) and the
@@ -471,8 +617,8 @@ PartScratch part_scratch(void* d_ws, int64_t nrows, int64_t ntiles, int32_t npar
 template <int ITEMS>
 px_status launch_partition(const Cols& cols, int32_t key_col, const int32_t* d_sel, const int64_t* d_n, int64_t ncap,
                            uint64_t seed, int32_t nparts, int64_t* d_offsets, const PartScratch& ps, int64_t ntiles,
-                           uint32_t stage_bytes, uint32_t row_bytes, int32_t blocks_per_sm, int32_t* status,
-                           cudaStream_t st) {
+                           uint32_t stage_bytes, uint32_t row_bytes, bool direct, int32_t blocks_per_sm,
+                           int32_t* status, cudaStream_t st) {
     px_status s;
     const int64_t* key = static_cast<const int64_t*>(cols.in[key_col]);
     cudaMemsetAsync(ps.scan, 0, ps.scan_bytes, st);  // before the histogram: the scan launches right after it
@@ -488,7 +634,7 @@ px_status launch_partition(const Cols& cols, int32_t key_col, const int32_t* d_s
     note_launch();
     if ((s = check_launch("px_partition scan")) != PX_OK) return s;
 
-    size_t smem = scatter_smem_bytes(ITEMS, stage_bytes, nparts);
+    size_t smem = direct ? direct_smem_bytes(ITEMS, nparts) : scatter_smem_bytes(ITEMS, stage_bytes, nparts);
     if (blocks_per_sm > 0) {
         int dev = 0, per_sm_smem = 0;
         cudaGetDevice(&dev);
@@ -500,25 +646,33 @@ px_status launch_partition(const Cols& cols, int32_t key_col, const int32_t* d_s
         cudaDeviceGetAttribute(&max_block, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
         if (want > smem) smem = std::min(want, static_cast<size_t>(max_block));
     }
-    auto go = [&](auto kern) {
+    auto go = [&](auto bits) {
+        if (direct) {
+            const auto kern = part_direct_kernel<ITEMS, decltype(bits)::value>;
+            cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+            launch_after(kern, dim3(static_cast<unsigned>(ntiles)), dim3(kThreads), smem, st, cols, key_col, d_sel, d_n,
+                         ncap, seed, static_cast<uint32_t>(nparts), ps.offs, ntiles, ps.pid);
+            return;
+        }
+        const auto kern = part_scatter_kernel<ITEMS, decltype(bits)::value>;
         cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
         launch_after(kern, dim3(static_cast<unsigned>(ntiles)), dim3(kThreads), smem, st, cols, key_col, d_sel, d_n,
                      ncap, seed, static_cast<uint32_t>(nparts), ps.offs, ntiles, stage_bytes, row_bytes, ps.pid,
                      status);
     };
     static_assert(PX_MAX_PARTS <= 1024, "partition ids need at most 10 bits");
-    switch (nparts <= 1 ? 0 : 32 - __builtin_clz(static_cast<unsigned>(nparts - 1))) {
-        case 0: go(part_scatter_kernel<ITEMS, 0>); break;
-        case 1: go(part_scatter_kernel<ITEMS, 1>); break;
-        case 2: go(part_scatter_kernel<ITEMS, 2>); break;
-        case 3: go(part_scatter_kernel<ITEMS, 3>); break;
-        case 4: go(part_scatter_kernel<ITEMS, 4>); break;
-        case 5: go(part_scatter_kernel<ITEMS, 5>); break;
-        case 6: go(part_scatter_kernel<ITEMS, 6>); break;
-        case 7: go(part_scatter_kernel<ITEMS, 7>); break;
-        case 8: go(part_scatter_kernel<ITEMS, 8>); break;
-        case 9: go(part_scatter_kernel<ITEMS, 9>); break;
-        default: go(part_scatter_kernel<ITEMS, 10>); break;
+    switch (id_bits(nparts)) {
+        case 0: go(std::integral_constant<int, 0>{}); break;
+        case 1: go(std::integral_constant<int, 1>{}); break;
+        case 2: go(std::integral_constant<int, 2>{}); break;
+        case 3: go(std::integral_constant<int, 3>{}); break;
+        case 4: go(std::integral_constant<int, 4>{}); break;
+        case 5: go(std::integral_constant<int, 5>{}); break;
+        case 6: go(std::integral_constant<int, 6>{}); break;
+        case 7: go(std::integral_constant<int, 7>{}); break;
+        case 8: go(std::integral_constant<int, 8>{}); break;
+        case 9: go(std::integral_constant<int, 9>{}); break;
+        default: go(std::integral_constant<int, 10>{}); break;
     }
     note_launch();
     return check_launch("px_partition scatter");
@@ -599,7 +753,17 @@ px_status px_partition_tuned(const px_batch* in, int32_t key_col, const int32_t*
     // Rows per thread: the caller's choice when a tile of every column fits the
     // staging budget, else the widest that fits.
     const int fit = items_for(row_bytes);
-    const int items = items_req > 0 && items_req <= fit ? items_req : fit;
+    const int staged = items_req > 0 && items_req <= fit ? items_req : fit;
+    // The kernel without staging (see part_direct_kernel): through a selection; with many
+    // partitions, whose short runs make the writes the bound (20M rows, staged against
+    // not: fact columns at 256 partitions 274 and 266 us, at 1024 623 and 599; four 8-byte
+    // columns at 256 471 and 367, at 64 296 and 282, at 16 246 and 273; the six columns of
+    // the plain batch at 200 453 and 366, at 64 300 and 311). A caller's own shape is
+    // staged. Tiles of 1024 rows while 2048 would not give every SM two.
+    const bool shaped = items_req > 0 && items_req <= fit;
+    const bool direct =
+        d_sel || (!shaped && (nparts > 64 || (nparts > 32 && fit < 8 && static_cast<int>(row_bytes) >= 6 * in->ncols)));
+    const int items = direct ? (ncap >= 2 * 2048 * static_cast<int64_t>(sm_count()) ? 8 : 4) : staged;
     const int64_t T = static_cast<int64_t>(kThreads) * items;
     uint32_t stage_bytes = 0;
     for (int c = 0; c < in->ncols; ++c) {
@@ -612,12 +776,12 @@ px_status px_partition_tuned(const px_batch* in, int32_t key_col, const int32_t*
     const int64_t* d_n = d_sel ? d_nsel : in->d_nrows;
     if (items == 8)
         return launch_partition<8>(cols, key_col, d_sel, d_n, ncap, seed, nparts, d_offsets, ps, ntiles, stage_bytes,
-                                   row_bytes, bps, status, st);
+                                   row_bytes, direct, bps, status, st);
     if (items == 4)
         return launch_partition<4>(cols, key_col, d_sel, d_n, ncap, seed, nparts, d_offsets, ps, ntiles, stage_bytes,
-                                   row_bytes, bps, status, st);
+                                   row_bytes, direct, bps, status, st);
     return launch_partition<2>(cols, key_col, d_sel, d_n, ncap, seed, nparts, d_offsets, ps, ntiles, stage_bytes,
-                               row_bytes, bps, status, st);
+                               row_bytes, direct, bps, status, st);
 }
 
 px_status px_partition(const px_batch* in, int32_t key_col, const int32_t* d_sel, const int64_t* d_nsel,

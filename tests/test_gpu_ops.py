@@ -599,3 +599,25 @@ def test_groupby_hash_stream_keeps_its_table(px):
     assert counts[:3] == [0, np.unique(k[:5000]).size, np.unique(k[:5000]).size]
     assert ws.status() == px.PX_OK
     assert_groups_equal(res, oracle.groupby([k], [(oracle.SUM, a, None), (oracle.COUNT, None, None)]), 1)
+
+
+# The exchange's two scatter kernels at their edges: row counts around tiles of 1024 and
+# 2048 rows (2048 from 2 tiles per SM on), partition counts on both sides of every rule
+# and id width, rows through a selection or not, a launch shape named or not.
+@pytest.mark.parametrize("P", [1, 32, 33, 64, 65, 256, 257, 513, 1024])
+@pytest.mark.parametrize("n", [1, 1023, 1025, 4097, 700_001])
+def test_partition_scatter_kernels_edges(px, P, n):
+    g = pxdata.rng(P + n)
+    wide = [pxdata.random_column(g, n, np.int64) for _ in range(4)]
+    mixed = [pxdata.random_column(g, n, t) for t in (np.int8, np.int64, np.int32, np.int64, np.int8)]
+    keep = g.random(n) < 0.9
+    sel = np.flatnonzero(keep).astype(np.int32)
+    for cols, key in ((wide, 0), (mixed, 3)):
+        for s in (None, sel):
+            for config in (None, (4, 0)) if n < 10**5 else (None,):
+                want, woff = oracle.partition(cols, key, P, 5, sel=s)
+                kw = {} if s is None else dict(sel=dev(s), nsel=dev(np.array([s.size], np.int64)))
+                out, off = px.px_partition([dev(c) for c in cols], key, P, 5, config=config, **kw)
+                np.testing.assert_array_equal(host(off), woff)
+                for o, w in zip(out, want):
+                    np.testing.assert_array_equal(host(o, w.size), w)
