@@ -453,6 +453,7 @@ frag_emit_kernel(const PlanHeader* __restrict__ ph, const int64_t* __restrict__ 
     __shared__ int64_t s_tile;
     __shared__ int64_t s_excl;
     __shared__ int32_t s_warp[kEmitThreads / 32];
+    wait_prior();  // the accumulators (and the plan)
     const int64_t tile = next_tile(counter, &s_tile);
     const int p = find_frag(emit_start, ph->nfrags, tile);
     const FragDev& f = fd[p];
@@ -517,7 +518,7 @@ frag_emit_kernel(const PlanHeader* __restrict__ ph, const int64_t* __restrict__ 
 bool valid_type(int32_t t) { return t == PX_I8 || t == PX_I32 || t == PX_I64; }
 
 struct WsLayout {
-    size_t counters, plan, acc, states, total;
+    size_t plan, counters, acc, states, total;
 };
 
 // Accumulator bytes of fragment f: naggs x D 64-bit words, then D occupancy flags
@@ -535,9 +536,9 @@ size_t frag_state_bytes(const px_fragment& f) {
 
 WsLayout frag_ws_layout(const px_fragment* frags, int32_t n) {
     WsLayout L;
-    L.counters = kWsScratch;
-    L.plan = L.counters + 256;
-    L.acc = L.plan + align_up(plan_layout(n).total, 256);
+    L.plan = kWsScratch;
+    L.counters = L.plan + align_up(plan_layout(n).total, 256);  // cleared with what follows
+    L.acc = L.counters + 256;
     size_t acc = 0, st = 0;
     for (int32_t i = 0; i < n; ++i) {
         acc += frag_acc_bytes(frags[i]);
@@ -775,8 +776,7 @@ px_status px_fragments_run(const px_fragment* frags, int32_t nfrags, const px_fr
     char* dplan = ws + L.plan;
     unsigned long long* counters = reinterpret_cast<unsigned long long*>(ws + L.counters);
     int32_t* status = &static_cast<WsHeader*>(d_ws)->status;
-    cudaMemsetAsync(counters, 0, 256, st);
-    cudaMemsetAsync(ws + L.acc, 0, L.total - L.acc, st);
+    cudaMemsetAsync(ws + L.counters, 0, L.total - L.counters, st);
     cudaMemcpyAsync(dplan, h_plan, PL.total, cudaMemcpyHostToDevice, st);
     const PlanHeader* d_ph = reinterpret_cast<const PlanHeader*>(dplan);
     const int64_t* d_items = reinterpret_cast<const int64_t*>(dplan + PL.items);
@@ -798,7 +798,8 @@ px_status px_fragments_run(const px_fragment* frags, int32_t nfrags, const px_fr
         else s = c.items == 2 ? go(t512, i2) : go(t512, i4);
         if (s != PX_OK) return s;
     }
-    frag_emit_kernel<<<static_cast<unsigned>(emits), kEmitThreads, 0, st>>>(d_ph, d_emits, d_fd, counters + 1, status);
+    launch_after(frag_emit_kernel, dim3(static_cast<unsigned>(emits)), dim3(kEmitThreads), 0, st, d_ph, d_emits, d_fd,
+                 counters + 1, status);
     note_launch();
     return check_launch("px_fragments_run emit");
 }

@@ -598,10 +598,10 @@ probe_seg_kernel(TableView t, int32_t S, int32_t segmented, const int64_t* __res
     }
 }
 
-// Probe workspace: [header][mrow: 4 B per position][tile counts][tile offsets]
-// [scan scratch over the tile counts].
+// Probe workspace: [header][mrow: 4 B per position][tile counts][scan scratch over the
+// tile counts][tile offsets]; counts and scratch are cleared together.
 struct ProbeWs {
-    size_t mrow, cnt, off, scan, total;
+    size_t mrow, cnt, scan, off, total;
     int64_t ntiles, nscan;
 };
 
@@ -612,9 +612,9 @@ ProbeWs probe_ws_layout(int64_t nprobe) {
     L.nscan = cdiv(L.ntiles, kScanTile);
     L.mrow = kWsScratch;
     L.cnt = L.mrow + align_up(4 * static_cast<size_t>(nprobe), 256);
-    L.off = L.cnt + align_up(4 * static_cast<size_t>(L.ntiles), 256);
-    L.scan = L.off + align_up(8 * static_cast<size_t>(L.ntiles), 256);
-    L.total = L.scan + scan_scratch_bytes(L.nscan);
+    L.scan = L.cnt + align_up(4 * static_cast<size_t>(L.ntiles), 256);
+    L.off = L.scan + scan_scratch_bytes(L.nscan);
+    L.total = L.off + align_up(8 * static_cast<size_t>(L.ntiles), 256);
     return L;
 }
 
@@ -756,8 +756,7 @@ px_status px_join_probe(const void* d_table, const px_batch* probe, int32_t fk_c
     int32_t* status = &static_cast<WsHeader*>(d_ws)->status;
     const int64_t* fk = static_cast<const int64_t*>(probe->cols[fk_col].data);
     const unsigned grid = static_cast<unsigned>(L.ntiles);
-    cudaMemsetAsync(tcnt, 0, 4 * static_cast<size_t>(L.ntiles), st);
-    cudaMemsetAsync(ws + L.scan, 0, scan_scratch_bytes(L.nscan), st);  // before the match: the scan follows it directly
+    cudaMemsetAsync(ws + L.cnt, 0, L.off - L.cnt, st);  // before the match: the scan follows it directly
     const bool has_sel = d_sel != nullptr;
     const auto match = has_sel ? probe_match_kernel<true> : probe_match_kernel<false>;
     int per_sm = 0;

@@ -621,3 +621,48 @@ def test_partition_scatter_kernels_edges(px, P, n):
                 np.testing.assert_array_equal(host(off), woff)
                 for o, w in zip(out, want):
                     np.testing.assert_array_equal(host(o, w.size), w)
+
+
+# Dense block arrays at the edges of their rules: ranges around each replica count (64
+# slots: one per lane, 2048: one), of the shared-memory budget and of the few-rows rule
+# (256 rows per slot); rows around a tile of 4096; keys of every width, one or two; with
+# and without COUNT, a selection, segments off the tiles, and keys outside the statistic.
+@pytest.mark.parametrize("D,n", [(1, 4095), (3, 4097), (64, 20_001), (65, 16_641), (65, 16_640), (1025, 300_001),
+                                 (2049, 70_003), (9000, 200_001), (300_000, 5003)])
+@pytest.mark.parametrize("kt", [np.int32, np.int64, "pair"])
+@pytest.mark.parametrize("form", ["all", "nocount", "seg", "sel"])
+def test_groupby_dense_edges(px, D, n, kt, form):
+    g = pxdata.rng(D + n)
+    code = g.integers(0, D, n)
+    if D > 1:
+        code[::997] = D + 3  # outside the statistic
+    if kt == "pair":
+        keys, kr = [(code // 7 - 2).astype(np.int32), (code % 7).astype(np.int8)], [(-2, (D - 1) // 7 - 2), (0, 6)]
+    else:
+        keys, kr = [(code - 5).astype(kt)], [(-5, D - 6)]
+    a, b = pxdata.random_column(g, n, np.int64), pxdata.random_column(g, n, np.int32)
+    nk = len(keys)
+    ops = [("SUM", nk, None), ("COUNT", None, None), ("SUM_MUL", nk + 1, nk)]
+    if form == "nocount":
+        ops = [o for o in ops if o[0] != "COUNT"]
+    cols = keys + [a, b]
+    naggs = 2 if form == "seg" else len(ops)  # with segments: the SUM + COUNT kernel
+    aggs = [(getattr(px, "PX_" + o), x, y) for o, x, y in ops[:naggs]]
+    oaggs = [(getattr(oracle, o), None if x is None else cols[x], None if y is None else cols[y])
+             for o, x, y in ops[:naggs]]
+    kw, okw, nseg = {}, {}, 1
+    if form == "seg":
+        seg = np.array([0, n // 5, n // 5, n // 2 + 1, n], np.int64)
+        kw, okw, nseg = dict(seg=dev(seg)), dict(seg=seg), 4
+        if kt == np.int64:
+            pytest.skip("64 key bits leave none for segments")
+    if form == "sel":
+        sel = np.flatnonzero(g.random(n) < 0.7).astype(np.int32)
+        kw, okw = dict(sel=dev(sel), nsel=dev(np.array([sel.size], np.int64))), dict(sel=sel)
+    want = oracle.groupby(keys, oaggs, **okw)
+    span = D if kt != "pair" else ((D - 1) // 7 + 1) * 7
+    for mg in {nseg * span + 8, max(1, want["ngroups"])}:  # a dense global result, or claimed groups
+        ws = px.Workspace(256)
+        res = _gb(px, cols, list(range(nk)), aggs, mg, key_range=kr, ws=ws, **kw)
+        assert ws.status() == px.PX_OK
+        assert_groups_equal(res, want, nk, segmented=form == "seg")
