@@ -189,7 +189,7 @@ template <int THREADS, int ITEMS, int NA, bool W8, bool SHARED>
 __device__ void frag_rows(const FragDev& f, int64_t r0, int64_t r1, uint32_t* s_lo, uint32_t* s_hi,
                           uint32_t* s_occ, uint32_t* queue, int32_t* status) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const uint32_t nb = static_cast<uint32_t>(table_buckets(f.t.hdr->nbuild, 1));
+    const uint32_t nb = static_cast<uint32_t>(table_buckets(f.t.hdr->nbuild, 1, f.t.hdr->spread));
     // the group column copied into the table at build time: read with the key
     const bool group_in_table = f.t.hdr->pay_src == f.group && f.t.hdr->pay_w == f.group_w;
     const int naggs = f.naggs;

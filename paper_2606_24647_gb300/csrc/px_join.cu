@@ -3,8 +3,8 @@
 // when segments are given.
 //
 // Table: caller memory with the private layout of px_table.cuh (32-byte buckets
-// of 2 slots: keys, build rows, payload values; segment q owns n_q + 1 buckets, so
-// every segment runs at load factor < 1/2 and the whole table is n + nsegs buckets
+// of 2 slots: keys, build rows, payload values; segment q owns n_q + 1 buckets, or
+// 2 n_q + 1 in a small table, so every segment runs at load factor < 1/2 or < 1/4
 // with no size known before the build). Linear probing over slots starts at the
 // first slot of the key's home bucket: the multiply-shift reduction of the LOWER
 // 32 bits of fmix64(key) (the exchange uses the upper 32) onto the segment's
@@ -20,8 +20,9 @@ namespace {
 
 // ------------------------------------------------------------------ build ----
 
-__global__ void build_init_kernel(TableView t, int32_t S, int32_t unique, const int64_t* __restrict__ d_seg,
-                                  const int64_t* __restrict__ d_n, int64_t ncap, const void* pay, int32_t pay_w) {
+__global__ void build_init_kernel(TableView t, int32_t S, int32_t unique, int32_t spread,
+                                  const int64_t* __restrict__ d_seg, const int64_t* __restrict__ d_n, int64_t ncap,
+                                  const void* pay, int32_t pay_w) {
     allow_dependents();  // the insert may launch; it waits for this grid before touching the table
     const int64_t n = actual_rows(d_n, ncap);
     const int64_t gtid = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
@@ -31,6 +32,7 @@ __global__ void build_init_kernel(TableView t, int32_t S, int32_t unique, const 
         t.hdr->nsegs = S;
         t.hdr->unique = unique;
         t.hdr->nbuild = n;
+        t.hdr->spread = spread;
         t.hdr->pay_src = pay;
         t.hdr->pay_w = pay ? pay_w : 0;
         // Segment offsets clamped to be non-decreasing within [0, n] and to end at
@@ -48,7 +50,7 @@ __global__ void build_init_kernel(TableView t, int32_t S, int32_t unique, const 
     // Every bucket cleared whole with one 32-byte store (keys empty, rows and payload
     // values zero): whole sectors written (clearing the keys alone, 16 bytes per
     // sector, measured 10 us slower at 2M build rows).
-    const int64_t nbk = table_buckets(n, S);
+    const int64_t nbk = table_buckets(n, S, spread);
     longlong4_32a e;
     e.x = kEmpty;
     e.y = kEmpty;
@@ -628,7 +630,10 @@ extern "C" {
 size_t px_join_table_bytes(int64_t nbuild, int32_t nsegs) {
     if (nbuild < 0) nbuild = 0;
     const int32_t S = nsegs > 0 ? nsegs : 1;
-    return 64 + seg_area_bytes(S) + 16 + static_cast<size_t>(table_buckets(nbuild, S)) * sizeof(Bucket);
+    // more rows never need less: a buffer sized for a capacity serves every smaller build
+    const int64_t buckets = std::max({table_buckets(nbuild, S, 0), table_buckets(std::min(nbuild, spread1_rows(S)), S, 1),
+                                      table_buckets(std::min(nbuild, kSpread2), S, 2)});
+    return 64 + seg_area_bytes(S) + 16 + static_cast<size_t>(buckets) * sizeof(Bucket);
 }
 
 size_t px_join_build_ws_bytes(int64_t nbuild) {
@@ -663,7 +668,8 @@ px_status px_join_build(const px_batch* build, int32_t pk_col, const int64_t* d_
     if (table_bytes < px_join_table_bytes(build->nrows, nsegs))
         return fail(PX_ERR_INVALID, "px_join_build: table of %zu bytes, %zu needed", table_bytes,
                     px_join_table_bytes(build->nrows, nsegs));
-    if (!unique && kSlots * table_buckets(build->nrows, nsegs > 0 ? nsegs : 1) + 2 > INT32_MAX)
+    const int32_t spread = table_spread(build->nrows, nsegs > 0 ? nsegs : 1);
+    if (!unique && kSlots * table_buckets(build->nrows, nsegs > 0 ? nsegs : 1, spread) + 2 > INT32_MAX)
         return fail(PX_ERR_UNSUPPORTED, "px_join_build: multi-map tables hold below about 2^30 rows");
     s = check_ws(d_ws, ws_bytes, px_join_build_ws_bytes(build->nrows), "px_join_build");
     if (s != PX_OK) return s;
@@ -671,10 +677,11 @@ px_status px_join_build(const px_batch* build, int32_t pk_col, const int64_t* d_
     const int32_t S = nsegs > 0 ? nsegs : 1;
     const TableView t = table_view(d_table, S);
     const int64_t ncap = build->nrows;
-    const int64_t nwords = table_buckets(ncap, S);  // buckets whose keys to clear
+    const int64_t nwords = table_buckets(ncap, S, spread);  // buckets to clear
     const int threads = 256;
     const unsigned init_blocks = static_cast<unsigned>(std::min<int64_t>(cdiv(nwords, threads), 8192));
-    build_init_kernel<<<init_blocks, threads, 0, st>>>(t, S, unique ? 1 : 0, d_seg, build->d_nrows, ncap, pay, pay_w);
+    build_init_kernel<<<init_blocks, threads, 0, st>>>(t, S, unique ? 1 : 0, spread, d_seg, build->d_nrows,
+                                                                   ncap, pay, pay_w);
     note_launch();
     if ((s = check_launch("px_join_build init")) != PX_OK) return s;
     if (ncap > 0) {

@@ -666,3 +666,32 @@ def test_groupby_dense_edges(px, D, n, kt, form):
         res = _gb(px, cols, list(range(nk)), aggs, mg, key_range=kr, ws=ws, **kw)
         assert ws.status() == px.PX_OK
         assert_groups_equal(res, want, nk, segmented=form == "seg")
+
+
+# Table sizes on both sides of each load factor's line (2^18 and 2^20 build rows, 2^17
+# per segment between 8 and 32 segments): lookups that hit and miss, and a buffer sized
+# for the larger side serving the smaller.
+@pytest.mark.parametrize("nb,nsegs", [(2**18, 0), (2**18 + 1, 0), (2**20, 0), (2**20 + 1, 0), (2**20 + 1, 9),
+                                      (2**21 + 1, 16)])
+def test_join_table_load_factors(px, nb, nsegs):
+    L = px.load()
+    sizes = [L.px_join_table_bytes(n, nsegs) for n in (1, 2**18, 2**18 + 1, 2**20, 2**20 + 1, 2**21, 2**22, 2**22 + 1)]
+    assert sizes == sorted(sizes)
+    g = pxdata.rng(nb)
+    pk = (g.permutation(nb) * 3).astype(np.int64)
+    fk = g.integers(0, 3 * nb, 50_000).astype(np.int64)
+    kw = {}
+    if nsegs:
+        (pk,), boff = oracle.partition([pk], 0, nsegs)
+        (fk,), poff = oracle.partition([fk], 0, nsegs)
+        kw = dict(build_seg=boff, probe_seg=poff)
+    d_fk = dev(fk)
+    ws = px.Workspace(256)
+    table = torch.empty(L.px_join_table_bytes(2**22 + 1, nsegs), dtype=torch.uint8, device="cuda")
+    t = px.px_join_build([dev(pk)], 0, seg=dev(boff) if nsegs else None, table=table, ws=ws)
+    r = px.px_join_probe(t, [d_fk], 0, seg=dev(poff) if nsegs else None, probe_row=True, build_row=True, ws=ws)
+    assert ws.status() == px.PX_OK
+    pr, br, _ = oracle.join(pk, fk, **kw)
+    n = count(r["nout"])
+    np.testing.assert_array_equal(host(r["probe_row"], n), pr)
+    np.testing.assert_array_equal(host(r["build_row"], n), br)
