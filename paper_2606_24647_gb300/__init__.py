@@ -12,6 +12,7 @@ streams (``torch.cuda.current_stream()`` unless one is passed).
 """
 from __future__ import annotations
 
+import array
 import ctypes
 import os
 
@@ -85,6 +86,7 @@ class px_fragments_config(ctypes.Structure):
 
 
 _lib = None
+_calls = None  # the same library with untyped pointer arguments: descriptors as raw addresses
 
 
 def _declare(lib):
@@ -128,9 +130,28 @@ def _declare(lib):
         f.restype = res
 
 
+def _declare_calls(lib):
+    """The operator calls with every pointer a plain address (see _pack)."""
+    P, I32, I64, U64, SZ = ctypes.c_void_p, ctypes.c_int32, ctypes.c_int64, ctypes.c_uint64, ctypes.c_size_t
+    sig = {
+        "px_filter": [P, I64, P, I64, I64, P, P, P, SZ, P],
+        "px_partition_tuned": [P, I32, P, P, I32, U64, P, P, P, P, SZ, P],
+        "px_join_build": [P, I32, P, I32, I32, I32, P, SZ, P, SZ, P],
+        "px_join_probe": [P, P, I32, P, P, P, I32, P, I32, P, P, P, P, P, P, P, SZ, P],
+        "px_groupby_agg_stream": [P, P, I32, P, I32, P, P, P, I32, P, I64, P, P, P, I32, P, SZ, P],
+        "px_groupby_agg": [P, P, I32, P, I32, P, P, P, I32, P, I64, P, P, P, P, SZ, P],
+        "px_gather": [P, P, P, P, P, SZ, P],
+        "px_join_probe_agg": [P, P, I32, P, P, P, I32, P, I64, I64, I64, P, I32, I64, P, P, P, P, SZ, P],
+    }
+    for name, args in sig.items():
+        f = getattr(lib, name)
+        f.argtypes = args
+        f.restype = I32
+
+
 def load(path: str | None = None):
     """Load libpx.so (building it first if its sources are newer). Raises if it is missing."""
-    global _lib
+    global _lib, _calls
     if _lib is None:
         from . import build as _build
         if path is None:
@@ -139,9 +160,10 @@ def load(path: str | None = None):
             path = LIB_PATH
         if not os.path.exists(path):
             raise RuntimeError(f"px CUDA library not found at {path}; run paper_2606_24647_gb300.build.build()")
-        lib = ctypes.CDLL(path)
+        lib, calls = ctypes.CDLL(path), ctypes.CDLL(path)
         _declare(lib)
-        _lib = lib
+        _declare_calls(calls)
+        _lib, _calls = lib, calls
     return _lib
 
 
@@ -184,9 +206,47 @@ def _sel_ptr(sel) -> int | None:
 _keep_alive: list = []
 
 
-def _stream(stream) -> ctypes.c_void_p:
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return ctypes.c_void_p(s.cuda_stream)
+def _stream(stream) -> int:
+    if stream is not None:
+        return stream.cuda_stream
+    # torch.cuda.current_stream().cuda_stream without building a Stream (2.8 us a call)
+    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+
+
+def _words(t: torch.Tensor) -> tuple:
+    """(type, address) of a column, checked like _col."""
+    code = _TYPES.get(t.dtype)
+    if code is None:
+        raise TypeError(f"unsupported column dtype {t.dtype}")
+    if not t.is_cuda or not t.is_contiguous() or t.dim() != 1:
+        raise ValueError("columns must be contiguous 1-D CUDA tensors")
+    return code, t.data_ptr()
+
+
+# Descriptors are packed as 64-bit words (a px_col is {type, reserved = 0 | data}, a
+# px_batch {ncols, reserved = 0 | cols | nrows | d_nrows}, little-endian) in one array
+# per batch, the columns behind the batch: a ctypes structure per column and call cost
+# 40 % of a small call's host time (three calls on 20,000 rows: 111 us, now 63).
+# The address is only used while the array is alive, that is during the call.
+def _pack(cols, nrows: int, d_nrows=None) -> array.array:
+    w = [len(cols), 0, nrows, _ptr(d_nrows) or 0]
+    for c in cols:
+        w += _words(c)
+    a = array.array("Q", w)
+    a[1] = a.buffer_info()[0] + 32
+    return a
+
+
+def _at(a) -> int | None:
+    """Address of a packed array (None: null)."""
+    return None if a is None else a.buffer_info()[0]
+
+
+def _pack_aggs(aggs) -> array.array:
+    w = []
+    for op, a, b in aggs:
+        w += (op, -1 if a is None else a, -1 if b is None else b)
+    return array.array("i", w or (0, 0, 0))
 
 
 def _col(t: torch.Tensor) -> px_col:
@@ -262,9 +322,9 @@ def px_filter(col, lo: int, hi: int, *, d_nrows=None, sel=None, nsel=None, ws=No
     sel = sel if sel is not None else torch.empty(max(n, 1), dtype=torch.int32, device=col.device)
     nsel = nsel if nsel is not None else torch.empty(1, dtype=torch.int64, device=col.device)
     ws = _ws(ws, L.px_filter_ws_bytes(n), stream)
-    c = _col(col)
-    _check(L.px_filter(ctypes.byref(c), n, _ptr(d_nrows), int(lo), int(hi), _ptr(sel), _ptr(nsel),
-                       ws.ptr, ws.nbytes, _stream(stream)), "px_filter")
+    c = array.array("Q", _words(col))
+    _check(_calls.px_filter(_at(c), n, _ptr(d_nrows), int(lo), int(hi), _ptr(sel), _ptr(nsel),
+                            ws.ptr, ws.nbytes, _stream(stream)), "px_filter")
     return sel, nsel
 
 
@@ -276,19 +336,15 @@ def px_partition(cols, key_col: int, nparts: int, seed: int = 0, *, sel=None, ns
     Returns (out_cols, offsets int64[nparts+1])."""
     L = load()
     n = cols[0].numel()
-    inb = _Batch(cols, n, d_nrows)
+    inb = _pack(cols, n, d_nrows)
     out = out if out is not None else [torch.empty(max(n, 1), dtype=c.dtype, device=c.device) for c in cols]
-    outb = _Batch(out, max(n, 1))
+    outb = _pack(out, max(n, 1))
     offsets = offsets if offsets is not None else torch.empty(nparts + 1, dtype=torch.int64, device=cols[0].device)
     ws = _ws(ws, L.px_partition_ws_bytes(n, nparts), stream)
-    if config is None:
-        _check(L.px_partition(inb.ref(), key_col, _sel_ptr(sel), _ptr(nsel), nparts, int(seed) & (2**64 - 1),
-                              outb.ref(), _ptr(offsets), ws.ptr, ws.nbytes, _stream(stream)), "px_partition")
-    else:
-        cfg = px_partition_config(*config)
-        _check(L.px_partition_tuned(inb.ref(), key_col, _sel_ptr(sel), _ptr(nsel), nparts, int(seed) & (2**64 - 1),
-                                    outb.ref(), _ptr(offsets), ctypes.byref(cfg), ws.ptr, ws.nbytes,
-                                    _stream(stream)), "px_partition")
+    cfg = None if config is None else array.array("i", config)
+    _check(_calls.px_partition_tuned(_at(inb), key_col, _sel_ptr(sel), _ptr(nsel), nparts, int(seed) & (2**64 - 1),
+                                     _at(outb), _ptr(offsets), _at(cfg), ws.ptr, ws.nbytes, _stream(stream)),
+           "px_partition")
     return out, offsets
 
 
@@ -304,9 +360,9 @@ def px_join_build(cols, pk_col: int, *, seg=None, unique: bool = True, pay_col=N
     need = L.px_join_table_bytes(n, nsegs)
     table = table if table is not None and table.numel() >= need else torch.empty(
         need, dtype=torch.uint8, device=cols[0].device)
-    b = _Batch(cols, n, d_nrows)
+    b = _pack(cols, n, d_nrows)
     ws = _ws(ws, L.px_join_build_ws_bytes(n), stream)
-    _check(L.px_join_build(b.ref(), pk_col, _ptr(seg), nsegs, 1 if unique else 0, -1 if pay_col is None else pay_col,
+    _check(_calls.px_join_build(_at(b), pk_col, _ptr(seg), nsegs, 1 if unique else 0, -1 if pay_col is None else pay_col,
                            table.data_ptr(), table.numel(), ws.ptr, ws.nbytes, _stream(stream)), "px_join_build")
     return table
 
@@ -327,9 +383,9 @@ def px_join_probe(table, cols, fk_col: int, *, sel=None, nsel=None, seg=None, d_
     if out is None:
         out = [torch.empty(cap, dtype=cols[c].dtype, device=dev) for c in carry] + \
               [torch.empty(cap, dtype=p.dtype, device=dev) for p in pay]
-    pb = _Batch(cols, n, d_nrows)
-    payb = _Batch(pay) if pay else None
-    outb = _Batch(out, cap)
+    pb = _pack(cols, n, d_nrows)
+    payb = _pack(pay, pay[0].numel()) if pay else None
+    outb = _pack(out, cap)
     res = {"cols": out, "nout": torch.empty(1, dtype=torch.int64, device=dev)}
     if probe_row:
         res["probe_row"] = torch.empty(cap, dtype=torch.int32, device=dev)
@@ -337,12 +393,12 @@ def px_join_probe(table, cols, fk_col: int, *, sel=None, nsel=None, seg=None, d_
         res["build_row"] = torch.empty(cap, dtype=torch.int32, device=dev)
     if out_seg:
         res["out_seg"] = torch.empty(max(nsegs, 1) + 1, dtype=torch.int64, device=dev)
-    carr = (ctypes.c_int32 * max(1, len(carry)))(*carry)
+    carr = array.array("i", carry or (0,))
     ws = _ws(ws, L.px_join_probe_ws_bytes(n), stream)
-    _check(L.px_join_probe(table.data_ptr(), pb.ref(), fk_col, _sel_ptr(sel), _ptr(nsel), _ptr(seg), nsegs,
-                           carr, len(carry), payb.ref() if payb else None, outb.ref(),
-                           _ptr(res.get("probe_row")), _ptr(res.get("build_row")), _ptr(res["nout"]),
-                           _ptr(res.get("out_seg")), ws.ptr, ws.nbytes, _stream(stream)), "px_join_probe")
+    _check(_calls.px_join_probe(table.data_ptr(), _at(pb), fk_col, _sel_ptr(sel), _ptr(nsel), _ptr(seg), nsegs,
+                                _at(carr), len(carry), _at(payb), _at(outb),
+                                _ptr(res.get("probe_row")), _ptr(res.get("build_row")), _ptr(res["nout"]),
+                                _ptr(res.get("out_seg")), ws.ptr, ws.nbytes, _stream(stream)), "px_join_probe")
     return res
 
 
@@ -362,28 +418,27 @@ def px_groupby_agg(cols, key_cols, aggs, *, max_groups: int, sel=None, nsel=None
     if out is None:
         out = [torch.empty(max_groups, dtype=cols[k].dtype, device=dev) for k in key_cols] + \
               [torch.empty(max_groups, dtype=torch.int64, device=dev) for _ in aggs]
-    inb = _Batch(cols, n, d_nrows)
-    outb = _Batch(out, max_groups)
-    karr = (ctypes.c_int32 * len(key_cols))(*key_cols)
-    aarr = (px_agg * max(1, len(aggs)))(*[px_agg(op, a if a is not None else -1, b if b is not None else -1)
-                                          for op, a, b in aggs])
+    inb = _pack(cols, n, d_nrows)
+    outb = _pack(out, max_groups)
+    karr = array.array("i", key_cols)
+    aarr = _pack_aggs(aggs)
     res = {"keys": out[:len(key_cols)], "aggs": out[len(key_cols):],
            "ngroups": ngroups if ngroups is not None else torch.empty(1, dtype=torch.int64, device=dev)}
     if nsegs > 0:
         res["seg"] = out_seg if out_seg is not None else torch.empty(max_groups, dtype=torch.int32, device=dev)
     rng = None
     if key_range is not None:
-        rng = px_key_range()
+        rng = array.array("q", [0, 0, 0, 0])  # lo[2], hi[2]
         for k, (lo, hi) in enumerate(key_range):
-            rng.lo[k], rng.hi[k] = int(lo), int(hi)
+            rng[k], rng[2 + k] = int(lo), int(hi)
     ws = _ws(ws, L.px_groupby_ws_bytes(n, max_groups), stream)
-    args = (inb.ref(), karr, len(key_cols), aarr, len(aggs), _sel_ptr(sel), _ptr(nsel), _ptr(seg), nsegs,
-            ctypes.byref(rng) if rng is not None else None, max_groups, outb.ref(), _ptr(res.get("seg")),
-            _ptr(res["ngroups"]))
+    args = (_at(inb), _at(karr), len(key_cols), _at(aarr), len(aggs), _sel_ptr(sel), _ptr(nsel), _ptr(seg), nsegs,
+            _at(rng), max_groups, _at(outb), _ptr(res.get("seg")), _ptr(res["ngroups"]))
     if flags:
-        _check(L.px_groupby_agg_stream(*args, int(flags), ws.ptr, ws.nbytes, _stream(stream)), "px_groupby_agg_stream")
+        _check(_calls.px_groupby_agg_stream(*args, int(flags), ws.ptr, ws.nbytes, _stream(stream)),
+               "px_groupby_agg_stream")
     else:
-        _check(L.px_groupby_agg(*args, ws.ptr, ws.nbytes, _stream(stream)), "px_groupby_agg")
+        _check(_calls.px_groupby_agg(*args, ws.ptr, ws.nbytes, _stream(stream)), "px_groupby_agg")
     return res
 
 
@@ -486,10 +541,10 @@ def px_gather(cols, idx, *, n=None, d_n=None, out=None, ws=None, stream=None):
     dev = idx.device
     if out is None:
         out = [torch.empty(max(cap, 1), dtype=c.dtype, device=dev) for c in cols]
-    inb = _Batch(cols, cols[0].numel(), None)
-    outb = _Batch(out, cap)
+    inb = _pack(cols, cols[0].numel())
+    outb = _pack(out, cap)
     ws = _ws(ws, 256, stream)
-    _check(L.px_gather(inb.ref(), _ptr(idx), _ptr(d_n), outb.ref(), ws.ptr, ws.nbytes, _stream(stream)), "px_gather")
+    _check(_calls.px_gather(_at(inb), _ptr(idx), _ptr(d_n), _at(outb), ws.ptr, ws.nbytes, _stream(stream)), "px_gather")
     return out
 
 
@@ -505,18 +560,17 @@ def px_join_probe_agg(table, cols, fk_col: int, group, group_range, aggs, *, max
     if out is None:
         out = [torch.empty(max_groups, dtype=group.dtype, device=dev)] + \
               [torch.empty(max_groups, dtype=torch.int64, device=dev) for _ in aggs]
-    inb = _Batch(cols, n, d_nrows)
-    outb = _Batch(out, max_groups)
-    aarr = (px_agg * max(1, len(aggs)))(*[px_agg(op, a if a is not None else -1, b if b is not None else -1)
-                                          for op, a, b in aggs])
-    g = _col(group)
+    inb = _pack(cols, n, d_nrows)
+    outb = _pack(out, max_groups)
+    aarr = _pack_aggs(aggs)
+    g = array.array("Q", _words(group))
     res = {"keys": out[:1], "aggs": out[1:],
            "ngroups": ngroups if ngroups is not None else torch.empty(1, dtype=torch.int64, device=dev)}
     if nsegs > 0:
         res["seg"] = out_seg if out_seg is not None else torch.empty(max_groups, dtype=torch.int32, device=dev)
     ws = _ws(ws, L.px_join_probe_agg_ws_bytes(n, max_groups), stream)
-    _check(L.px_join_probe_agg(_ptr(table), inb.ref(), fk_col, _sel_ptr(sel), _ptr(nsel), _ptr(seg), nsegs,
-                               ctypes.byref(g), group.numel(), int(group_range[0]), int(group_range[1]), aarr,
-                               len(aggs), max_groups, outb.ref(), _ptr(res.get("seg")), _ptr(res["ngroups"]),
-                               ws.ptr, ws.nbytes, _stream(stream)), "px_join_probe_agg")
+    _check(_calls.px_join_probe_agg(_ptr(table), _at(inb), fk_col, _sel_ptr(sel), _ptr(nsel), _ptr(seg), nsegs,
+                                    _at(g), group.numel(), int(group_range[0]), int(group_range[1]), _at(aarr),
+                                    len(aggs), max_groups, _at(outb), _ptr(res.get("seg")), _ptr(res["ngroups"]),
+                                    ws.ptr, ws.nbytes, _stream(stream)), "px_join_probe_agg")
     return res

@@ -357,6 +357,14 @@ px_status check_ws(const void* d_ws, size_t ws_bytes, size_t need, const char* w
 
 __host__ __device__ inline int64_t cdiv(int64_t a, int64_t b) { return (a + b - 1) / b; }
 
+// Lets `kernel` use `bytes` of dynamic shared memory; up to 48 KB needs no asking (and
+// no host call).
+template <typename K>
+inline void allow_smem(K kernel, size_t bytes) {
+    if (bytes > 48 * 1024)
+        cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(bytes));
+}
+
 // Streaming multiprocessors of the current device.
 inline int sm_count() {
     int dev = 0, n = 0;

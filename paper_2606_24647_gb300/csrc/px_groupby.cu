@@ -1140,7 +1140,7 @@ px_status launch_sum_count(const Spec& sp, int32_t sum_slot, int32_t cnt_slot, c
     constexpr int ITEMS = 16 / sizeof(KT) > 16 / sizeof(VT) ? 16 / sizeof(KT) : 16 / sizeof(VT);
     auto kernel = groupby_sum_count_kernel<KT, VT, ITEMS>;
     const size_t smem = 12 * static_cast<size_t>(sp.D);
-    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+    allow_smem(kernel, smem);
     // A block flushes its D slots at every segment end: give each at least 4 D rows.
     const int64_t grid = std::max<int64_t>(
         1, std::min<int64_t>(cdiv(ncap, std::max<int64_t>(kThreads * ITEMS, 4 * static_cast<int64_t>(sp.D))),
@@ -1316,7 +1316,7 @@ px_status launch_probe_sum_count(const Spec& sp, int32_t sum_slot, int32_t cnt_s
                                  int32_t* status, cudaStream_t st) {
     auto kernel = groupby_probe_sum_count_kernel<VT>;
     const size_t smem = 12 * static_cast<size_t>(sp.D);
-    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+    allow_smem(kernel, smem);
     const int64_t grid = std::max<int64_t>(
         1, std::min<int64_t>(cdiv(ncap, std::max<int64_t>(kThreads * 2, 4 * static_cast<int64_t>(sp.D))), sm_count()));
     kernel<<<static_cast<unsigned>(grid), kThreads, smem, st>>>(sp, sum_slot, cnt_slot, d_n, ncap, d_seg, g,
@@ -1436,7 +1436,7 @@ px_status launch_mode(const Spec& sp, size_t smem, const int32_t* sel, const int
                       const int64_t* d_seg, const GTable& g, int64_t max_groups, int32_t* out_seg, int32_t* status,
                       cudaStream_t st) {
     auto kernel = groupby_kernel<NA, MODE, PROBE>;
-    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+    allow_smem(kernel, smem);
     int per_sm = 0;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kThreads, smem);
     // A dense block flushes its D slots into the global result at every segment end,
@@ -1468,7 +1468,7 @@ template <int NS, int NK>
 px_status launch_runs(const Spec& sp, size_t smem, const int64_t* d_n, int64_t ncap, const int64_t* d_seg,
                       const GTable& g, int64_t max_groups, int32_t* out_seg, int32_t* status, cudaStream_t st) {
     auto kernel = groupby_runs_kernel<NS, NK>;
-    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+    allow_smem(kernel, smem);
     const int64_t min_rows = std::max<int64_t>(kTile, 4 * static_cast<int64_t>(sp.D));  // see launch_mode
     const int64_t grid = std::max<int64_t>(1, std::min<int64_t>(cdiv(ncap, min_rows), num_sms()));
     kernel<<<static_cast<unsigned>(grid), kThreads, smem, st>>>(sp, d_n, ncap, d_seg, g, max_groups, out_seg, status);
@@ -1482,7 +1482,7 @@ px_status launch_hash(const Spec& sp, const int32_t* sel, const int64_t* d_n, in
     auto kernel = groupby_hash_kernel<NA>;
     const uint32_t C = cache_slots(sp.naggs);
     const size_t smem = static_cast<size_t>(C) * (8 + 8 * static_cast<size_t>(sp.naggs));
-    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+    allow_smem(kernel, smem);
     const int64_t grid = std::min<int64_t>(cdiv(ncap, kHashTile), static_cast<int64_t>(num_sms()) * kHashBlocksPerSm);
     kernel<<<static_cast<unsigned>(grid), kHashThreads, smem, st>>>(sp, sel, d_n, ncap, d_seg, h, C, status);
     note_launch();

@@ -182,6 +182,7 @@ __device__ __forceinline__ int32_t count_matches(const Bucket* segb, uint32_t nb
 }
 
 constexpr int kMatchThreads = 512;
+constexpr int kMatchBlocksPerSm = 3;
 constexpr int kMatchItems = kTile / kMatchThreads;  // positions per thread per tile (same tiles as emit)
 
 // Keys of this thread's positions of the tile whose first position is j0 (kEmpty
@@ -246,7 +247,7 @@ __device__ __forceinline__ int32_t walk_on(const Bucket* segb, uint32_t nb, uint
 // only in warps where some lane needs it. Only positions below the row count are
 // written: the emit reads no other.
 template <bool kSel>
-__global__ void __launch_bounds__(kMatchThreads, 3)
+__global__ void __launch_bounds__(kMatchThreads, kMatchBlocksPerSm)
 probe_match_kernel(TableView t, int32_t S, const int64_t* __restrict__ fk, const int32_t* __restrict__ sel,
                    const int64_t* __restrict__ d_n, int64_t ncap, const int64_t* __restrict__ pseg,
                    int32_t* __restrict__ mrow, int32_t* __restrict__ tile_cnt, int32_t* status, int32_t npay,
@@ -766,9 +767,7 @@ px_status px_join_probe(const void* d_table, const px_batch* probe, int32_t fk_c
     cudaMemsetAsync(ws + L.cnt, 0, L.off - L.cnt, st);  // before the match: the scan follows it directly
     const bool has_sel = d_sel != nullptr;
     const auto match = has_sel ? probe_match_kernel<true> : probe_match_kernel<false>;
-    int per_sm = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, match, kMatchThreads, 0);
-    const unsigned mgrid = static_cast<unsigned>(std::min<int64_t>(L.ntiles, int64_t(sm_count()) * std::max(1, per_sm)));
+    const unsigned mgrid = static_cast<unsigned>(std::min<int64_t>(L.ntiles, int64_t(sm_count()) * kMatchBlocksPerSm));
     match<<<mgrid, kMatchThreads, 0, st>>>(t, S, fk, d_sel, d_n, ncap, d_seg, mrow, tcnt, status, npay,
                                            build_payload ? build_payload->nrows : 0, static_cast<uint32_t>(L.ntiles));
     note_launch();

@@ -649,13 +649,13 @@ px_status launch_partition(const Cols& cols, int32_t key_col, const int32_t* d_s
     auto go = [&](auto bits) {
         if (direct) {
             const auto kern = part_direct_kernel<ITEMS, decltype(bits)::value>;
-            cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+            allow_smem(kern, smem);
             launch_after(kern, dim3(static_cast<unsigned>(ntiles)), dim3(kThreads), smem, st, cols, key_col, d_sel, d_n,
                          ncap, seed, static_cast<uint32_t>(nparts), ps.offs, ntiles, ps.pid);
             return;
         }
         const auto kern = part_scatter_kernel<ITEMS, decltype(bits)::value>;
-        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+        allow_smem(kern, smem);
         launch_after(kern, dim3(static_cast<unsigned>(ntiles)), dim3(kThreads), smem, st, cols, key_col, d_sel, d_n,
                      ncap, seed, static_cast<uint32_t>(nparts), ps.offs, ntiles, stage_bytes, row_bytes, ps.pid,
                      status);
