@@ -287,6 +287,42 @@ __device__ __forceinline__ void load_col(const void* p, int w, const int32_t (&r
     else load_col_t<int8_t>(p, row, v);
 }
 
+// The distinct input columns of the kernels that read rows in runs.
+constexpr int kMaxStream = PX_MAX_KEYS + 6;
+struct Streams {
+    int32_t n;
+    int32_t w[kMaxStream];
+    const void* col[kMaxStream];
+};
+
+Streams input_streams(const Spec& sp) {
+    Streams t = {};
+    const auto add = [&](const void* p, int32_t w) {
+        for (int c = 0; c < t.n; ++c)
+            if (t.col[c] == p) return;
+        if (!p || t.n == kMaxStream) return;
+        t.col[t.n] = p;
+        t.w[t.n++] = w;
+    };
+    for (int k = 0; k < sp.nkeys; ++k) add(sp.key_in[k], sp.key_w[k]);
+    for (int a = 0; a < sp.naggs; ++a) {
+        add(sp.a_in[a], sp.a_w[a]);
+        add(sp.b_in[a], sp.b_w[a]);
+    }
+    return t;
+}
+
+// Starts rows [r0, r1) of every input column on their way to L2: thread c takes column
+// c. Columns are 16-byte aligned; the ends are rounded down to 16 bytes. The next
+// tile's rows, asked for while this one is aggregated: 60M rows of SUM + COUNT 188 ->
+// 178 us, 30M rows of two int8 keys and four aggregates 190 -> 177.
+__device__ __forceinline__ void prefetch_rows(const Streams& t, int64_t r0, int64_t r1) {
+    const int c = threadIdx.x;
+    if (c >= t.n || r0 >= r1) return;
+    const int64_t b0 = r0 * t.w[c] & ~int64_t(15), b1 = r1 * t.w[c] & ~int64_t(15);
+    if (b1 > b0) prefetch_l2(static_cast<const char*>(t.col[c]) + b0, static_cast<uint32_t>(b1 - b0));
+}
+
 // v[i] = column value at row r0 + i, 0 from row ncap on; r0 is a multiple of kItems and
 // the column 16-byte aligned, so a full run is one load of 4 to 16 bytes (two of 16 for
 // 8-byte columns).
@@ -518,7 +554,7 @@ __device__ void aggregate_range_dense(const Spec& sp, const Smem& m, const int32
 // 30M rows 306 -> 189 us; 1000 groups, SUM + SUM_MUL + COUNT 152 -> 109; 2 sums without
 // COUNT, 100 groups 134 -> 104.
 template <int NS, int NK>
-__device__ __forceinline__ void aggregate_runs(const Spec& sp, const Smem& m, int64_t ncap, int64_t a0, int64_t a1,
+__device__ __forceinline__ void aggregate_runs(const Spec& sp, const Streams& in, const Smem& m, int64_t ncap, int64_t a0, int64_t a1,
                                                int q, const GTable& g, int64_t max_groups, int32_t* out_seg,
                                                int32_t* status) {
     const int tid = threadIdx.x, lane = tid & 31;
@@ -528,6 +564,7 @@ __device__ __forceinline__ void aggregate_runs(const Spec& sp, const Smem& m, in
     uint32_t* const cnts = mine + (m.u32 << sh);
     const uint32_t hi_off = m.hi << sh, Dsh = sp.D << sh;
     for (int64_t tb = a0 / kTile * kTile; tb < a1; tb += kTile) {
+        prefetch_rows(in, tb + kTile, tb + 2 * kTile < a1 ? tb + 2 * kTile : a1);
         const int64_t r0 = tb + static_cast<int64_t>(tid) * kItems;
         // the tile's rows in [a0, a1): first .. first + rows
         const uint32_t first = a0 > tb ? static_cast<uint32_t>(a0 - tb) : 0;
@@ -984,7 +1021,7 @@ groupby_kernel(Spec sp, const int32_t* __restrict__ sel, const int64_t* __restri
 // See aggregate_runs.
 template <int NS, int NK>
 __global__ void __launch_bounds__(kThreads, 1)
-groupby_runs_kernel(Spec sp, const int64_t* __restrict__ d_n, int64_t ncap, const int64_t* __restrict__ d_seg, GTable g,
+groupby_runs_kernel(Spec sp, const __grid_constant__ Streams in, const int64_t* __restrict__ d_n, int64_t ncap, const int64_t* __restrict__ d_seg, GTable g,
                     int64_t max_groups, int32_t* __restrict__ out_seg, int32_t* status) {
     extern __shared__ __align__(16) unsigned char smem[];
     const Smem m = dense_smem(sp, smem);
@@ -1005,7 +1042,7 @@ groupby_runs_kernel(Spec sp, const int64_t* __restrict__ d_n, int64_t ncap, cons
                 if (e > pos && e < ce) qend = e;
             }
         }
-        aggregate_runs<NS, NK>(sp, m, ncap, pos, qend, q, g, max_groups, out_seg, status);
+        aggregate_runs<NS, NK>(sp, in, m, ncap, pos, qend, q, g, max_groups, out_seg, status);
         flush_block_table(sp, m, q, g, max_groups, out_seg, status);
         pos = qend;
     }
@@ -1024,7 +1061,7 @@ groupby_runs_kernel(Spec sp, const int64_t* __restrict__ d_n, int64_t ncap, cons
 // Rows whose key lies outside the range take the global hash path.
 template <typename KT, typename VT, int ITEMS>
 __global__ void __launch_bounds__(kThreads, 1)
-groupby_sum_count_kernel(Spec sp, int32_t sum_slot, int32_t cnt_slot, const int64_t* __restrict__ d_n, int64_t ncap,
+groupby_sum_count_kernel(Spec sp, const __grid_constant__ Streams in, int32_t sum_slot, int32_t cnt_slot, const int64_t* __restrict__ d_n, int64_t ncap,
                          const int64_t* __restrict__ d_seg, GTable g, int64_t max_groups, int32_t* __restrict__ out_seg,
                          int32_t* status) {
     constexpr int T = kThreads * ITEMS;
@@ -1059,6 +1096,7 @@ groupby_sum_count_kernel(Spec sp, int32_t sum_slot, int32_t cnt_slot, const int6
         // Tiles aligned to T, rows outside [pos, qend) masked: a tile that straddles
         // a segment boundary is read once for each side.
         for (int64_t tb = pos / T * T; tb < qend; tb += T) {
+            prefetch_rows(in, tb + T, tb + 2 * T < qend ? tb + 2 * T : qend);
             const int64_t r0 = tb + static_cast<int64_t>(tid) * ITEMS;
             KT k[ITEMS];
             VT v[ITEMS];
@@ -1145,8 +1183,8 @@ px_status launch_sum_count(const Spec& sp, int32_t sum_slot, int32_t cnt_slot, c
     const int64_t grid = std::max<int64_t>(
         1, std::min<int64_t>(cdiv(ncap, std::max<int64_t>(kThreads * ITEMS, 4 * static_cast<int64_t>(sp.D))),
                              sm_count()));
-    kernel<<<static_cast<unsigned>(grid), kThreads, smem, st>>>(sp, sum_slot, cnt_slot, d_n, ncap, d_seg, g,
-                                                              max_groups, out_seg, status);
+    kernel<<<static_cast<unsigned>(grid), kThreads, smem, st>>>(sp, input_streams(sp), sum_slot, cnt_slot, d_n, ncap,
+                                                              d_seg, g, max_groups, out_seg, status);
     note_launch();
     return check_launch("px_groupby_agg sum-count");
 }
@@ -1471,7 +1509,8 @@ px_status launch_runs(const Spec& sp, size_t smem, const int64_t* d_n, int64_t n
     allow_smem(kernel, smem);
     const int64_t min_rows = std::max<int64_t>(kTile, 4 * static_cast<int64_t>(sp.D));  // see launch_mode
     const int64_t grid = std::max<int64_t>(1, std::min<int64_t>(cdiv(ncap, min_rows), num_sms()));
-    kernel<<<static_cast<unsigned>(grid), kThreads, smem, st>>>(sp, d_n, ncap, d_seg, g, max_groups, out_seg, status);
+    kernel<<<static_cast<unsigned>(grid), kThreads, smem, st>>>(sp, input_streams(sp), d_n, ncap, d_seg, g, max_groups,
+                                                              out_seg, status);
     note_launch();
     return check_launch("px_groupby_agg runs");
 }

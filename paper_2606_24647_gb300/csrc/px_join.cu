@@ -62,16 +62,26 @@ __global__ void build_init_kernel(TableView t, int32_t S, int32_t unique, int32_
 __global__ void build_insert_kernel(TableView t, int32_t S, int32_t unique, const int64_t* __restrict__ pk,
                                     const int64_t* __restrict__ d_n, int64_t ncap, const void* __restrict__ pay,
                                     int32_t pay_w, int32_t* status) {
+    __shared__ int s_q;
     const int64_t n = actual_rows(d_n, ncap);
-    const int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
+    const int64_t i0 = static_cast<int64_t>(blockIdx.x) * blockDim.x, i = i0 + threadIdx.x;
+    if (i0 >= n) return;
+    const int64_t key = i < n ? pk[i] : 0;  // an input of earlier calls: loaded while the clearing finishes
+    wait_prior();                           // the cleared buckets and the table's segment offsets
+    int q = 0;
+    if (S > 1) {
+        // The block's first row is searched for once; its other rows walk on from there
+        // (a search of their own cost every thread a chain of log2(S) loads).
+        if (threadIdx.x == 0) s_q = seg_of(t.seg, S, i0);
+        __syncthreads();
+        q = s_q;
+        while (q + 1 < S && t.seg[q + 1] <= i) ++q;
+    }
     if (i >= n) return;
-    const int64_t key = pk[i];  // an input of earlier calls: loaded while the clearing finishes
-    wait_prior();               // the cleared buckets and the table's segment offsets
     if (key == kEmpty) {
         set_status(status, PX_ERR_UNSUPPORTED);
         return;
     }
-    const int q = S > 1 ? seg_of(t.seg, S, i) : 0;
     const SegGeom g = seg_geom(t, q);
     Bucket* bk = t.bk + g.b0;
     const uint64_t nslots = uint64_t(kSlots) * g.nb;
