@@ -8,10 +8,10 @@
 //
 // Work items are (fragment, chunk of rows), handed out by a device counter in
 // the order of decreasing fragment size. Every warp of a block walks its own runs of
-// 128 rows of the chunk: it reads the filter column alone (4 consecutive rows per
-// lane, one vector load) and appends the passing rows to a queue in shared memory;
-// whenever the queue holds 32 x ITEMS rows the warp takes them off, every lane with
-// ITEMS rows: their join keys, then their home buckets (one sector: keys, build rows
+// 128 rows of the chunk: it reads the filter column and the join keys (4 consecutive
+// rows per lane, vector loads) and appends the passing rows and their keys to a queue in
+// shared memory; whenever the queue holds 32 x ITEMS rows the warp takes them off, every
+// lane with ITEMS rows: their home buckets (one sector: keys, build rows
 // and, when the dimension was built with its group column copied, the group keys;
 // else the group key is gathered from the build column at the build row) with the
 // aggregate inputs loading beside them; the aggregates go into the fragment's dense
@@ -22,14 +22,15 @@
 // The emit kernel compacts each fragment's occupied slots into its output in
 // key order (single pass, per-fragment bounded look-back).
 //
-// What bounds it: the lookups' dependent round trips (filter, key, bucket, the next
-// bucket for one key in eight) at 32 warps per SM, then DRAM (49 % busy): 512
+// What bounds it: the lookups' dependent round trips (filter and key, bucket, now and
+// then the next bucket) at 32 warps per SM, then DRAM (56 % busy): 512
 // fragments, 388M rows, 28 B per row of columns and 2.4 GB of tables. Measured on
 // that batch: every row looked up in place 12.8 ms; passing rows queued and looked up
 // by full warps 6.0 ms; the next run's columns prefetched into L2, the items' walks
-// merged and small block arrays 3.8 ms (3.1 TB/s). Blocks of 512 threads with 2 rows
-// in flight per thread (two per SM, 64 registers): 3.8 ms; 256 x 2 4.0 ms, 512 x 4
-// (one per SM, 128 registers) 4.3 ms.
+// merged and small block arrays 3.8 ms; spread tables, items of 32768 rows and the keys
+// read beside the filter 3.5 ms (3.4 TB/s). Blocks of 512 threads with 2 rows in flight
+// per thread (two per SM, 64 registers): 3.5 ms; 256 x 2 3.9 ms, 512 x 4 (one per SM, 128
+// registers) 3.8 ms.
 #include <algorithm>
 #include <type_traits>
 #include <vector>
@@ -181,14 +182,14 @@ __device__ __forceinline__ uint32_t filter_rows(const T* col, int64_t lo, int64_
 // Rows [r0, r1) of fragment f (r0 a multiple of kFilterRows). SHARED: accumulate
 // into the block arrays lo/hi ([naggs][D][replicas] each) and occupancy bits; else
 // reduce into the global arrays. `queue`: this warp's kQueue<ITEMS> entries.
-// Only rows that pass the filter touch the key, value and table memory, and every
+// Only rows that pass the filter touch the value and table memory, and every
 // lane of a lookup holds one: with the lookups predicated in place a filter that
 // keeps 30 % of the rows left two lanes of three idle through them (ncu: 19.5
 // threads per instruction).
 // W8: every aggregated column of the batch is 8 bytes wide (no width switches).
 template <int THREADS, int ITEMS, int NA, bool W8, bool SHARED>
 __device__ void frag_rows(const FragDev& f, int64_t r0, int64_t r1, uint32_t* s_lo, uint32_t* s_hi,
-                          uint32_t* s_occ, uint32_t* queue, int32_t* status) {
+                          uint32_t* s_occ, int64_t* queue_key, uint32_t* queue, int32_t* status) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t nb = static_cast<uint32_t>(table_buckets(f.t.hdr->nbuild, 1, f.t.hdr->spread));
     // the group column copied into the table at build time: read with the key
@@ -208,11 +209,10 @@ __device__ void frag_rows(const FragDev& f, int64_t r0, int64_t r1, uint32_t* s_
         for (int i = 0; i < ITEMS; ++i) {
             const uint32_t e = 32 * i + lane;
             row[i] = e < n ? queue[held - n + e] : kNone;
+            key[i] = e < n ? queue_key[held - n + e] : kEmpty;
         }
         __syncwarp();  // the entries are read: the next append may overwrite them
         held -= n;
-#pragma unroll
-        for (int i = 0; i < ITEMS; ++i) key[i] = row[i] != kNone ? f.key[r0 + row[i]] : kEmpty;
 #pragma unroll
         for (int i = 0; i < ITEMS; ++i) {
             hb[i] = home_bucket(static_cast<uint64_t>(key[i]), nb);
@@ -348,7 +348,21 @@ __device__ void frag_rows(const FragDev& f, int64_t r0, int64_t r1, uint32_t* s_
                 const int64_t bytes = ((r1 - nt < kWarpRows ? r1 - nt : kWarpRows) * w) & ~int64_t(15);
                 if (bytes) prefetch_l2(static_cast<const char*>(f.stream[lane]) + nt * w, static_cast<uint32_t>(bytes));
             }
+            // The keys are read beside the filter column (their sectors are needed for one
+            // passing row in four anyway), so a lookup waits for its bucket alone.
             const int64_t r = tb + kFilterRows * lane;
+            int64_t k[kFilterRows];
+            if (r + kFilterRows <= r1) {
+#pragma unroll
+                for (int j = 0; j < kFilterRows; j += 2) {
+                    const longlong2 x = *reinterpret_cast<const longlong2*>(f.key + r + j);
+                    k[j] = x.x;
+                    k[j + 1] = x.y;
+                }
+            } else {
+#pragma unroll
+                for (int j = 0; j < kFilterRows; ++j) k[j] = r + j < r1 ? f.key[r + j] : kEmpty;
+            }
             uint32_t ok;
             if (!f.filter) {
                 ok = r + kFilterRows <= r1 ? (1u << kFilterRows) - 1 : (r < r1 ? (1u << (r1 - r)) - 1 : 0);
@@ -364,7 +378,10 @@ __device__ void frag_rows(const FragDev& f, int64_t r0, int64_t r1, uint32_t* s_
             for (int j = 0; j < kFilterRows; ++j) {
                 const bool p = (ok >> j) & 1u;
                 const uint32_t m = __ballot_sync(FULL, p);
-                if (p) queue[held + __popc(m & lt)] = rel + j;
+                if (p) {
+                    queue[held + __popc(m & lt)] = rel + j;
+                    queue_key[held + __popc(m & lt)] = k[j];
+                }
                 held += __popc(m);
             }
             __syncwarp();
@@ -387,7 +404,9 @@ frag_kernel(const PlanHeader* __restrict__ ph, const int64_t* __restrict__ item_
     // reductions' memory clobbers would otherwise reload its fields from global
     // memory after every update.
     __shared__ __align__(16) FragDev s_f;
+    __shared__ int64_t s_queue_key[THREADS / 32][kQueue<ITEMS>];
     __shared__ uint32_t s_queue[THREADS / 32][kQueue<ITEMS>];
+    int64_t* queue_key = s_queue_key[threadIdx.x >> 5];
     uint32_t* queue = s_queue[threadIdx.x >> 5];
     const int n = ph->nfrags;
     const int64_t nitems = ph->nitems;
@@ -416,7 +435,7 @@ frag_kernel(const PlanHeader* __restrict__ ph, const int64_t* __restrict__ item_
         const int64_t r0 = (item - item_start[p]) * f.chunk;
         const int64_t r1 = r0 + f.chunk < f.nrows ? r0 + f.chunk : f.nrows;
         if (!f.shared) {
-            frag_rows<THREADS, ITEMS, NA, W8, false>(f, r0, r1, nullptr, nullptr, nullptr, queue, status);
+            frag_rows<THREADS, ITEMS, NA, W8, false>(f, r0, r1, nullptr, nullptr, nullptr, queue_key, queue, status);
             continue;
         }
         const uint32_t D = f.D;
@@ -429,7 +448,7 @@ frag_kernel(const PlanHeader* __restrict__ ph, const int64_t* __restrict__ item_
         const uint32_t words = 2 * slots + (f.count_agg < 0 ? (D + 31) / 32 : 0);
         for (uint32_t w = threadIdx.x; w < words; w += THREADS) s_lo[w] = 0;
         __syncthreads();
-        frag_rows<THREADS, ITEMS, NA, W8, true>(f, r0, r1, s_lo, s_hi, s_occ, queue, status);
+        frag_rows<THREADS, ITEMS, NA, W8, true>(f, r0, r1, s_lo, s_hi, s_occ, queue_key, queue, status);
         __syncthreads();
         const uint32_t reps = 1u << rs;
         for (uint32_t o = threadIdx.x; o < naggs * D; o += THREADS) {

@@ -74,7 +74,8 @@ template <int ITEMS>
 __global__ void __launch_bounds__(kThreads)
 part_hist_kernel(const int64_t* __restrict__ key, const int32_t* __restrict__ sel,
                  const int64_t* __restrict__ d_nsel, int64_t ncap, uint64_t seed, uint32_t nparts,
-                 int32_t* __restrict__ cnt, int64_t ntiles, uint8_t* __restrict__ pid_out) {
+                 int32_t* __restrict__ cnt, int64_t ntiles, uint8_t* __restrict__ pid_out,
+                 uint64_t* __restrict__ scan_words, int64_t nscan_words) {
     constexpr int T = kThreads * ITEMS;
     extern __shared__ int32_t s_hist[];  // [kWarps][nparts]
     allow_dependents();  // the scan may launch now; it waits for this grid's counts
@@ -124,6 +125,11 @@ part_hist_kernel(const int64_t* __restrict__ key, const int32_t* __restrict__ se
         for (int w = 0; w < kWarps; ++w) c += s_hist[w * nparts + q];
         cnt[static_cast<int64_t>(q) * ntiles + blockIdx.x] = c;
     }
+    // The scan's counter and look-back words, cleared here for the launch that waits for
+    // this grid (a memset between the calls cost a launch of its own).
+    for (int64_t w = static_cast<int64_t>(blockIdx.x) * kThreads + tid; w < nscan_words;
+         w += static_cast<int64_t>(gridDim.x) * kThreads)
+        scan_words[w] = 0;
 }
 
 // Exclusive scan of cnt[0..total) (partition-major) into offs; offsets[q] is the
@@ -621,9 +627,9 @@ px_status launch_partition(const Cols& cols, int32_t key_col, const int32_t* d_s
                            int32_t* status, cudaStream_t st) {
     px_status s;
     const int64_t* key = static_cast<const int64_t*>(cols.in[key_col]);
-    cudaMemsetAsync(ps.scan, 0, ps.scan_bytes, st);  // before the histogram: the scan launches right after it
     part_hist_kernel<ITEMS><<<static_cast<unsigned>(ntiles), kThreads, kWarps * nparts * sizeof(int32_t), st>>>(
-        key, d_sel, d_n, ncap, seed, static_cast<uint32_t>(nparts), ps.cnt, ntiles, ps.pid);
+        key, d_sel, d_n, ncap, seed, static_cast<uint32_t>(nparts), ps.cnt, ntiles, ps.pid,
+        static_cast<uint64_t*>(ps.scan), static_cast<int64_t>(ps.scan_bytes / 8));
     note_launch();
     if ((s = check_launch("px_partition hist")) != PX_OK) return s;
 
