@@ -390,8 +390,8 @@ typedef struct {
 /* Launch configuration of px_fragments_run (NULL: library defaults). threads per
  * block (256 or 512), rows each thread looks up at a time (items: 2 or 4), rows per
  * work item (a multiple of threads * items, or 0: chosen from the batch's total rows
- * so that the persistent grid gets about four items per block, within [4 rows per
- * thread, 65536]; fragments whose dense accumulators live in shared memory take at
+ * so that the persistent grid gets one item per block of a small batch and about four
+ * of a large one, within [4 rows per thread, 32768]; fragments whose dense accumulators live in shared memory take at
  * least 4 group slots' worth of rows per item), and resident blocks per SM of the
  * persistent grid (1..8; capped by what fits). A project autotuner picks these per
  * GPU; every configuration gives the same results. */
