@@ -242,6 +242,11 @@ def _at(a) -> int | None:
     return None if a is None else a.buffer_info()[0]
 
 
+def _i64(v) -> int:
+    """v as a 64-bit two's complement value (as a ctypes field takes it)."""
+    return ((int(v) + 2**63) & (2**64 - 1)) - 2**63
+
+
 def _pack_aggs(aggs) -> array.array:
     w = []
     for op, a, b in aggs:
@@ -341,9 +346,10 @@ def px_partition(cols, key_col: int, nparts: int, seed: int = 0, *, sel=None, ns
     outb = _pack(out, max(n, 1))
     offsets = offsets if offsets is not None else torch.empty(nparts + 1, dtype=torch.int64, device=cols[0].device)
     ws = _ws(ws, L.px_partition_ws_bytes(n, nparts), stream)
-    cfg = None if config is None else array.array("i", config)
+    cfg = None if config is None else px_partition_config(*config)
     _check(_calls.px_partition_tuned(_at(inb), key_col, _sel_ptr(sel), _ptr(nsel), nparts, int(seed) & (2**64 - 1),
-                                     _at(outb), _ptr(offsets), _at(cfg), ws.ptr, ws.nbytes, _stream(stream)),
+                                     _at(outb), _ptr(offsets),
+                                     None if cfg is None else ctypes.addressof(cfg), ws.ptr, ws.nbytes, _stream(stream)),
            "px_partition")
     return out, offsets
 
@@ -430,7 +436,7 @@ def px_groupby_agg(cols, key_cols, aggs, *, max_groups: int, sel=None, nsel=None
     if key_range is not None:
         rng = array.array("q", [0, 0, 0, 0])  # lo[2], hi[2]
         for k, (lo, hi) in enumerate(key_range):
-            rng[k], rng[2 + k] = int(lo), int(hi)
+            rng[k], rng[2 + k] = _i64(lo), _i64(hi)
     ws = _ws(ws, L.px_groupby_ws_bytes(n, max_groups), stream)
     args = (_at(inb), _at(karr), len(key_cols), _at(aarr), len(aggs), _sel_ptr(sel), _ptr(nsel), _ptr(seg), nsegs,
             _at(rng), max_groups, _at(outb), _ptr(res.get("seg")), _ptr(res["ngroups"]))

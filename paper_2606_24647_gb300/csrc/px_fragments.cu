@@ -827,8 +827,12 @@ px_status px_fragments_run(const px_fragment* frags, int32_t nfrags, const px_fr
         else s = c.items == 2 ? go(t512, i2) : go(t512, i4);
         if (s != PX_OK) return s;
     }
-    launch_after(frag_emit_kernel, dim3(static_cast<unsigned>(emits)), dim3(kEmitThreads), 0, st, d_ph, d_emits, d_fd,
-                 counters + 1, status);
+    // launch_after only behind a kernel: with no rows the work before is the plan's copy
+    const dim3 grid(static_cast<unsigned>(emits));
+    if (items > 0)
+        launch_after(frag_emit_kernel, grid, dim3(kEmitThreads), 0, st, d_ph, d_emits, d_fd, counters + 1, status);
+    else
+        frag_emit_kernel<<<grid, kEmitThreads, 0, st>>>(d_ph, d_emits, d_fd, counters + 1, status);
     note_launch();
     return check_launch("px_fragments_run emit");
 }

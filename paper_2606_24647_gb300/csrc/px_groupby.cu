@@ -1556,7 +1556,7 @@ WsLayout ws_layout(int64_t max_groups) {
     L.key = L.dg_acc + align_up((8 * PX_MAX_AGGS + 1) * M, 256);
     L.gidx = L.key + align_up(8 * G, 256);
     L.total = std::max(L.gidx + align_up(4 * G, 256),
-                       kWsScratch + kEmittedBytes + htable_bytes(static_cast<uint32_t>(G), PX_MAX_AGGS));
+                       kWsScratch + kEmittedBytes + 32 + htable_bytes(static_cast<uint32_t>(G), PX_MAX_AGGS));
     return L;
 }
 
@@ -1730,12 +1730,13 @@ static px_status groupby_impl(const px_batch* in, const int32_t* key_cols, int32
         char* base = static_cast<char*>(d_ws) + kWsScratch;
         HTable h;
         h.emitted = reinterpret_cast<unsigned long long*>(base);
-        h.key = reinterpret_cast<unsigned long long*>(base + kEmittedBytes);
-        h.acc = reinterpret_cast<unsigned long long*>(base + kEmittedBytes +
-                                                      align_up(8 * (static_cast<size_t>(slots) + 1), 256));
+        // a bucket is one 32-byte load; the caller's workspace is only 16-byte aligned
+        char* keys = reinterpret_cast<char*>(align_up(reinterpret_cast<uintptr_t>(base) + kEmittedBytes, 32));
+        h.key = reinterpret_cast<unsigned long long*>(keys);
+        h.acc = reinterpret_cast<unsigned long long*>(keys + align_up(8 * (static_cast<size_t>(slots) + 1), 256));
         h.slots = slots;
         h.shift = acc_shift(naggs);
-        if (!accumulate) cudaMemsetAsync(base, 0, kEmittedBytes + htable_bytes(slots, naggs), st);
+        if (!accumulate) cudaMemsetAsync(base, 0, kEmittedBytes + 32 + htable_bytes(slots, naggs), st);
         if (ncap > 0) {
             const int64_t* d_n = d_sel ? d_nsel : in->d_nrows;
             const auto go = [&](auto launch) { return launch(sp, d_sel, d_n, ncap, d_seg, h, status, st); };
@@ -1749,8 +1750,13 @@ static px_status groupby_impl(const px_batch* in, const int32_t* key_cols, int32
             }
             if (s != PX_OK) return s;
         }
-        launch_after(hash_emit_kernel, dim3(static_cast<unsigned>(cdiv(static_cast<int64_t>(slots) + 1, kEmitTile))),
-                     dim3(kEmitThreads), 0, st, sp, h, max_groups, d_out_seg, d_ngroups, status);
+        // (launch_after only behind a kernel: with no rows the work before is a memset)
+        const dim3 grid(static_cast<unsigned>(cdiv(static_cast<int64_t>(slots) + 1, kEmitTile)));
+        if (ncap > 0)
+            launch_after(hash_emit_kernel, grid, dim3(kEmitThreads), 0, st, sp, h, max_groups, d_out_seg, d_ngroups,
+                         status);
+        else
+            hash_emit_kernel<<<grid, kEmitThreads, 0, st>>>(sp, h, max_groups, d_out_seg, d_ngroups, status);
         note_launch();
         return check_launch("px_groupby_agg hash emit");
     }
@@ -1841,8 +1847,13 @@ static px_status groupby_impl(const px_batch* in, const int32_t* key_cols, int32
     }
     if (sp.dglobal) {
         const int64_t ntiles = cdiv(static_cast<int64_t>(sp.E), kEmitTile);
-        launch_after(dense_emit_kernel, dim3(static_cast<unsigned>(ntiles)), dim3(kEmitThreads), 0, st, sp, g.ngroups,
-                     max_groups, d_out_seg, d_ngroups, scan_scratch(ws + L.emit_scan), status, ntiles);
+        const dim3 grid(static_cast<unsigned>(ntiles));
+        if (ncap > 0)  // as above
+            launch_after(dense_emit_kernel, grid, dim3(kEmitThreads), 0, st, sp, g.ngroups, max_groups, d_out_seg,
+                         d_ngroups, scan_scratch(ws + L.emit_scan), status, ntiles);
+        else
+            dense_emit_kernel<<<grid, kEmitThreads, 0, st>>>(sp, g.ngroups, max_groups, d_out_seg, d_ngroups,
+                                                             scan_scratch(ws + L.emit_scan), status, ntiles);
         note_launch();
         return check_launch("px_groupby_agg emit");
     }

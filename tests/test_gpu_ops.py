@@ -695,3 +695,70 @@ def test_join_table_load_factors(px, nb, nsegs):
     n = count(r["nout"])
     np.testing.assert_array_equal(host(r["probe_row"], n), pr)
     np.testing.assert_array_equal(host(r["build_row"], n), br)
+
+
+class _OffsetWorkspace:
+    """A workspace at a 16-byte (not 32-byte) address, as the C ABI allows."""
+
+    def __init__(self, px):
+        self.px, self.buf = px, torch.zeros(64, dtype=torch.uint8, device="cuda")
+
+    def ensure(self, nbytes, stream=None):
+        if self.buf.numel() < nbytes + 16:
+            self.buf = torch.zeros(nbytes + 16, dtype=torch.uint8, device="cuda")
+        return self
+
+    ptr = property(lambda self: self.buf.data_ptr() + 16)
+    nbytes = property(lambda self: self.buf.numel() - 16)
+
+    def status(self):
+        return int(self.px.load().px_stream_status(None, self.ptr))
+
+
+def test_operators_with_a_workspace_at_a_16_byte_offset(px):
+    g = pxdata.rng(1234)
+    n = 30_001
+    k, a = pxdata.random_column(g, n, np.int64, 0, 5000), pxdata.random_column(g, n, np.int64)
+    ws = _OffsetWorkspace(px).ensure(256)
+    for kr in (None, [(0, 5000)]):
+        want = oracle.groupby([k], [(oracle.SUM, a, None), (oracle.COUNT, None, None)])
+        res = _gb(px, [k, a], [0], [(px.PX_SUM, 1, None), (px.PX_COUNT, None, None)], 5001, key_range=kr, ws=ws)
+        assert ws.status() == px.PX_OK
+        assert_groups_equal(res, want, 1)
+    sel, nsel = px.px_filter(dev(k), 100, 3000, ws=ws)
+    np.testing.assert_array_equal(host(sel, count(nsel)), oracle.filter(k, 100, 3000))
+    for P in (8, 300):
+        out, off = px.px_partition([dev(k), dev(a)], 0, P, ws=ws)
+        want, woff = oracle.partition([k, a], 0, P)
+        np.testing.assert_array_equal(host(off), woff)
+        np.testing.assert_array_equal(host(out[1], n), want[1])
+    pk = g.permutation(5001).astype(np.int64)
+    t = px.px_join_build([dev(pk)], 0, ws=ws)
+    r = px.px_join_probe(t, [dev(k)], 0, build_row=True, ws=ws)
+    np.testing.assert_array_equal(host(r["build_row"], count(r["nout"])), oracle.join(pk, k)[1])
+    assert ws.status() == px.PX_OK
+
+
+def test_groupby_without_rows_in_a_cuda_graph(px):
+    # no kernel before the emit: the group count must come out zero on every replay
+    keys, vals = dev(np.zeros(0, np.int64)), dev(np.zeros(0, np.int64))
+    for kr in (None, [(0, 9)]):
+        ws = px.Workspace(1 << 16)
+        out = [torch.zeros(16, dtype=torch.int64, device="cuda") for _ in range(2)]
+        ng = torch.zeros(1, dtype=torch.int64, device="cuda")
+
+        def call():
+            px.px_groupby_agg([keys, vals], [0], [(px.PX_SUM, 1, None)], max_groups=16, key_range=kr, out=out,
+                              ngroups=ng, ws=ws)
+        side = torch.cuda.Stream()
+        side.wait_stream(torch.cuda.current_stream())
+        with torch.cuda.stream(side):
+            call()
+        torch.cuda.current_stream().wait_stream(side)
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph):
+            call()
+        for _ in range(2):
+            ng.fill_(-1)
+            graph.replay()
+            assert count(ng) == 0
