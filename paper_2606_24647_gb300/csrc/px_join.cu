@@ -62,7 +62,7 @@ __global__ void build_init_kernel(TableView t, int32_t S, int32_t unique, int32_
 __global__ void build_insert_kernel(TableView t, int32_t S, int32_t unique, const int64_t* __restrict__ pk,
                                     const int64_t* __restrict__ d_n, int64_t ncap, const void* __restrict__ pay,
                                     int32_t pay_w, int32_t* status) {
-    __shared__ int s_q;
+    __shared__ int s_q[2];
     const int64_t n = actual_rows(d_n, ncap);
     const int64_t i0 = static_cast<int64_t>(blockIdx.x) * blockDim.x, i = i0 + threadIdx.x;
     if (i0 >= n) return;
@@ -70,12 +70,16 @@ __global__ void build_insert_kernel(TableView t, int32_t S, int32_t unique, cons
     wait_prior();                           // the cleared buckets and the table's segment offsets
     int q = 0;
     if (S > 1) {
-        // The block's first row is searched for once; its other rows walk on from there
-        // (a search of their own cost every thread a chain of log2(S) loads).
-        if (threadIdx.x == 0) s_q = seg_of(t.seg, S, i0);
+        // The block's first and last rows are searched for once; where they share a segment
+        // (nearly always) its other rows need no search, else they search between the two
+        // (a search of their own over all segments cost every thread a chain of log2(S)
+        // loads).
+        if (threadIdx.x < 2) {
+            const int64_t end = i0 + blockDim.x < n ? i0 + blockDim.x : n;
+            s_q[threadIdx.x] = seg_of(t.seg, S, threadIdx.x == 0 ? i0 : end - 1);
+        }
         __syncthreads();
-        q = s_q;
-        while (q + 1 < S && t.seg[q + 1] <= i) ++q;
+        q = s_q[0] + seg_of(t.seg + s_q[0], s_q[1] - s_q[0] + 1, i);
     }
     if (i >= n) return;
     if (key == kEmpty) {

@@ -697,6 +697,25 @@ def test_join_table_load_factors(px, nb, nsegs):
     np.testing.assert_array_equal(host(r["build_row"], n), br)
 
 
+# Build blocks of 256 rows that lie in one segment, in a few and in very many (most of
+# them empty), and a last block that is not full.
+@pytest.mark.parametrize("nb,nsegs", [(1, 4096), (255, 4096), (256, 2), (700, 4096), (5000, 300), (60_001, 7)])
+def test_join_build_segments_within_a_block(px, nb, nsegs):
+    g = pxdata.rng(nb + nsegs)
+    pk = (g.permutation(nb) * 3).astype(np.int64)
+    fk = g.integers(0, 3 * nb, 9_000).astype(np.int64)
+    (pk,), boff = oracle.partition([pk], 0, nsegs)
+    (fk,), poff = oracle.partition([fk], 0, nsegs)
+    ws = px.Workspace(256)
+    t = px.px_join_build([dev(pk)], 0, seg=dev(boff), ws=ws)
+    r = px.px_join_probe(t, [dev(fk)], 0, seg=dev(poff), probe_row=True, build_row=True, ws=ws)
+    assert ws.status() == px.PX_OK
+    pr, br, _ = oracle.join(pk, fk, build_seg=boff, probe_seg=poff)
+    n = count(r["nout"])
+    np.testing.assert_array_equal(host(r["probe_row"], n), pr)
+    np.testing.assert_array_equal(host(r["build_row"], n), br)
+
+
 class _OffsetWorkspace:
     """A workspace at a 16-byte (not 32-byte) address, as the C ABI allows."""
 
