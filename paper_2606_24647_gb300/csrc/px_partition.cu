@@ -103,6 +103,25 @@ part_hist_kernel(const int64_t* __restrict__ key, const int32_t* __restrict__ se
             else if (ITEMS == 4) *reinterpret_cast<uint32_t*>(o) = static_cast<uint32_t>(w);
             else *reinterpret_cast<uint16_t*>(o) = static_cast<uint16_t>(w);
         }
+    } else if (sel && tbase + T <= n) {
+        // A full tile of a selection: all of a thread's row numbers in flight together,
+        // then all of its keys. Row by row, each key waited for its own row number: 29.4M of
+        // 30M rows into 64 partitions 106 us, now 71 (12 bytes read and 1 written a row: 5.4
+        // TB/s).
+        const int32_t* sj = sel + tbase + local_pos<ITEMS>(warp, 0, lane);
+        int32_t row[ITEMS];
+#pragma unroll
+        for (int i = 0; i < ITEMS; ++i) row[i] = sj[32 * i];
+        int64_t k[ITEMS];
+#pragma unroll
+        for (int i = 0; i < ITEMS; ++i) k[i] = key[row[i]];
+#pragma unroll
+        for (int i = 0; i < ITEMS; ++i) p[i] = part_of(k[i], seed, nparts);
+        if (pid_out) {
+            uint8_t* o = pid_out + tbase + local_pos<ITEMS>(warp, 0, lane);
+#pragma unroll
+            for (int i = 0; i < ITEMS; ++i) o[32 * i] = static_cast<uint8_t>(p[i]);
+        }
     } else {
 #pragma unroll
         for (int i = 0; i < ITEMS; ++i) {
