@@ -357,11 +357,12 @@ px_status check_ws(const void* d_ws, size_t ws_bytes, size_t need, const char* w
 
 __host__ __device__ inline int64_t cdiv(int64_t a, int64_t b) { return (a + b - 1) / b; }
 
-// Lets `kernel` use `bytes` of dynamic shared memory; up to 48 KB needs no asking (and
-// no host call).
+// Lets `kernel` use `bytes` of dynamic shared memory beside at most kStaticSmem of static
+// shared memory; up to 48 KB of the two together needs no asking (and no host call).
+constexpr size_t kStaticSmem = 1024;
 template <typename K>
 inline void allow_smem(K kernel, size_t bytes) {
-    if (bytes > 48 * 1024)
+    if (bytes + kStaticSmem > 48 * 1024)
         cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(bytes));
 }
 

@@ -402,12 +402,11 @@ part_scatter_kernel(Cols cols, int32_t key_col, const int32_t* __restrict__ sel,
     void* sorted = smem + stage_bytes;                                             // T x 8 B
     int32_t* s_dest = reinterpret_cast<int32_t*>(smem + stage_bytes + T * 8);     // T
     uint64_t* bar = reinterpret_cast<uint64_t*>(smem + stage_bytes + T * 12);     // 16 B
-    int32_t* s_delta = reinterpret_cast<int32_t*>(smem + stage_bytes + T * 12 + 16);  // np1p
+    int32_t* s_part = reinterpret_cast<int32_t*>(smem + stage_bytes + T * 12 + 16);  // kWarps (rank_tile's)
+    int32_t* s_delta = s_part + kWarps;                                            // np1p
     int32_t* s_whist = s_delta + np1p;                                             // kWarps x np1
     // partition ids from the histogram pass (T bytes), when it wrote them
-    uint8_t* s_pid = smem + ((stage_bytes + T * 12 + 16 + (np1p + kWarps * np1) * 4 + 15) & ~15u);
-
-    __shared__ int32_t s_part[kWarps];  // rank_tile's
+    uint8_t* s_pid = smem + ((stage_bytes + T * 12 + 16 + (kWarps + np1p + kWarps * np1) * 4 + 15) & ~15u);
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int64_t tile = blockIdx.x;
@@ -542,9 +541,9 @@ part_direct_kernel(Cols cols, int32_t key_col, const int32_t* __restrict__ sel, 
     extern __shared__ __align__(16) unsigned char smem[];
     int32_t* s_dest = reinterpret_cast<int32_t*>(smem + T * 8);  // after the buffer of T 8-byte values
     const int np1 = static_cast<int>(nparts) + 1;
-    int32_t* s_delta = s_dest + T;
+    int32_t* s_part = s_dest + T;  // kWarps (rank_tile's)
+    int32_t* s_delta = s_part + kWarps;
     int32_t* s_whist = s_delta + np1;
-    __shared__ int32_t s_part[kWarps];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int64_t tile = blockIdx.x;
     const int64_t n = actual_rows(d_nsel, ncap);
@@ -603,16 +602,19 @@ part_direct_kernel(Cols cols, int32_t key_col, const int32_t* __restrict__ sel, 
 
 int id_bits(int32_t nparts) { return nparts <= 1 ? 0 : 32 - __builtin_clz(static_cast<unsigned>(nparts - 1)); }
 
+// All of the two scatters' shared memory is dynamic: the limits that a launch is held to
+// (48 KB unless the kernel was allowed more, the SM's share per block) are on the sum of
+// dynamic and static bytes.
 size_t scatter_smem_bytes(int items, uint32_t stage_bytes, int32_t nparts) {
     const size_t T = static_cast<size_t>(kThreads) * items;
     const size_t np1 = static_cast<size_t>(nparts) + 1;
     const size_t np1p = (np1 + 3) & ~static_cast<size_t>(3);
-    return align_up(stage_bytes + T * 12 + 16 + np1p * 4 + kWarps * np1 * 4, size_t(16)) + T;  // + ids
+    return align_up(stage_bytes + T * 12 + 16 + (kWarps + np1p + kWarps * np1) * 4, size_t(16)) + T;  // + ids
 }
 
 size_t direct_smem_bytes(int items, int32_t nparts) {
     const size_t np1 = static_cast<size_t>(nparts) + 1;
-    return static_cast<size_t>(kThreads) * items * 12 + np1 * 4 + kWarps * np1 * 4;
+    return static_cast<size_t>(kThreads) * items * 12 + (kWarps + np1 + kWarps * np1) * 4;
 }
 
 // Workspace: count matrix, offset matrix (partition-major, P x tiles int32) and the
