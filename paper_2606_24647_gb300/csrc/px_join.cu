@@ -65,9 +65,11 @@ __global__ void build_insert_kernel(TableView t, int32_t S, int32_t unique, cons
     __shared__ int s_q[2];
     const int64_t n = actual_rows(d_n, ncap);
     const int64_t i0 = static_cast<int64_t>(blockIdx.x) * blockDim.x, i = i0 + threadIdx.x;
-    if (i0 >= n) return;
     const int64_t key = i < n ? pk[i] : 0;  // an input of earlier calls: loaded while the clearing finishes
-    wait_prior();                           // the cleared buckets and the table's segment offsets
+    // The cleared buckets and the table's segment offsets. Every block waits, those without
+    // a row too: the next call is ordered behind this grid alone, not behind the clearing.
+    wait_prior();
+    if (i0 >= n) return;
     int q = 0;
     if (S > 1) {
         // The block's first and last rows are searched for once; where they share a segment
@@ -436,7 +438,10 @@ probe_emit_kernel(TableView t, int32_t S, const int64_t* __restrict__ fk, const 
     // Positions fit 32 bits (batches hold at most INT32_MAX rows).
     const uint32_t tb = static_cast<uint32_t>(blockIdx.x) * kTile;
     const int rows = n - tb >= kTile ? kTile : static_cast<int>(n - tb);  // valid positions in this tile (<= 0: none)
-    if (rows <= 0) return;
+    if (rows <= 0) {
+        wait_prior();  // as in build_insert_kernel: the scan writes the row count that the next call reads
+        return;
+    }
     int lp[kItems];  // position within the tile
     int32_t mr[kItems], prow[kItems];
 #pragma unroll
