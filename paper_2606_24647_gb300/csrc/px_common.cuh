@@ -279,8 +279,11 @@ __device__ __forceinline__ void prefetch_l2(const void* p, uint32_t bytes) {
 // that kernel writes. Work that needs no such data (staging inputs of earlier
 // calls, clearing shared memory) runs before the wait and overlaps the tail of the
 // kernel before. wait_prior() returns when the kernel before has completed and its
-// memory is visible; since that kernel waited for its own predecessor the same way,
-// the whole stream before is then complete.
+// memory is visible; since every block of that kernel waited for its own predecessor the
+// same way (also a block that finds nothing to do), the whole stream before is then
+// complete. What the kernel before writes is not passed as `const T* __restrict__`: that
+// promises memory nobody writes while the kernel lives, so the compiler could load it
+// ahead of the wait or through the non-coherent path.
 __device__ __forceinline__ void wait_prior() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void allow_dependents() { asm volatile("griddepcontrol.launch_dependents;" :::); }
 

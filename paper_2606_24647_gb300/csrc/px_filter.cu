@@ -164,8 +164,8 @@ filter_count_kernel(const T* __restrict__ col, int64_t ncap, const int64_t* __re
 template <typename T, int W>
 __global__ void __launch_bounds__(kThreads, kBlocksPerSm)
 filter_write_kernel(const T* __restrict__ col, int64_t ncap, const int64_t* __restrict__ d_nrows, Range<T> g,
-                    int64_t ntiles, const int32_t* __restrict__ tile_cnt, const uint32_t* __restrict__ bits,
-                    int32_t* __restrict__ sel, int64_t* __restrict__ d_nsel) {
+                    int64_t ntiles, const int32_t* tile_cnt, const uint32_t* bits, int32_t* __restrict__ sel,
+                    int64_t* __restrict__ d_nsel) {
     constexpr int kTile = kWarps * 32 * W;
     __shared__ uint32_t s_warp[2][kWarps];
     __shared__ int32_t s_rows[W == 32 ? kWarps : 1][W == 32 ? kStage : 1];

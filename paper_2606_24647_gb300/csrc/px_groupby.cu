@@ -1367,7 +1367,7 @@ px_status launch_probe_sum_count(const Spec& sp, int32_t sum_slot, int32_t cnt_s
 // (segment, key) order, after the groups the hash path claimed (rows whose keys
 // fell outside the key range). Single pass with a bounded look-back.
 __global__ void __launch_bounds__(kEmitThreads)
-dense_emit_kernel(Spec sp, const unsigned long long* __restrict__ ngroups_hash, int64_t max_groups,
+dense_emit_kernel(Spec sp, const unsigned long long* ngroups_hash, int64_t max_groups,
                   int32_t* __restrict__ out_seg, int64_t* __restrict__ d_ngroups, ScanScratch scan, int32_t* status,
                   int64_t ntiles) {
     __shared__ int64_t s_tile;

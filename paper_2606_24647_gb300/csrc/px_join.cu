@@ -377,7 +377,7 @@ constexpr int kScanTile = kScanThreads * kScanItems;
 // Exclusive scan of the tile counts (single pass, bounded look-back); the last
 // tile writes the total to *d_nout and flags an output over capacity.
 __global__ void __launch_bounds__(kScanThreads)
-probe_scan_kernel(const int32_t* __restrict__ cnt, int64_t* __restrict__ off, int64_t total, int64_t out_cap,
+probe_scan_kernel(const int32_t* cnt, int64_t* __restrict__ off, int64_t total, int64_t out_cap,
                   int64_t* __restrict__ d_nout, ScanScratch scan, int32_t* status, int64_t nscan_tiles) {
     __shared__ int64_t s_tile;
     __shared__ int64_t s_warp[kScanThreads / 32];
@@ -429,8 +429,7 @@ template <bool kSel>
 __global__ void __launch_bounds__(kThreads)
 probe_emit_kernel(TableView t, int32_t S, const int64_t* __restrict__ fk, const int32_t* __restrict__ sel,
                   const int64_t* __restrict__ d_n, int64_t ncap, const int64_t* __restrict__ pseg,
-                  const int32_t* __restrict__ mrow, const int32_t* __restrict__ tile_cnt,
-                  const int64_t* __restrict__ tile_off, OutCols oc, int32_t* __restrict__ probe_row,
+                  const int32_t* mrow, const int32_t* tile_cnt, const int64_t* tile_off, OutCols oc, int32_t* __restrict__ probe_row,
                   int32_t* __restrict__ build_row, int64_t out_cap) {
     __shared__ int32_t s_warp[kWarps];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -585,8 +584,8 @@ probe_emit_kernel(TableView t, int32_t S, const int64_t* __restrict__ fk, const 
 __global__ void __launch_bounds__(kTile)
 probe_seg_kernel(TableView t, int32_t S, int32_t segmented, const int64_t* __restrict__ pseg,
                  const int64_t* __restrict__ fk, const int32_t* __restrict__ sel, const int64_t* __restrict__ d_n,
-                 int64_t ncap, const int32_t* __restrict__ mrow, const int64_t* __restrict__ tile_off,
-                 const int64_t* __restrict__ d_nout, int64_t* __restrict__ d_out_seg) {
+                 int64_t ncap, const int32_t* mrow, const int64_t* tile_off, const int64_t* d_nout,
+                 int64_t* __restrict__ d_out_seg) {
     __shared__ int32_t s_warp[kTile / 32];
     wait_prior();  // the match rows, tile offsets and row count
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;

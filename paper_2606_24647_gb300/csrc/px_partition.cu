@@ -159,7 +159,7 @@ part_hist_kernel(const int64_t* __restrict__ key, const int32_t* __restrict__ se
 // Exclusive scan of cnt[0..total) (partition-major) into offs; offsets[q] is the
 // scanned value at (q, tile 0) and offsets[nparts] the grand total.
 __global__ void __launch_bounds__(kScanThreads)
-part_scan_kernel(const int32_t* __restrict__ cnt, int32_t* __restrict__ offs, int64_t total,
+part_scan_kernel(const int32_t* cnt, int32_t* __restrict__ offs, int64_t total,
                  int64_t ntiles, uint32_t nparts, int64_t* __restrict__ d_offsets, ScanScratch scan,
                  int32_t* status, int64_t nscan_tiles) {
     __shared__ int64_t s_tile;
@@ -378,7 +378,7 @@ __device__ __forceinline__ void rank_tile(const uint32_t* pidv, int32_t* posv, i
 
 // The tile's output start in each of this thread's partitions (one strided load each).
 template <int NBITS>
-__device__ __forceinline__ void load_offs(int32_t (&my_off)[kPer<NBITS>], const int32_t* __restrict__ offs,
+__device__ __forceinline__ void load_offs(int32_t (&my_off)[kPer<NBITS>], const int32_t* offs,
                                           uint32_t nparts, int64_t ntiles, int64_t tile) {
 #pragma unroll
     for (int r = 0; r < kPer<NBITS>; ++r) {
@@ -392,8 +392,8 @@ template <int ITEMS, int NBITS>
 __global__ void __launch_bounds__(kThreads, ITEMS >= 8 ? 3 : 4)
 part_scatter_kernel(Cols cols, int32_t key_col, const int32_t* __restrict__ sel,
                     const int64_t* __restrict__ d_nsel, int64_t ncap, uint64_t seed, uint32_t nparts,
-                    const int32_t* __restrict__ offs, int64_t ntiles, uint32_t stage_bytes, uint32_t row_bytes,
-                    const uint8_t* __restrict__ pid_in, int32_t* status) {
+                    const int32_t* offs, int64_t ntiles, uint32_t stage_bytes, uint32_t row_bytes,
+                    const uint8_t* pid_in, int32_t* status) {
     constexpr int T = kThreads * ITEMS;
     extern __shared__ __align__(16) unsigned char smem[];
     const int np1 = static_cast<int>(nparts) + 1;
@@ -535,8 +535,8 @@ __device__ __forceinline__ void place_t(void* buf, const int32_t* row, const int
 template <int ITEMS, int NBITS>
 __global__ void __launch_bounds__(kThreads, ITEMS >= 8 ? 3 : 4)
 part_direct_kernel(Cols cols, int32_t key_col, const int32_t* __restrict__ sel, const int64_t* __restrict__ d_nsel,
-                   int64_t ncap, uint64_t seed, uint32_t nparts, const int32_t* __restrict__ offs, int64_t ntiles,
-                   const uint8_t* __restrict__ pid_in) {
+                   int64_t ncap, uint64_t seed, uint32_t nparts, const int32_t* offs, int64_t ntiles,
+                   const uint8_t* pid_in) {
     constexpr int T = kThreads * ITEMS;
     extern __shared__ __align__(16) unsigned char smem[];
     int32_t* s_dest = reinterpret_cast<int32_t*>(smem + T * 8);  // after the buffer of T 8-byte values
