@@ -229,7 +229,7 @@ def _words(t: torch.Tensor) -> tuple:
 # 40 % of a small call's host time (three calls on 20,000 rows: 111 us, now 63).
 # The address is only used while the array is alive, that is during the call.
 def _pack(cols, nrows: int, d_nrows=None) -> array.array:
-    w = [len(cols), 0, nrows, _ptr(d_nrows) or 0]
+    w = [len(cols), 0, nrows & (2**64 - 1), _ptr(d_nrows) or 0]  # a negative count is for the library to refuse
     for c in cols:
         w += _words(c)
     a = array.array("Q", w)
