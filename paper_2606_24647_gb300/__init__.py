@@ -163,7 +163,8 @@ def load(path: str | None = None):
         lib, calls = ctypes.CDLL(path), ctypes.CDLL(path)
         _declare(lib)
         _declare_calls(calls)
-        _lib, _calls = lib, calls
+        _calls = calls  # before _lib: another thread that finds _lib set uses both
+        _lib = lib
     return _lib
 
 

@@ -1,5 +1,6 @@
 """The binding's packed descriptors and its loading of the library (no GPU)."""
 import ctypes
+import dis
 
 import paper_2606_24647_gb300 as px
 
@@ -17,3 +18,10 @@ def test_negative_row_count_reaches_the_library():
     px.load()
     st = px._calls.px_gather(px._at(a), None, None, px._at(a), None, 0, None)
     assert st == px.PX_ERR_UNSUPPORTED and "nrows -1" in px.last_error()
+
+
+def test_library_appears_with_its_calls():
+    """A thread that finds the library loaded finds the operator calls too: load() stores
+    them first."""
+    stores = [i.argval for i in dis.get_instructions(px.load) if i.opname == "STORE_GLOBAL"]
+    assert stores == ["_calls", "_lib"]
