@@ -2,6 +2,8 @@
 import ctypes
 import dis
 
+import torch
+
 import paper_2606_24647_gb300 as px
 
 
@@ -25,3 +27,11 @@ def test_library_appears_with_its_calls():
     them first."""
     stores = [i.argval for i in dis.get_instructions(px.load) if i.opname == "STORE_GLOBAL"]
     assert stores == ["_calls", "_lib"]
+
+
+def test_current_stream_without_the_private_call(monkeypatch):
+    class Stream:
+        cuda_stream = 0x1234
+    monkeypatch.delattr(torch._C, "_cuda_getCurrentRawStream", raising=False)
+    monkeypatch.setattr(torch.cuda, "current_stream", lambda: Stream)
+    assert px._stream(None) == 0x1234 and px._stream(Stream) == 0x1234
