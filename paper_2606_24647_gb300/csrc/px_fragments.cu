@@ -27,7 +27,7 @@
 // fragments, 388M rows, 28 B per row of columns and 2.4 GB of tables. Measured on
 // that batch: every row looked up in place 12.8 ms; passing rows queued and looked up
 // by full warps 6.0 ms; the next run's columns prefetched into L2, the items' walks
-// merged and small block arrays 3.8 ms; spread tables, items of 32768 rows and the keys
+// merged and block arrays of 24 KB 3.8 ms; spread tables, items of 32768 rows and the keys
 // read beside the filter 3.5 ms (3.4 TB/s). Blocks of 512 threads with 2 rows in flight
 // per thread (two per SM, 64 registers): 3.5 ms; 256 x 2 3.9 ms, 512 x 4 (one per SM, 128
 // registers) 3.8 ms.
@@ -41,10 +41,14 @@
 namespace px {
 namespace {
 
-// Shared-mode block accumulators. Direct mode above: 64M rows over 1M-key tables, 3
-// aggregates: 4000 groups take 0.89 ms direct and 1.28 ms with 96 KB block arrays
-// (two such blocks leave the SM no L1 for the table); 1000 groups 0.82 ms shared.
-constexpr size_t kSmemAccBudget = 24 * 1024;
+// Shared-mode block accumulators, direct mode above. 48M rows over 500,000-key tables, a
+// 30 % filter, 3 aggregates (24 bytes a group), uniform keys / Zipf(1.1) keys, us: 1100 groups
+// shared 494 / 410, direct 733 / 956; 2000 groups 557 / 448 and 673 / 934; 2700 groups (63 KB)
+// 834 / 622 and 661 / 878; 4000 groups (94 KB) 682 / 645 and 643 / 957. Direct reductions of a
+// hot group queue at one address; large arrays leave every fragment of the batch less L1:
+// with the queues, two blocks of up to 42 KB fit the 164 KB split of the SM's memory
+// (512 fragments: 24 KB 3.48 ms, 40 KB 3.45, 48 KB 3.70).
+constexpr size_t kSmemAccBudget = 42 * 1024;
 constexpr int64_t kMaxChunk = 32768;               // rows per work item, unless the caller says (65536: 3 % slower)
 constexpr uint64_t kRepSlots = 1024;               // shared-mode slots with their replicas, at most
 constexpr int kEmitThreads = 256;
