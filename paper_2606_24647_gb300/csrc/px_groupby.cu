@@ -1440,10 +1440,13 @@ dense_emit_kernel(Spec sp, const unsigned long long* ngroups_hash, int64_t max_g
     }
 }
 
+// Slots of a table of up to max_groups (< 2^31) groups: a power of two, two per group or
+// more, but no more than 32-bit slot numbers hold; above 2^30 groups that is still more
+// than one.
 uint32_t gtable_slots(int64_t max_groups) {
-    uint64_t G = 1024;
-    while (G < 2 * static_cast<uint64_t>(max_groups)) G <<= 1;
-    return static_cast<uint32_t>(G);
+    uint32_t G = 1024;
+    while (G < 2 * static_cast<uint64_t>(max_groups) && G < (1u << 31)) G <<= 1;
+    return G;
 }
 
 // Slots of the hash mode's block-local cache: keys and split accumulators.
