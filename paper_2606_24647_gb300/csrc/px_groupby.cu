@@ -120,11 +120,22 @@ __device__ __forceinline__ void write_group(const Spec& sp, uint64_t code, int32
     if (out_seg) out_seg[gi] = sp.segbits ? static_cast<int32_t>(code >> sp.keybits) : 0;
 }
 
+// A table of more groups than the output holds is given up before it is full: the result
+// is over capacity anyway, and every row of an absent group would walk the longer the
+// fuller the table is, in the end all of it. 1M distinct keys, capacity 20,000: this table
+// 670 ms, now 0.73; hash mode (see kWalk) 34 ms, now 0.52. A table of up to kFilledSlots is filled whole.
+constexpr uint32_t kFilledSlots = 16384;
+
 // Output row of a group code, claiming a slot (and a row) on first sight.
 __device__ int32_t global_group(const GTable& g, const Spec& sp, uint64_t code, int64_t max_groups, int32_t* out_seg,
                                 int32_t* status) {
     uint32_t s = static_cast<uint32_t>(fmix64(code)) & g.mask;
     for (uint32_t probe = 0; probe <= g.mask; ++probe) {
+        if (probe % 64 == 8) {
+            const uint64_t most = g.mask < kFilledSlots ? g.mask : g.mask - g.mask / 16;
+            const uint64_t claimed = *static_cast<volatile unsigned long long*>(g.ngroups);
+            if (claimed > most && claimed > static_cast<uint64_t>(max_groups)) break;
+        }
         uint32_t st = ld_acquire_u32(&g.state[s]);
         if (st == 0) {
             st = atomicCAS(&g.state[s], 0u, 1u);
@@ -640,6 +651,7 @@ __device__ __forceinline__ void aggregate_runs(const Spec& sp, const Streams& in
 // on, so a lookup mostly reads one sector and ends at the first empty slot.
 struct HTable {
     unsigned long long* emitted;  // the emit's counter (see hash_emit_kernel), zero between calls
+    uint32_t* done;           // blocks of the emit done where rows were lost, zero between calls
     unsigned long long* key;  // [slots + 1], 32-byte aligned
     unsigned long long* acc;  // [slots + 1] << shift
     uint32_t slots;           // a power of two
@@ -691,16 +703,31 @@ __device__ __forceinline__ uint32_t bucket_slot(const HTable& h, uint32_t bucket
     return at;
 }
 
+// Buckets that a lookup walks past its home bucket. Up to half of the slots are taken by as
+// many groups as the output holds, and a run of 65 full buckets does not come about then by
+// any keys but chosen ones; beyond that the table is mostly too small, and a walk through
+// all of it, by every row of an absent group, has no end to speak of. Rows that find no
+// slot are `lost` to the kernel: the emit sees to them (hash_lost).
+constexpr uint32_t kWalk = 64;
+
 // The slot of `inv` from bucket `bucket` on (its first bucket was full); kNoSlot where
-// the table is full.
+// kWalk buckets are full. Kept small: registers that it needs are taken from the kernel
+// (the end of the walk decided here: 100,000 groups 208 -> 300 us).
 __device__ __noinline__ uint32_t hash_walk(const HTable& h, uint32_t bucket, unsigned long long inv) {
     const uint32_t last = h.slots / kBucketSlots - 1;
-    for (uint32_t round = 0; round < last; ++round) {
+#pragma unroll 1
+    for (uint32_t round = 0; round < kWalk; ++round) {
         bucket = (bucket + 1) & last;
         const uint32_t at = bucket_slot(h, bucket, load_keys(h, bucket), inv);
         if (at != kNoSlot) return at;
     }
     return kNoSlot;
+}
+
+// Tells the emit that a row found no slot.
+constexpr unsigned long long kLostBit = 1ull << 63;  // of *HTable::emitted
+__device__ __forceinline__ void note_lost(const HTable& h) {
+    if (!(*static_cast<volatile unsigned long long*>(h.emitted) & kLostBit)) atomicOr(h.emitted, kLostBit);
 }
 
 // Two neighbouring 64-bit words of shared memory, read anew.
@@ -736,7 +763,7 @@ __device__ __forceinline__ uint32_t cache_claim(unsigned long long* c_key, uint3
 template <int NA>
 __global__ void __launch_bounds__(kHashThreads, kHashBlocksPerSm)
 groupby_hash_kernel(Spec sp, const int32_t* __restrict__ sel, const int64_t* __restrict__ d_n, int64_t ncap,
-                    const int64_t* __restrict__ d_seg, HTable h, uint32_t cache_slots, int32_t* status) {
+                    const int64_t* __restrict__ d_seg, HTable h, uint32_t cache_slots) {
     extern __shared__ __align__(16) unsigned char smem[];
     const uint32_t C = cache_slots;
     unsigned long long* c_key = reinterpret_cast<unsigned long long*>(smem);  // [C], ~code or 0
@@ -859,7 +886,7 @@ groupby_hash_kernel(Spec sp, const int32_t* __restrict__ sel, const int64_t* __r
                         if (slot == kNoSlot) slot = hash_walk(h, bucket[i], inv[i]);
                     }
                     if (slot == kNoSlot) {
-                        set_status(status, PX_ERR_CAPACITY);
+                        note_lost(h);
                     } else {
                         unsigned long long* acc = h.acc + (static_cast<size_t>(slot) << h.shift);
 #pragma unroll
@@ -879,7 +906,7 @@ groupby_hash_kernel(Spec sp, const int32_t* __restrict__ sel, const int64_t* __r
             const uint32_t home = static_cast<uint32_t>(fmix64(~ci)) & (h.slots / kBucketSlots - 1);
             uint32_t slot = bucket_slot(h, home, load_keys(h, home), ci);
             if (slot == kNoSlot) slot = hash_walk(h, home, ci);
-            if (slot == kNoSlot) set_status(status, PX_ERR_CAPACITY);
+            if (slot == kNoSlot) note_lost(h);
             for (int a = 0; a < sp.naggs; ++a) {
                 const uint32_t o = static_cast<uint32_t>(a) * C + c;
                 const uint64_t x = (static_cast<uint64_t>(c_hi[o]) << 32) | c_lo[o];
@@ -898,19 +925,64 @@ constexpr int kEmitItems = 8;
 constexpr int kEmitTile = kEmitThreads * kEmitItems;
 constexpr int kEmitWarps = kEmitThreads / 32;
 
-// Writes the table's groups out, in no particular order: each block takes its tile's
-// output rows with one add to *h.emitted, whose low bits count groups and whose high
-// bits count blocks; the last block writes the total and clears it.
-constexpr int kEmittedBits = 40;
-__global__ void __launch_bounds__(kEmitThreads)
-hash_emit_kernel(Spec sp, HTable h, int64_t max_groups, int32_t* __restrict__ out_seg, int64_t* __restrict__ d_ngroups,
-                 int32_t* status) {
-    __shared__ int32_t s_warp[kEmitWarps];
-    __shared__ int64_t s_base;
+// Adds the lost rows of a table of `groups` groups, at slots beyond their walk: buckets
+// never empty again, so a code that is not among its first kWalk + 1 buckets has no row in
+// the table yet. For one block, alone.
+__device__ void hash_lost(const Spec& sp, const int32_t* sel, int64_t n, const int64_t* d_seg, const HTable& h,
+                          int64_t groups, int64_t max_groups, int32_t* status) {
+    __shared__ unsigned long long s_groups;
+    if (threadIdx.x == 0) s_groups = static_cast<unsigned long long>(groups);
+    __syncthreads();
+    volatile unsigned long long* now = &s_groups;
+    const uint32_t buckets = h.slots / kBucketSlots;
+    for (int64_t j = threadIdx.x; j < n && *now <= static_cast<unsigned long long>(max_groups); j += blockDim.x) {
+        const int64_t r = sel ? sel[j] : j;
+        const int q = sp.nsegs > 1 ? seg_of(d_seg, sp.nsegs, j) : 0;
+        const uint64_t code = compose(sp, load_int(sp.key_in[0], sp.key_w[0], r),
+                                      sp.nkeys > 1 ? load_int(sp.key_in[1], sp.key_w[1], r) : 0, q);
+        const unsigned long long inv = ~code;
+        if (inv == 0) continue;  // has a slot of its own
+        uint32_t b = static_cast<uint32_t>(fmix64(code)) & (buckets - 1);
+        uint32_t slot = kNoSlot;
+        bool walked = true;  // to the end of its walk without a slot: a lost row
+        for (uint32_t round = 0; round < buckets && slot == kNoSlot; ++round, b = (b + 1) & (buckets - 1)) {
+            const KeyBucket kb = load_keys(h, b);
+            for (uint32_t k = 0; k < kBucketSlots && slot == kNoSlot; ++k) {
+                unsigned long long key = kb.k[k];
+                if (key == 0 && round > kWalk) {
+                    key = atomicCAS(&h.key[b * kBucketSlots + k], 0ull, inv);
+                    if (key == 0) {
+                        atomicAdd(&s_groups, 1ull);
+                        key = inv;
+                    }
+                }
+                if (key == inv) {
+                    slot = b * kBucketSlots + k;
+                    walked = round > kWalk;
+                }
+            }
+        }
+        if (slot == kNoSlot) set_status(status, PX_ERR_CAPACITY);
+        if (slot == kNoSlot || !walked) continue;
+        unsigned long long* acc = h.acc + (static_cast<size_t>(slot) << h.shift);
+        for (int a = 0; a < sp.naggs; ++a) {
+            uint64_t x = 1;
+            if (sp.op[a] != PX_COUNT) x = static_cast<uint64_t>(load_int(sp.a_in[a], sp.a_w[a], r));
+            if (sp.op[a] == PX_SUM_MUL) x *= static_cast<uint64_t>(load_int(sp.b_in[a], sp.b_w[a], r));
+            red_add_global(acc + a, x);
+        }
+    }
+    __syncthreads();
+}
+
+// Writes out the groups in tile `tile` of the table's slots, from the output row that
+// first_row(groups in the tile) gives thread 0 on.
+template <typename F>
+__device__ __forceinline__ void hash_emit_tile(const Spec& sp, const HTable& h, int64_t tile, int64_t max_groups,
+                                               int32_t* out_seg, int32_t* s_warp, int64_t* s_base, F first_row) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    wait_prior();  // the table
     const int64_t nslots = static_cast<int64_t>(h.slots) + 1;
-    const int64_t base = static_cast<int64_t>(blockIdx.x) * kEmitTile + warp * (32 * kEmitItems) + lane;
+    const int64_t base = tile * kEmitTile + warp * (32 * kEmitItems) + lane;
     unsigned long long key[kEmitItems];
 #pragma unroll
     for (int i = 0; i < kEmitItems; ++i) key[i] = base + i * 32 < nslots ? h.key[base + i * 32] : 0;
@@ -930,19 +1002,12 @@ hash_emit_kernel(Spec sp, HTable h, int64_t max_groups, int32_t* __restrict__ ou
             s_warp[w] = total;
             total += c;
         }
-        const unsigned long long old =
-            atomicAdd(h.emitted, (1ull << kEmittedBits) | static_cast<unsigned long long>(total));
-        s_base = static_cast<int64_t>(old & ((1ull << kEmittedBits) - 1));
-        if ((old >> kEmittedBits) == gridDim.x - 1) {
-            *h.emitted = 0;
-            *d_ngroups = s_base + total;
-            if (s_base + total > max_groups) set_status(status, PX_ERR_CAPACITY);
-        }
+        *s_base = first_row(total);
     }
     __syncthreads();
     const uint32_t lt = lanemask_lt();
     int64_t p[kEmitItems];  // output row, or -1
-    int64_t pos = s_base + s_warp[warp];
+    int64_t pos = *s_base + s_warp[warp];
 #pragma unroll
     for (int i = 0; i < kEmitItems; ++i) {
         p[i] = pos + __popc(mask[i] & lt);
@@ -964,6 +1029,69 @@ hash_emit_kernel(Spec sp, HTable h, int64_t max_groups, int32_t* __restrict__ ou
         for (int i = 0; i < kEmitItems; ++i)
             if (p[i] >= 0) out[p[i]] = static_cast<int64_t>(v[i]);
     }
+}
+
+// The end of the emit where rows were lost. If the groups exceed the output, that is the
+// result; else (keys chosen to meet in one place) the last block to be done adds the lost
+// rows and writes all groups out anew.
+__device__ __noinline__ void hash_emit_lost(const Spec& sp, const HTable& h, int64_t max_groups, int32_t* out_seg,
+                                            int64_t* d_ngroups, int32_t* status, const int32_t* sel,
+                                            const int64_t* d_n, int64_t ncap, const int64_t* d_seg) {
+    __shared__ int32_t s_warp[kEmitWarps];
+    __shared__ int64_t s_base;
+    __shared__ bool s_last;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();  // with the barrier above: the block's output rows
+        s_last = atomicAdd(h.done, 1u) == gridDim.x - 1;
+        __threadfence();
+    }
+    __syncthreads();
+    if (!s_last) return;
+    if (threadIdx.x == 0) *h.done = 0;
+    const int64_t groups = *static_cast<volatile int64_t*>(d_ngroups);
+    if (groups > max_groups) return;
+    hash_lost(sp, sel, actual_rows(d_n, ncap), d_seg, h, groups, max_groups, status);
+    int64_t run = 0;
+    for (int64_t tile = 0; tile < gridDim.x; ++tile) {
+        hash_emit_tile(sp, h, tile, max_groups, out_seg, s_warp, &s_base, [&](int32_t total) {
+            run += total;
+            return run - total;
+        });
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) {
+        *d_ngroups = run;
+        if (run > max_groups) set_status(status, PX_ERR_CAPACITY);
+    }
+}
+
+// Writes the table's groups out, in no particular order: each block takes its tile's
+// output rows with one add to *h.emitted, whose low bits count groups, whose high bits
+// count blocks and whose highest bit tells of lost rows; the last block writes the total and
+// clears it.
+constexpr int kEmittedBits = 40;
+__global__ void __launch_bounds__(kEmitThreads, 4)
+hash_emit_kernel(const __grid_constant__ Spec sp, const __grid_constant__ HTable h, int64_t max_groups,
+                 int32_t* __restrict__ out_seg, int64_t* d_ngroups, int32_t* status, const int32_t* __restrict__ sel,
+                 const int64_t* __restrict__ d_n, int64_t ncap, const int64_t* __restrict__ d_seg) {
+    __shared__ int32_t s_warp[kEmitWarps];
+    __shared__ int64_t s_base;
+    wait_prior();  // the table
+    __shared__ bool s_lost;
+    hash_emit_tile(sp, h, blockIdx.x, max_groups, out_seg, s_warp, &s_base, [&](int32_t total) {
+        const unsigned long long old =
+            atomicAdd(h.emitted, (1ull << kEmittedBits) | static_cast<unsigned long long>(total));
+        const int64_t first = static_cast<int64_t>(old & ((1ull << kEmittedBits) - 1));
+        s_lost = (old & kLostBit) != 0;
+        if (((old & ~kLostBit) >> kEmittedBits) == gridDim.x - 1) {
+            *h.emitted = 0;
+            *d_ngroups = first + total;
+            if (first + total > max_groups) set_status(status, PX_ERR_CAPACITY);
+        }
+        return first;
+    });
+    if (s_lost) hash_emit_lost(sp, h, max_groups, out_seg, d_ngroups, status, sel, d_n, ncap, d_seg);
 }
 
 // Dense modes: kDenseBlock (block arrays) and kDenseDirect (rows straight into the
@@ -1449,6 +1577,11 @@ uint32_t gtable_slots(int64_t max_groups) {
     return G;
 }
 
+// Slots of the hash mode's table. Not fewer than kMinHashSlots, so that a small capacity
+// that is exceeded still gets a full count of a few thousand groups.
+constexpr uint32_t kMinHashSlots = 8192;
+uint32_t htable_slots(int64_t max_groups) { return std::max(gtable_slots(max_groups), kMinHashSlots); }
+
 // Slots of the hash mode's block-local cache: keys and split accumulators.
 uint32_t cache_slots(int naggs) {
     uint32_t s = 4096;
@@ -1463,7 +1596,7 @@ int acc_shift(int naggs) { return naggs <= 1 ? 0 : (naggs == 2 ? 1 : (naggs <= 4
 size_t htable_bytes(uint32_t slots, int naggs) {
     return align_up(8 * (static_cast<size_t>(slots) + 1), 256) + (8 * (static_cast<size_t>(slots) + 1) << acc_shift(naggs));
 }
-constexpr size_t kEmittedBytes = 256;  // the emit's counter, before the table
+constexpr size_t kEmittedBytes = 256;  // HTable::emitted and done, before the table
 
 int num_sms() {
     int dev = 0, n = 0;
@@ -1520,13 +1653,13 @@ px_status launch_runs(const Spec& sp, size_t smem, const int64_t* d_n, int64_t n
 
 template <int NA>
 px_status launch_hash(const Spec& sp, const int32_t* sel, const int64_t* d_n, int64_t ncap, const int64_t* d_seg,
-                      const HTable& h, int32_t* status, cudaStream_t st) {
+                      const HTable& h, cudaStream_t st) {
     auto kernel = groupby_hash_kernel<NA>;
     const uint32_t C = cache_slots(sp.naggs);
     const size_t smem = static_cast<size_t>(C) * (8 + 8 * static_cast<size_t>(sp.naggs));
     allow_smem(kernel, smem);
     const int64_t grid = std::min<int64_t>(cdiv(ncap, kHashTile), static_cast<int64_t>(num_sms()) * kHashBlocksPerSm);
-    kernel<<<static_cast<unsigned>(grid), kHashThreads, smem, st>>>(sp, sel, d_n, ncap, d_seg, h, C, status);
+    kernel<<<static_cast<unsigned>(grid), kHashThreads, smem, st>>>(sp, sel, d_n, ncap, d_seg, h, C);
     note_launch();
     return check_launch("px_groupby_agg hash");
 }
@@ -1559,7 +1692,7 @@ WsLayout ws_layout(int64_t max_groups) {
     L.key = L.dg_acc + align_up((8 * PX_MAX_AGGS + 1) * M, 256);
     L.gidx = L.key + align_up(8 * G, 256);
     L.total = std::max(L.gidx + align_up(4 * G, 256),
-                       kWsScratch + kEmittedBytes + 32 + htable_bytes(static_cast<uint32_t>(G), PX_MAX_AGGS));
+                       kWsScratch + kEmittedBytes + 32 + htable_bytes(htable_slots(max_groups), PX_MAX_AGGS));
     return L;
 }
 
@@ -1729,10 +1862,11 @@ static px_status groupby_impl(const px_batch* in, const int32_t* key_cols, int32
     if (!sp.dense) {
         // Hash mode. The table has two slots for every possible group; a stream of
         // calls keeps one table, so its size must not depend on a call's rows.
-        const uint32_t slots = gtable_slots(streaming ? max_groups : std::max<int64_t>(1, std::min(max_groups, ncap)));
+        const uint32_t slots = htable_slots(streaming ? max_groups : std::max<int64_t>(1, std::min(max_groups, ncap)));
         char* base = static_cast<char*>(d_ws) + kWsScratch;
         HTable h;
         h.emitted = reinterpret_cast<unsigned long long*>(base);
+        h.done = reinterpret_cast<uint32_t*>(base + 8);
         // a bucket is one 32-byte load; the caller's workspace is only 16-byte aligned
         char* keys = reinterpret_cast<char*>(align_up(reinterpret_cast<uintptr_t>(base) + kEmittedBytes, 32));
         h.key = reinterpret_cast<unsigned long long*>(keys);
@@ -1740,9 +1874,9 @@ static px_status groupby_impl(const px_batch* in, const int32_t* key_cols, int32
         h.slots = slots;
         h.shift = acc_shift(naggs);
         if (!accumulate) cudaMemsetAsync(base, 0, kEmittedBytes + 32 + htable_bytes(slots, naggs), st);
+        const int64_t* d_n = d_sel ? d_nsel : in->d_nrows;
         if (ncap > 0) {
-            const int64_t* d_n = d_sel ? d_nsel : in->d_nrows;
-            const auto go = [&](auto launch) { return launch(sp, d_sel, d_n, ncap, d_seg, h, status, st); };
+            const auto go = [&](auto launch) { return launch(sp, d_sel, d_n, ncap, d_seg, h, st); };
             switch (naggs) {
                 case 0: s = go(launch_hash<0>); break;
                 case 1: s = go(launch_hash<1>); break;
@@ -1757,9 +1891,10 @@ static px_status groupby_impl(const px_batch* in, const int32_t* key_cols, int32
         const dim3 grid(static_cast<unsigned>(cdiv(static_cast<int64_t>(slots) + 1, kEmitTile)));
         if (ncap > 0)
             launch_after(hash_emit_kernel, grid, dim3(kEmitThreads), 0, st, sp, h, max_groups, d_out_seg, d_ngroups,
-                         status);
+                         status, d_sel, d_n, ncap, d_seg);
         else
-            hash_emit_kernel<<<grid, kEmitThreads, 0, st>>>(sp, h, max_groups, d_out_seg, d_ngroups, status);
+            hash_emit_kernel<<<grid, kEmitThreads, 0, st>>>(sp, h, max_groups, d_out_seg, d_ngroups, status, d_sel, d_n,
+                                                            ncap, d_seg);
         note_launch();
         return check_launch("px_groupby_agg hash emit");
     }
