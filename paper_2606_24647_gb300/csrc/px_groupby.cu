@@ -643,7 +643,7 @@ __device__ __forceinline__ void aggregate_runs(const Spec& sp, const Streams& in
 
 // ---------------------------------------------------------------- hash mode ----
 // The table of groups, in the workspace: buckets of four slots (one 32-byte sector of
-// keys), at least two slots per possible group, and one slot more for the code whose
+// keys), one and a half slots or more per possible group, and one slot more for the code whose
 // stored form would read as empty. Keys hold ~code, 0 where empty; a slot's
 // accumulators sit together. A key is set once, by a CAS, and nothing else is published
 // with it: accumulators start at zero (cleared with the keys before the call), so no
@@ -654,7 +654,7 @@ struct HTable {
     uint32_t* done;           // blocks of the emit done where rows were lost, zero between calls
     unsigned long long* key;  // [slots + 1], 32-byte aligned
     unsigned long long* acc;  // [slots + 1] << shift
-    uint32_t slots;           // a power of two
+    uint32_t slots;           // a multiple of kBucketSlots
     int32_t shift;
 };
 
@@ -703,21 +703,22 @@ __device__ __forceinline__ uint32_t bucket_slot(const HTable& h, uint32_t bucket
     return at;
 }
 
-// Buckets that a lookup walks past its home bucket. Up to half of the slots are taken by as
-// many groups as the output holds, and a run of 65 full buckets does not come about then by
-// any keys but chosen ones; beyond that the table is mostly too small, and a walk through
-// all of it, by every row of an absent group, has no end to speak of. Rows that find no
-// slot are `lost` to the kernel: the emit sees to them (hash_lost).
+// Buckets that a lookup walks past its home bucket. As many groups as the output holds take
+// 0.4 of the slots, or two thirds; the longest run of full buckets is 17 at load 0.5 and 55 at
+// two thirds (simulated, 2^26 buckets), unless the keys were chosen for it. Beyond that the
+// table is mostly too small, and a walk through all of it, by every row of an absent group,
+// has no end to speak of. Rows that find no slot are `lost` to the kernel: the emit sees to
+// them (hash_lost).
 constexpr uint32_t kWalk = 64;
 
 // The slot of `inv` from bucket `bucket` on (its first bucket was full); kNoSlot where
 // kWalk buckets are full. Kept small: registers that it needs are taken from the kernel
 // (the end of the walk decided here: 100,000 groups 208 -> 300 us).
 __device__ __noinline__ uint32_t hash_walk(const HTable& h, uint32_t bucket, unsigned long long inv) {
-    const uint32_t last = h.slots / kBucketSlots - 1;
+    const uint32_t buckets = h.slots / kBucketSlots;
 #pragma unroll 1
     for (uint32_t round = 0; round < kWalk; ++round) {
-        bucket = (bucket + 1) & last;
+        bucket = bucket + 1 == buckets ? 0 : bucket + 1;
         const uint32_t at = bucket_slot(h, bucket, load_keys(h, bucket), inv);
         if (at != kNoSlot) return at;
     }
@@ -805,7 +806,7 @@ groupby_hash_kernel(Spec sp, const int32_t* __restrict__ sel, const int64_t* __r
                     const uint64_t code = compose(sp, k0[i], sp.nkeys > 1 ? k1[i] : 0, q);
                     const uint64_t hash = fmix64(code);
                     inv[i] = ~code;
-                    bucket[i] = static_cast<uint32_t>(hash) & (h.slots / kBucketSlots - 1);
+                    bucket[i] = slot_of(hash, h.slots / kBucketSlots);
                     cslot[i] = static_cast<uint32_t>(hash >> 32) & (C - 2);
                 }
             }
@@ -903,7 +904,7 @@ groupby_hash_kernel(Spec sp, const int32_t* __restrict__ sel, const int64_t* __r
         for (uint32_t c = tid; c < C; c += kHashThreads) {
             const unsigned long long ci = c_key[c];
             if (ci == 0) continue;
-            const uint32_t home = static_cast<uint32_t>(fmix64(~ci)) & (h.slots / kBucketSlots - 1);
+            const uint32_t home = slot_of(fmix64(~ci), h.slots / kBucketSlots);
             uint32_t slot = bucket_slot(h, home, load_keys(h, home), ci);
             if (slot == kNoSlot) slot = hash_walk(h, home, ci);
             if (slot == kNoSlot) note_lost(h);
@@ -942,10 +943,10 @@ __device__ void hash_lost(const Spec& sp, const int32_t* sel, int64_t n, const i
                                       sp.nkeys > 1 ? load_int(sp.key_in[1], sp.key_w[1], r) : 0, q);
         const unsigned long long inv = ~code;
         if (inv == 0) continue;  // has a slot of its own
-        uint32_t b = static_cast<uint32_t>(fmix64(code)) & (buckets - 1);
+        uint32_t b = slot_of(fmix64(code), buckets);
         uint32_t slot = kNoSlot;
         bool walked = true;  // to the end of its walk without a slot: a lost row
-        for (uint32_t round = 0; round < buckets && slot == kNoSlot; ++round, b = (b + 1) & (buckets - 1)) {
+        for (uint32_t round = 0; round < buckets && slot == kNoSlot; ++round, b = b + 1 == buckets ? 0 : b + 1) {
             const KeyBucket kb = load_keys(h, b);
             for (uint32_t k = 0; k < kBucketSlots && slot == kNoSlot; ++k) {
                 unsigned long long key = kb.k[k];
@@ -1577,10 +1578,23 @@ uint32_t gtable_slots(int64_t max_groups) {
     return G;
 }
 
-// Slots of the hash mode's table. Not fewer than kMinHashSlots, so that a small capacity
-// that is exceeded still gets a full count of a few thousand groups.
-constexpr uint32_t kMinHashSlots = 8192;
-uint32_t htable_slots(int64_t max_groups) { return std::max(gtable_slots(max_groups), kMinHashSlots); }
+// Slots of the hash mode's table: two and a half per group, or one and a half where a slot's
+// accumulators take 64 bytes, so that the table needs hardly more memory than the dense
+// modes (10M groups: 2.42 GB with a power of two of slots, now 1.19); small tables up to four.
+// Less to clear, at a load between those of the powers of two (10M rows: 1M groups 352 us,
+// now 308; 100,000 208 and 207; 30,000 200 and 206). Not fewer than kMinHashSlots, so that a
+// small capacity that is exceeded still gets a full count of a few thousand groups; as many
+// as 32-bit slot numbers hold.
+constexpr uint64_t kMinHashSlots = 8192;
+uint32_t htable_slots(int64_t max_groups, int naggs) {
+    const uint64_t m = static_cast<uint64_t>(max_groups);
+    uint64_t s = m + m / 2;
+    if (naggs <= 4) {
+        s = 2 * m + m / 2;
+        if (m <= 1 << 16) s = std::max<uint64_t>(s, gtable_slots(max_groups));
+    }
+    return static_cast<uint32_t>(std::min<uint64_t>(align_up(std::max(s, kMinHashSlots), kBucketSlots), 0xfffffff0u));
+}
 
 // Slots of the hash mode's block-local cache: keys and split accumulators.
 uint32_t cache_slots(int naggs) {
@@ -1691,8 +1705,9 @@ WsLayout ws_layout(int64_t max_groups) {
     L.dg_acc = L.state + align_up(4 * G, 256);
     L.key = L.dg_acc + align_up((8 * PX_MAX_AGGS + 1) * M, 256);
     L.gidx = L.key + align_up(8 * G, 256);
-    L.total = std::max(L.gidx + align_up(4 * G, 256),
-                       kWsScratch + kEmittedBytes + 32 + htable_bytes(htable_slots(max_groups), PX_MAX_AGGS));
+    L.total = L.gidx + align_up(4 * G, 256);
+    for (int naggs : {4, PX_MAX_AGGS})
+        L.total = std::max(L.total, kWsScratch + kEmittedBytes + 32 + htable_bytes(htable_slots(max_groups, naggs), naggs));
     return L;
 }
 
@@ -1860,9 +1875,9 @@ static px_status groupby_impl(const px_batch* in, const int32_t* key_cols, int32
     int32_t* status = &static_cast<WsHeader*>(d_ws)->status;
     const int64_t ncap = in->nrows;
     if (!sp.dense) {
-        // Hash mode. The table has two slots for every possible group; a stream of
-        // calls keeps one table, so its size must not depend on a call's rows.
-        const uint32_t slots = htable_slots(streaming ? max_groups : std::max<int64_t>(1, std::min(max_groups, ncap)));
+        // Hash mode. A stream of calls keeps one table, so its size must not depend on a
+        // call's rows.
+        const uint32_t slots = htable_slots(streaming ? max_groups : std::min(max_groups, ncap), naggs);
         char* base = static_cast<char*>(d_ws) + kWsScratch;
         HTable h;
         h.emitted = reinterpret_cast<unsigned long long*>(base);
