@@ -655,6 +655,7 @@ struct HTable {
     unsigned long long* key;  // [slots + 1], 32-byte aligned
     unsigned long long* acc;  // [slots + 1] << shift
     uint32_t slots;           // a multiple of kBucketSlots
+    uint32_t* chosen;         // LOOSE: the slots that are used (see hash_estimate_kernel)
     int32_t shift;
 };
 
@@ -666,6 +667,7 @@ constexpr size_t kCacheBudget = 64 * 1024;  // the block-local cache
 constexpr int kHashMajority = 12;           // smallest group worth a warp reduction here
 constexpr uint32_t kNoSlot = 0xffffffffu;
 constexpr uint32_t kBucketSlots = 4;
+constexpr uint64_t kMinHashSlots = 8192;    // see htable_slots
 
 struct KeyBucket {
     unsigned long long k[kBucketSlots];
@@ -761,11 +763,13 @@ __device__ __forceinline__ uint32_t cache_claim(unsigned long long* c_key, uint3
 // 207 us, Zipf(1.1) 1209 -> 153; 3000 groups 833 -> 152; 1M groups 1469 -> 353; 100
 // groups 97 -> 94. A cache slot pair is read with one 16-byte load and a bucket with
 // one 32-byte load; single-slot probing took 408 us at 100,000 groups.
-template <int NA>
+// LOOSE: the table's slots were chosen on the device.
+template <int NA, bool LOOSE>
 __global__ void __launch_bounds__(kHashThreads, kHashBlocksPerSm)
 groupby_hash_kernel(Spec sp, const int32_t* __restrict__ sel, const int64_t* __restrict__ d_n, int64_t ncap,
                     const int64_t* __restrict__ d_seg, HTable h, uint32_t cache_slots) {
     extern __shared__ __align__(16) unsigned char smem[];
+    if (LOOSE) h.slots = *h.chosen;
     const uint32_t C = cache_slots;
     unsigned long long* c_key = reinterpret_cast<unsigned long long*>(smem);  // [C], ~code or 0
     uint32_t* c_lo = reinterpret_cast<uint32_t*>(c_key + C);                  // [naggs][C]
@@ -928,29 +932,34 @@ constexpr int kEmitWarps = kEmitThreads / 32;
 
 // Adds the lost rows of a table of `groups` groups, at slots beyond their walk: buckets
 // never empty again, so a code that is not among its first kWalk + 1 buckets has no row in
-// the table yet. For one block, alone.
+// the table yet. With all_rows: adds every row, wherever its slot is (to a cleared table).
+// For one block, alone.
 __device__ void hash_lost(const Spec& sp, const int32_t* sel, int64_t n, const int64_t* d_seg, const HTable& h,
-                          int64_t groups, int64_t max_groups, int32_t* status) {
+                          bool all_rows, int64_t groups, int64_t max_groups, int32_t* status) {
     __shared__ unsigned long long s_groups;
     if (threadIdx.x == 0) s_groups = static_cast<unsigned long long>(groups);
     __syncthreads();
     volatile unsigned long long* now = &s_groups;
-    const uint32_t buckets = h.slots / kBucketSlots;
+    const uint32_t buckets = h.slots / kBucketSlots, from = all_rows ? 0 : kWalk + 1;
     for (int64_t j = threadIdx.x; j < n && *now <= static_cast<unsigned long long>(max_groups); j += blockDim.x) {
         const int64_t r = sel ? sel[j] : j;
         const int q = sp.nsegs > 1 ? seg_of(d_seg, sp.nsegs, j) : 0;
         const uint64_t code = compose(sp, load_int(sp.key_in[0], sp.key_w[0], r),
                                       sp.nkeys > 1 ? load_int(sp.key_in[1], sp.key_w[1], r) : 0, q);
         const unsigned long long inv = ~code;
-        if (inv == 0) continue;  // has a slot of its own
         uint32_t b = slot_of(fmix64(code), buckets);
         uint32_t slot = kNoSlot;
-        bool walked = true;  // to the end of its walk without a slot: a lost row
+        bool walked = true;  // past its walk without a slot: a lost row
+        if (inv == 0) {      // has a slot of its own
+            if (!all_rows) continue;
+            slot = h.slots;
+            if (atomicExch(&h.key[slot], 1ull) == 0) atomicAdd(&s_groups, 1ull);
+        }
         for (uint32_t round = 0; round < buckets && slot == kNoSlot; ++round, b = b + 1 == buckets ? 0 : b + 1) {
             const KeyBucket kb = load_keys(h, b);
             for (uint32_t k = 0; k < kBucketSlots && slot == kNoSlot; ++k) {
                 unsigned long long key = kb.k[k];
-                if (key == 0 && round > kWalk) {
+                if (key == 0 && round >= from) {
                     key = atomicCAS(&h.key[b * kBucketSlots + k], 0ull, inv);
                     if (key == 0) {
                         atomicAdd(&s_groups, 1ull);
@@ -959,7 +968,7 @@ __device__ void hash_lost(const Spec& sp, const int32_t* sel, int64_t n, const i
                 }
                 if (key == inv) {
                     slot = b * kBucketSlots + k;
-                    walked = round > kWalk;
+                    walked = round >= from;
                 }
             }
         }
@@ -1032,29 +1041,51 @@ __device__ __forceinline__ void hash_emit_tile(const Spec& sp, const HTable& h, 
     }
 }
 
-// The end of the emit where rows were lost. If the groups exceed the output, that is the
-// result; else (keys chosen to meet in one place) the last block to be done adds the lost
-// rows and writes all groups out anew.
-__device__ __noinline__ void hash_emit_lost(const Spec& sp, const HTable& h, int64_t max_groups, int32_t* out_seg,
-                                            int64_t* d_ngroups, int32_t* status, const int32_t* sel,
-                                            const int64_t* d_n, int64_t ncap, const int64_t* d_seg) {
+// Clears slots [0, slots] of the table, as thread `i` of `n`.
+__device__ void hash_clear(const HTable& h, uint32_t slots, size_t i, size_t n) {
+    const size_t keys = static_cast<size_t>(slots) + 1, words = keys << h.shift;
+    const ulonglong2 zero = {};
+    for (size_t k = i; k < keys / 2; k += n) reinterpret_cast<ulonglong2*>(h.key)[k] = zero;
+    for (size_t k = i; k < words / 2; k += n) reinterpret_cast<ulonglong2*>(h.acc)[k] = zero;
+    if (i == 0) {  // an odd last word
+        h.key[keys - 1] = 0;
+        h.acc[words - 1] = 0;
+    }
+}
+
+// The end of the emit where rows were lost, in the `blocks` blocks that emit. If the groups
+// exceed the output, that is the result; else (keys chosen to meet in one place) the last
+// block to be done adds the lost rows and writes all groups out anew. Where the slots were
+// chosen by an estimate, that was too low: the block makes the table of all `most` slots.
+__device__ __noinline__ void hash_emit_lost(const Spec& sp, const HTable& used, uint32_t most, uint32_t blocks,
+                                            int64_t max_groups, int32_t* out_seg, int64_t* d_ngroups, int32_t* status,
+                                            const int32_t* sel, const int64_t* d_n, int64_t ncap,
+                                            const int64_t* d_seg) {
+    HTable h = used;
     __shared__ int32_t s_warp[kEmitWarps];
     __shared__ int64_t s_base;
     __shared__ bool s_last;
     __syncthreads();
     if (threadIdx.x == 0) {
         __threadfence();  // with the barrier above: the block's output rows
-        s_last = atomicAdd(h.done, 1u) == gridDim.x - 1;
+        s_last = atomicAdd(h.done, 1u) == blocks - 1;
         __threadfence();
     }
     __syncthreads();
     if (!s_last) return;
     if (threadIdx.x == 0) *h.done = 0;
-    const int64_t groups = *static_cast<volatile int64_t*>(d_ngroups);
+    int64_t groups = *static_cast<volatile int64_t*>(d_ngroups);
     if (groups > max_groups) return;
-    hash_lost(sp, sel, actual_rows(d_n, ncap), d_seg, h, groups, max_groups, status);
+    const bool anew = h.slots < most;
+    if (anew) {
+        h.slots = most;
+        hash_clear(h, most, threadIdx.x, blockDim.x);
+        groups = 0;
+        __syncthreads();
+    }
+    hash_lost(sp, sel, actual_rows(d_n, ncap), d_seg, h, anew, groups, max_groups, status);
     int64_t run = 0;
-    for (int64_t tile = 0; tile < gridDim.x; ++tile) {
+    for (int64_t tile = 0; tile < cdiv(static_cast<int64_t>(h.slots) + 1, kEmitTile); ++tile) {
         hash_emit_tile(sp, h, tile, max_groups, out_seg, s_warp, &s_base, [&](int32_t total) {
             run += total;
             return run - total;
@@ -1067,32 +1098,159 @@ __device__ __noinline__ void hash_emit_lost(const Spec& sp, const HTable& h, int
     }
 }
 
-// Writes the table's groups out, in no particular order: each block takes its tile's
-// output rows with one add to *h.emitted, whose low bits count groups, whose high bits
-// count blocks and whose highest bit tells of lost rows; the last block writes the total and
-// clears it.
+// Writes the table's groups out, in no particular order: each tile's output rows are taken
+// with one add to *h.emitted, whose low bits count groups, whose high bits count tiles and
+// whose highest bit tells of lost rows; the last tile's block writes the total and clears it.
+// A block per tile, or (LOOSE) as many as are in flight at a time.
 constexpr int kEmittedBits = 40;
+template <bool LOOSE>
 __global__ void __launch_bounds__(kEmitThreads, 4)
-hash_emit_kernel(const __grid_constant__ Spec sp, const __grid_constant__ HTable h, int64_t max_groups,
+hash_emit_kernel(const __grid_constant__ Spec sp, const __grid_constant__ HTable h0, int64_t max_groups,
                  int32_t* __restrict__ out_seg, int64_t* d_ngroups, int32_t* status, const int32_t* __restrict__ sel,
                  const int64_t* __restrict__ d_n, int64_t ncap, const int64_t* __restrict__ d_seg) {
     __shared__ int32_t s_warp[kEmitWarps];
     __shared__ int64_t s_base;
-    wait_prior();  // the table
     __shared__ bool s_lost;
-    hash_emit_tile(sp, h, blockIdx.x, max_groups, out_seg, s_warp, &s_base, [&](int32_t total) {
-        const unsigned long long old =
-            atomicAdd(h.emitted, (1ull << kEmittedBits) | static_cast<unsigned long long>(total));
-        const int64_t first = static_cast<int64_t>(old & ((1ull << kEmittedBits) - 1));
-        s_lost = (old & kLostBit) != 0;
-        if (((old & ~kLostBit) >> kEmittedBits) == gridDim.x - 1) {
-            *h.emitted = 0;
-            *d_ngroups = first + total;
-            if (first + total > max_groups) set_status(status, PX_ERR_CAPACITY);
+    wait_prior();  // the table
+    HTable h = h0;
+    int64_t tiles = gridDim.x;
+    if (LOOSE) {
+        h.slots = *h.chosen;
+        tiles = cdiv(static_cast<int64_t>(h.slots) + 1, kEmitTile);
+        if (blockIdx.x >= tiles) return;
+    }
+    for (int64_t tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
+        if (LOOSE) __syncthreads();  // the tile before has read s_warp and s_base
+        hash_emit_tile(sp, h, tile, max_groups, out_seg, s_warp, &s_base, [&](int32_t total) {
+            const unsigned long long old =
+                atomicAdd(h.emitted, (1ull << kEmittedBits) | static_cast<unsigned long long>(total));
+            const int64_t first = static_cast<int64_t>(old & ((1ull << kEmittedBits) - 1));
+            s_lost = (old & kLostBit) != 0;
+            if (static_cast<int64_t>((old & ~kLostBit) >> kEmittedBits) == tiles - 1) {
+                *h.emitted = 0;
+                *d_ngroups = first + total;
+                if (first + total > max_groups) set_status(status, PX_ERR_CAPACITY);
+            }
+            return first;
+        });
+        if (!LOOSE) break;
+    }
+    if (s_lost)
+        hash_emit_lost(sp, h, h0.slots, static_cast<uint32_t>(gridDim.x < tiles ? gridDim.x : tiles), max_groups, out_seg,
+                       d_ngroups, status, sel, d_n, ncap, d_seg);
+}
+
+// How many slots the table of a large capacity uses: cleared and scanned whole it may cost
+// more than the rows do, and rows spread over more memory than they need go slower. Counts
+// distinct codes by HyperLogLog (Flajolet et al., 2007) in one row in eight, in two halves:
+// as a sample grows its distinct codes grow ever more slowly, so the whole has at most
+// d + 14 (d - h) of them, with d in the sample and h in half of it. A count that is too low
+// all the same (see hash_emit_lost) costs time, not rows.
+// 10M rows, 3 aggregates, capacity 10M: 100 groups 312 us, now 115; 100,000 groups 1004, now
+// 226; 1M groups 1055, now 718; 4.3M groups 1084 and 1096. The estimate itself takes 13 us
+// there, a chain of latencies.
+constexpr int kEstThreads = 1024;
+constexpr int kEstItems = 4;
+constexpr int kEstTile = kEstThreads * kEstItems;
+constexpr int kEstRegs = 2048;       // registers of one count: standard error 2.3 %
+constexpr int kEstRate = 8;          // one tile in so many is read,
+constexpr int64_t kEstAll = 1 << 20; // but every one of fewer rows than this
+constexpr size_t kEstBytes = 2 * kEstRegs * 4;
+
+__device__ __forceinline__ float hll_count(float sum, int zero) {
+    constexpr float m = kEstRegs;
+    const float e = 0.7213f / (1.0f + 1.079f / m) * m * m / sum;
+    return e <= 2.5f * m && zero > 0 ? m * logf(m / static_cast<float>(zero)) : e;
+}
+
+// regs: 2 x kEstRegs words, zero on entry, in memory of the table's keys; done: a counter of
+// blocks, zero on entry.
+__global__ void __launch_bounds__(kEstThreads)
+hash_estimate_kernel(const __grid_constant__ Spec sp, const int32_t* __restrict__ sel, const int64_t* __restrict__ d_n,
+                     int64_t ncap, const int64_t* __restrict__ d_seg, HTable h, uint32_t* regs, uint32_t* done) {
+    __shared__ uint32_t s_reg[2 * kEstRegs];
+    __shared__ float s_sum[3];  // of 2^-register: either half, both
+    __shared__ int s_zero[3];
+    __shared__ bool s_last;
+    const int tid = threadIdx.x;
+    allow_dependents();
+    for (int k = tid; k < 2 * kEstRegs; k += kEstThreads) s_reg[k] = 0;
+    if (tid < 3) {
+        s_sum[tid] = 0;
+        s_zero[tid] = 0;
+    }
+    __syncthreads();
+    const int64_t n = actual_rows(d_n, ncap);
+    const int rate = n >= kEstAll ? kEstRate : 1;
+    const int64_t tiles = cdiv(cdiv(n, kEstTile), rate);
+    for (int64_t t = blockIdx.x; t < tiles; t += gridDim.x) {
+        // a tile of each eight, not always the same one
+        const int64_t first = (t * rate + (rate > 1 ? static_cast<int64_t>(fmix64(t) % kEstRate) : 0)) * kEstTile;
+        uint32_t* const reg = s_reg + (t & 1) * kEstRegs;
+        int32_t row[kEstItems];
+#pragma unroll
+        for (int i = 0; i < kEstItems; ++i) {
+            const int64_t j = first + i * kEstThreads + tid;
+            row[i] = j < n ? (sel ? sel[j] : static_cast<int32_t>(j)) : -1;
         }
-        return first;
-    });
-    if (s_lost) hash_emit_lost(sp, h, max_groups, out_seg, d_ngroups, status, sel, d_n, ncap, d_seg);
+        int64_t k0[kEstItems], k1[kEstItems];
+        load_col(sp.key_in[0], sp.key_w[0], row, k0);
+        if (sp.nkeys > 1) load_col(sp.key_in[1], sp.key_w[1], row, k1);
+#pragma unroll
+        for (int i = 0; i < kEstItems; ++i) {
+            if (row[i] < 0) continue;
+            const int q = sp.nsegs > 1 ? seg_of(d_seg, sp.nsegs, first + i * kEstThreads + tid) : 0;
+            const uint64_t hash = fmix64(compose(sp, k0[i], sp.nkeys > 1 ? k1[i] : 0, q));
+            const uint32_t rank = __clzll(hash << 11 | 1024) + 1;
+            uint32_t* r = &reg[hash >> 53];
+            if (*static_cast<volatile uint32_t*>(r) < rank) atomicMax(r, rank);
+        }
+    }
+    __syncthreads();
+    for (int k = tid; k < 2 * kEstRegs; k += kEstThreads)
+        if (s_reg[k]) atomicMax(&regs[k], s_reg[k]);
+    __threadfence();
+    __syncthreads();
+    if (tid == 0) s_last = atomicAdd(done, 1u) == gridDim.x - 1;
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+    float sum[3] = {};
+    int zero[3] = {};
+    for (int k = tid; k < kEstRegs; k += kEstThreads) {
+        const uint32_t a = *static_cast<volatile uint32_t*>(&regs[k]), b = *static_cast<volatile uint32_t*>(&regs[kEstRegs + k]);
+        const uint32_t x[3] = {a, b, a > b ? a : b};
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            sum[c] += exp2f(-static_cast<float>(x[c]));
+            zero[c] += x[c] == 0;
+        }
+    }
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        const float w = warp_sum(sum[c]);
+        const int z = warp_sum(zero[c]);
+        if (tid % 32 == 0) {
+            atomicAdd(&s_sum[c], w);
+            atomicAdd(&s_zero[c], z);
+        }
+    }
+    __syncthreads();
+    if (tid == 0) {
+        *done = 0;
+        const float d = hll_count(s_sum[2], s_zero[2]);
+        const float half = 0.5f * (hll_count(s_sum[0], s_zero[0]) + hll_count(s_sum[1], s_zero[1]));
+        float most = 1.1f * d;
+        if (rate > 1) most = d + 14.0f * (fmaxf(d - half, 0.0f) + 0.04f * d);  // with two errors' room
+        const uint64_t want = static_cast<uint64_t>(2.5f * most) + kMinHashSlots;
+        *h.chosen = static_cast<uint32_t>(want < h.slots ? want / kBucketSlots * kBucketSlots : h.slots);
+    }
+}
+
+__global__ void hash_clear_kernel(HTable h) {
+    wait_prior();  // the slots chosen
+    hash_clear(h, *static_cast<volatile uint32_t*>(h.chosen), static_cast<size_t>(blockIdx.x) * blockDim.x + threadIdx.x,
+               static_cast<size_t>(gridDim.x) * blockDim.x);
 }
 
 // Dense modes: kDenseBlock (block arrays) and kDenseDirect (rows straight into the
@@ -1585,7 +1743,6 @@ uint32_t gtable_slots(int64_t max_groups) {
 // now 308; 100,000 208 and 207; 30,000 200 and 206). Not fewer than kMinHashSlots, so that a
 // small capacity that is exceeded still gets a full count of a few thousand groups; as many
 // as 32-bit slot numbers hold.
-constexpr uint64_t kMinHashSlots = 8192;
 uint32_t htable_slots(int64_t max_groups, int naggs) {
     const uint64_t m = static_cast<uint64_t>(max_groups);
     uint64_t s = m + m / 2;
@@ -1610,6 +1767,11 @@ int acc_shift(int naggs) { return naggs <= 1 ? 0 : (naggs == 2 ? 1 : (naggs <= 4
 size_t htable_bytes(uint32_t slots, int naggs) {
     return align_up(8 * (static_cast<size_t>(slots) + 1), 256) + (8 * (static_cast<size_t>(slots) + 1) << acc_shift(naggs));
 }
+// A table that takes more than this to clear is used as far as an estimate of the groups
+// says (with 3 aggregates from a capacity of about 1M on). The estimate and its kernels take
+// about as long as clearing and scanning 96 MB (10M rows in 100 groups: capacity 1M, without,
+// 117 us; capacity 10M, with it, 115).
+constexpr size_t kLooseBytes = 96 << 20;
 constexpr size_t kEmittedBytes = 256;  // HTable::emitted and done, before the table
 
 int num_sms() {
@@ -1665,10 +1827,10 @@ px_status launch_runs(const Spec& sp, size_t smem, const int64_t* d_n, int64_t n
     return check_launch("px_groupby_agg runs");
 }
 
-template <int NA>
+template <int NA, bool LOOSE>
 px_status launch_hash(const Spec& sp, const int32_t* sel, const int64_t* d_n, int64_t ncap, const int64_t* d_seg,
                       const HTable& h, cudaStream_t st) {
-    auto kernel = groupby_hash_kernel<NA>;
+    auto kernel = groupby_hash_kernel<NA, LOOSE>;
     const uint32_t C = cache_slots(sp.naggs);
     const size_t smem = static_cast<size_t>(C) * (8 + 8 * static_cast<size_t>(sp.naggs));
     allow_smem(kernel, smem);
@@ -1888,28 +2050,39 @@ static px_status groupby_impl(const px_batch* in, const int32_t* key_cols, int32
         h.acc = reinterpret_cast<unsigned long long*>(keys + align_up(8 * (static_cast<size_t>(slots) + 1), 256));
         h.slots = slots;
         h.shift = acc_shift(naggs);
-        if (!accumulate) cudaMemsetAsync(base, 0, kEmittedBytes + 32 + htable_bytes(slots, naggs), st);
+        h.chosen = reinterpret_cast<uint32_t*>(base + 16);
+        const bool loose = !streaming && htable_bytes(slots, naggs) > kLooseBytes;
+        if (!accumulate)
+            cudaMemsetAsync(base, 0, kEmittedBytes + 32 + (loose ? kEstBytes : htable_bytes(slots, naggs)), st);
         const int64_t* d_n = d_sel ? d_nsel : in->d_nrows;
         if (ncap > 0) {
             const auto go = [&](auto launch) { return launch(sp, d_sel, d_n, ncap, d_seg, h, st); };
+            if (loose) {
+                const int64_t tiles = cdiv(cdiv(ncap, kEstTile), ncap >= kEstAll ? kEstRate : 1);
+                hash_estimate_kernel<<<static_cast<unsigned>(std::min<int64_t>(tiles, num_sms())), kEstThreads, 0, st>>>(
+                    sp, d_sel, d_n, ncap, d_seg, h, reinterpret_cast<uint32_t*>(keys), h.done);
+                note_launch();
+                launch_after(hash_clear_kernel, dim3(num_sms() * 8), dim3(256), 0, st, h);
+                note_launch();
+            }
             switch (naggs) {
-                case 0: s = go(launch_hash<0>); break;
-                case 1: s = go(launch_hash<1>); break;
-                case 2: s = go(launch_hash<2>); break;
-                case 3: s = go(launch_hash<3>); break;
-                case 4: s = go(launch_hash<4>); break;
-                default: s = go(launch_hash<PX_MAX_AGGS>); break;
+                case 0: s = loose ? go(launch_hash<0, true>) : go(launch_hash<0, false>); break;
+                case 1: s = loose ? go(launch_hash<1, true>) : go(launch_hash<1, false>); break;
+                case 2: s = loose ? go(launch_hash<2, true>) : go(launch_hash<2, false>); break;
+                case 3: s = loose ? go(launch_hash<3, true>) : go(launch_hash<3, false>); break;
+                case 4: s = loose ? go(launch_hash<4, true>) : go(launch_hash<4, false>); break;
+                default: s = loose ? go(launch_hash<PX_MAX_AGGS, true>) : go(launch_hash<PX_MAX_AGGS, false>); break;
             }
             if (s != PX_OK) return s;
         }
-        // (launch_after only behind a kernel: with no rows the work before is a memset)
-        const dim3 grid(static_cast<unsigned>(cdiv(static_cast<int64_t>(slots) + 1, kEmitTile)));
-        if (ncap > 0)
-            launch_after(hash_emit_kernel, grid, dim3(kEmitThreads), 0, st, sp, h, max_groups, d_out_seg, d_ngroups,
-                         status, d_sel, d_n, ncap, d_seg);
+        const int64_t tiles = cdiv(static_cast<int64_t>(slots) + 1, kEmitTile);
+        const dim3 grid(static_cast<unsigned>(loose ? std::min<int64_t>(tiles, num_sms() * 4) : tiles));
+        const auto emit = loose ? hash_emit_kernel<true> : hash_emit_kernel<false>;
+        if (ncap > 0)  // launch_after only behind a kernel: with no rows the work before is a memset
+            launch_after(emit, grid, dim3(kEmitThreads), 0, st, sp, h, max_groups, d_out_seg, d_ngroups, status, d_sel,
+                         d_n, ncap, d_seg);
         else
-            hash_emit_kernel<<<grid, kEmitThreads, 0, st>>>(sp, h, max_groups, d_out_seg, d_ngroups, status, d_sel, d_n,
-                                                            ncap, d_seg);
+            emit<<<grid, kEmitThreads, 0, st>>>(sp, h, max_groups, d_out_seg, d_ngroups, status, d_sel, d_n, ncap, d_seg);
         note_launch();
         return check_launch("px_groupby_agg hash emit");
     }
