@@ -13,12 +13,15 @@
 // straight into the output columns.
 // Without such a statistic: groupby_hash_kernel, an open-addressing table of keys and
 // accumulators in the workspace with a small block-local cache in front of it, and
-// hash_emit_kernel, which writes its groups out.
+// hash_emit_kernel, which writes its groups out. Of a table for many groups only as much is
+// used as an estimate says (hash_estimate_kernel); in a stream of calls a group keeps its
+// output row, and small calls write out the groups that they touch (hash_emit_marked_kernel).
 // Rows of one warp with lane 0's group are first combined across the warp, so a hot
 // key costs one update per warp, not 32.
 // All arithmetic is mod 2^64. Every thread loads all of its rows' inputs for a
 // tile before aggregating any of them, so each thread keeps many loads in flight.
 #include <algorithm>
+#include <type_traits>
 
 #include "px_common.cuh"
 #include "px_table.cuh"
@@ -655,7 +658,9 @@ struct HTable {
     unsigned long long* key;  // [slots + 1], 32-byte aligned
     unsigned long long* acc;  // [slots + 1] << shift
     uint32_t slots;           // a multiple of kBucketSlots
-    uint32_t* chosen;         // LOOSE: the slots that are used (see hash_estimate_kernel)
+    uint32_t* chosen;         // kLoose: the slots that are used (see hash_estimate_kernel)
+    uint32_t* row;            // a stream's: [slots + 1], 1 + the slot's output row, 0 where it has none yet
+    uint32_t* touched;        // a stream's: one bit per slot, zero between calls
     int32_t shift;
 };
 
@@ -666,6 +671,9 @@ constexpr int kHashBlocksPerSm = 2;
 constexpr size_t kCacheBudget = 64 * 1024;  // the block-local cache
 constexpr int kHashMajority = 12;           // smallest group worth a warp reduction here
 constexpr uint32_t kNoSlot = 0xffffffffu;
+// How a call uses the table: whole; as far as chosen on the device; a stream's, whose
+// groups keep their output rows, all written out or (kMarked) those that the call touches.
+constexpr int kWhole = 0, kLoose = 1, kStream = 2, kMarked = 3;
 constexpr uint32_t kBucketSlots = 4;
 constexpr uint64_t kMinHashSlots = 8192;    // see htable_slots
 
@@ -733,6 +741,15 @@ __device__ __forceinline__ void note_lost(const HTable& h) {
     if (!(*static_cast<volatile unsigned long long*>(h.emitted) & kLostBit)) atomicOr(h.emitted, kLostBit);
 }
 
+// Marks a slot for the emit of a stream's small call.
+__device__ __forceinline__ void mark_touched(const HTable& h, uint32_t slot) {
+    uint32_t* w = &h.touched[slot / 32];
+    const uint32_t bit = 1u << (slot % 32);
+    uint32_t now;  // from L2: a line in L1 would not show the marks of this call
+    asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(now) : "l"(w) : "memory");
+    if (!(now & bit)) atomicOr(w, bit);
+}
+
 // Two neighbouring 64-bit words of shared memory, read anew.
 __device__ __forceinline__ ulonglong2 ld_shared_pair(const unsigned long long* p) {
     ulonglong2 v;
@@ -763,13 +780,13 @@ __device__ __forceinline__ uint32_t cache_claim(unsigned long long* c_key, uint3
 // 207 us, Zipf(1.1) 1209 -> 153; 3000 groups 833 -> 152; 1M groups 1469 -> 353; 100
 // groups 97 -> 94. A cache slot pair is read with one 16-byte load and a bucket with
 // one 32-byte load; single-slot probing took 408 us at 100,000 groups.
-// LOOSE: the table's slots were chosen on the device.
-template <int NA, bool LOOSE>
+// MODE: kWhole (for kStream too), kLoose or kMarked.
+template <int NA, int MODE>
 __global__ void __launch_bounds__(kHashThreads, kHashBlocksPerSm)
 groupby_hash_kernel(Spec sp, const int32_t* __restrict__ sel, const int64_t* __restrict__ d_n, int64_t ncap,
                     const int64_t* __restrict__ d_seg, HTable h, uint32_t cache_slots) {
     extern __shared__ __align__(16) unsigned char smem[];
-    if (LOOSE) h.slots = *h.chosen;
+    if (MODE == kLoose) h.slots = *h.chosen;
     const uint32_t C = cache_slots;
     unsigned long long* c_key = reinterpret_cast<unsigned long long*>(smem);  // [C], ~code or 0
     uint32_t* c_lo = reinterpret_cast<uint32_t*>(c_key + C);                  // [naggs][C]
@@ -893,6 +910,7 @@ groupby_hash_kernel(Spec sp, const int32_t* __restrict__ sel, const int64_t* __r
                     if (slot == kNoSlot) {
                         note_lost(h);
                     } else {
+                        if (MODE == kMarked) mark_touched(h, slot);
                         unsigned long long* acc = h.acc + (static_cast<size_t>(slot) << h.shift);
 #pragma unroll
                         for (int a = 0; a < NA; ++a) {
@@ -912,6 +930,7 @@ groupby_hash_kernel(Spec sp, const int32_t* __restrict__ sel, const int64_t* __r
             uint32_t slot = bucket_slot(h, home, load_keys(h, home), ci);
             if (slot == kNoSlot) slot = hash_walk(h, home, ci);
             if (slot == kNoSlot) note_lost(h);
+            else if (MODE == kMarked) mark_touched(h, slot);
             for (int a = 0; a < sp.naggs; ++a) {
                 const uint32_t o = static_cast<uint32_t>(a) * C + c;
                 const uint64_t x = (static_cast<uint64_t>(c_hi[o]) << 32) | c_lo[o];
@@ -985,9 +1004,9 @@ __device__ void hash_lost(const Spec& sp, const int32_t* sel, int64_t n, const i
     __syncthreads();
 }
 
-// Writes out the groups in tile `tile` of the table's slots, from the output row that
-// first_row(groups in the tile) gives thread 0 on.
-template <typename F>
+// Writes out the groups in tile `tile` of the table's slots: those without an output row
+// (in a stream, the new ones) from the one that first_row(their number) gives thread 0 on.
+template <bool STREAM, typename F>
 __device__ __forceinline__ void hash_emit_tile(const Spec& sp, const HTable& h, int64_t tile, int64_t max_groups,
                                                int32_t* out_seg, int32_t* s_warp, int64_t* s_base, F first_row) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -996,11 +1015,13 @@ __device__ __forceinline__ void hash_emit_tile(const Spec& sp, const HTable& h, 
     unsigned long long key[kEmitItems];
 #pragma unroll
     for (int i = 0; i < kEmitItems; ++i) key[i] = base + i * 32 < nslots ? h.key[base + i * 32] : 0;
+    uint32_t had[kEmitItems];  // STREAM: the output row from earlier calls, as in HTable::row
     uint32_t mask[kEmitItems];
     int32_t cnt = 0;
 #pragma unroll
     for (int i = 0; i < kEmitItems; ++i) {
-        mask[i] = __ballot_sync(FULL, key[i] != 0);
+        had[i] = STREAM && key[i] != 0 ? h.row[base + i * 32] : 0;
+        mask[i] = __ballot_sync(FULL, key[i] != 0 && had[i] == 0);
         cnt += __popc(mask[i]);
     }
     if (lane == 0) s_warp[warp] = cnt;
@@ -1021,9 +1042,11 @@ __device__ __forceinline__ void hash_emit_tile(const Spec& sp, const HTable& h, 
 #pragma unroll
     for (int i = 0; i < kEmitItems; ++i) {
         p[i] = pos + __popc(mask[i] & lt);
+        if (STREAM && had[i]) p[i] = had[i] - 1;
+        if (STREAM && key[i] != 0 && !had[i]) h.row[base + i * 32] = static_cast<uint32_t>(p[i]) + 1;
         if (key[i] == 0 || p[i] >= max_groups) p[i] = -1;
         pos += __popc(mask[i]);
-        if (p[i] >= 0) {
+        if (p[i] >= 0 && !had[i]) {
             const uint64_t code = base + i * 32 == nslots - 1 ? ~0ull : ~key[i];
             write_group(sp, code, static_cast<int32_t>(p[i]), out_seg);
         }
@@ -1057,6 +1080,7 @@ __device__ void hash_clear(const HTable& h, uint32_t slots, size_t i, size_t n) 
 // exceed the output, that is the result; else (keys chosen to meet in one place) the last
 // block to be done adds the lost rows and writes all groups out anew. Where the slots were
 // chosen by an estimate, that was too low: the block makes the table of all `most` slots.
+template <bool STREAM>
 __device__ __noinline__ void hash_emit_lost(const Spec& sp, const HTable& used, uint32_t most, uint32_t blocks,
                                             int64_t max_groups, int32_t* out_seg, int64_t* d_ngroups, int32_t* status,
                                             const int32_t* sel, const int64_t* d_n, int64_t ncap,
@@ -1084,26 +1108,42 @@ __device__ __noinline__ void hash_emit_lost(const Spec& sp, const HTable& used, 
         __syncthreads();
     }
     hash_lost(sp, sel, actual_rows(d_n, ncap), d_seg, h, anew, groups, max_groups, status);
-    int64_t run = 0;
+    int64_t run = STREAM ? groups : 0;
     for (int64_t tile = 0; tile < cdiv(static_cast<int64_t>(h.slots) + 1, kEmitTile); ++tile) {
-        hash_emit_tile(sp, h, tile, max_groups, out_seg, s_warp, &s_base, [&](int32_t total) {
+        hash_emit_tile<STREAM>(sp, h, tile, max_groups, out_seg, s_warp, &s_base, [&](int32_t total) {
             run += total;
             return run - total;
         });
         __syncthreads();
     }
     if (threadIdx.x == 0) {
+        if (STREAM) *h.emitted = static_cast<unsigned long long>(run);
         *d_ngroups = run;
         if (run > max_groups) set_status(status, PX_ERR_CAPACITY);
     }
 }
 
-// Writes the table's groups out, in no particular order: each tile's output rows are taken
-// with one add to *h.emitted, whose low bits count groups, whose high bits count tiles and
-// whose highest bit tells of lost rows; the last tile's block writes the total and clears it.
-// A block per tile, or (LOOSE) as many as are in flight at a time.
+// A block's add to *h.emitted for `total` more groups, as one of `parts`; called by one
+// thread. Gives the first of their output rows. The low bits count groups (a stream's stay
+// from call to call), the high bits parts, and the highest bit tells of lost rows; the last
+// part writes the number of groups and clears the rest.
 constexpr int kEmittedBits = 40;
-template <bool LOOSE>
+__device__ __forceinline__ int64_t take_rows(const HTable& h, int32_t total, int64_t parts, int64_t max_groups,
+                                             bool* s_lost, int64_t* d_ngroups, int32_t* status) {
+    const unsigned long long old = atomicAdd(h.emitted, (1ull << kEmittedBits) | static_cast<unsigned long long>(total));
+    const int64_t first = static_cast<int64_t>(old & ((1ull << kEmittedBits) - 1));
+    *s_lost = (old & kLostBit) != 0;
+    if (static_cast<int64_t>((old & ~kLostBit) >> kEmittedBits) == parts - 1) {
+        *h.emitted = static_cast<unsigned long long>(first + total);
+        *d_ngroups = first + total;
+        if (first + total > max_groups) set_status(status, PX_ERR_CAPACITY);
+    }
+    return first;
+}
+
+// Writes the table's groups out, in no particular order. A block per tile, or (kLoose) as
+// many as are in flight at a time. MODE: kWhole, kLoose or kStream.
+template <int MODE>
 __global__ void __launch_bounds__(kEmitThreads, 4)
 hash_emit_kernel(const __grid_constant__ Spec sp, const __grid_constant__ HTable h0, int64_t max_groups,
                  int32_t* __restrict__ out_seg, int64_t* d_ngroups, int32_t* status, const int32_t* __restrict__ sel,
@@ -1114,30 +1154,67 @@ hash_emit_kernel(const __grid_constant__ Spec sp, const __grid_constant__ HTable
     wait_prior();  // the table
     HTable h = h0;
     int64_t tiles = gridDim.x;
-    if (LOOSE) {
+    if (MODE == kLoose) {
         h.slots = *h.chosen;
         tiles = cdiv(static_cast<int64_t>(h.slots) + 1, kEmitTile);
         if (blockIdx.x >= tiles) return;
     }
     for (int64_t tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
-        if (LOOSE) __syncthreads();  // the tile before has read s_warp and s_base
-        hash_emit_tile(sp, h, tile, max_groups, out_seg, s_warp, &s_base, [&](int32_t total) {
-            const unsigned long long old =
-                atomicAdd(h.emitted, (1ull << kEmittedBits) | static_cast<unsigned long long>(total));
-            const int64_t first = static_cast<int64_t>(old & ((1ull << kEmittedBits) - 1));
-            s_lost = (old & kLostBit) != 0;
-            if (static_cast<int64_t>((old & ~kLostBit) >> kEmittedBits) == tiles - 1) {
-                *h.emitted = 0;
-                *d_ngroups = first + total;
-                if (first + total > max_groups) set_status(status, PX_ERR_CAPACITY);
-            }
-            return first;
+        if (MODE == kLoose) __syncthreads();  // the tile before has read s_warp and s_base
+        hash_emit_tile<MODE == kStream>(sp, h, tile, max_groups, out_seg, s_warp, &s_base, [&](int32_t total) {
+            return take_rows(h, total, tiles, max_groups, &s_lost, d_ngroups, status);
         });
-        if (!LOOSE) break;
+        if (MODE != kLoose) break;
     }
     if (s_lost)
-        hash_emit_lost(sp, h, h0.slots, static_cast<uint32_t>(gridDim.x < tiles ? gridDim.x : tiles), max_groups, out_seg,
-                       d_ngroups, status, sel, d_n, ncap, d_seg);
+        hash_emit_lost<MODE == kStream>(sp, h, h0.slots, static_cast<uint32_t>(gridDim.x < tiles ? gridDim.x : tiles),
+                                        max_groups, out_seg, d_ngroups, status, sel, d_n, ncap, d_seg);
+}
+
+// The emit of a stream's small call: a thread per 32 slots, which writes out those that the
+// call touched (10,000 rows a call, capacity 10M, 8M groups: 224 us a call with all groups
+// written out, now 52).
+__global__ void __launch_bounds__(kEmitThreads)
+hash_emit_marked_kernel(const __grid_constant__ Spec sp, const __grid_constant__ HTable h, int64_t max_groups,
+                        int32_t* __restrict__ out_seg, int64_t* d_ngroups, int32_t* status,
+                        const int32_t* __restrict__ sel, const int64_t* __restrict__ d_n, int64_t ncap,
+                        const int64_t* __restrict__ d_seg) {
+    __shared__ int32_t s_warp[kEmitWarps];
+    __shared__ int64_t s_base;
+    __shared__ bool s_lost;
+    wait_prior();  // the table
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int64_t w = static_cast<int64_t>(blockIdx.x) * kEmitThreads + tid;
+    const uint32_t word = w * 32 <= h.slots ? h.touched[w] : 0;
+    int32_t fresh = 0;
+    for (uint32_t b = word; b; b &= b - 1) fresh += h.row[w * 32 + __ffs(b) - 1] == 0;
+    const int32_t incl = warp_incl_scan(fresh);
+    if (lane == 31) s_warp[warp] = incl;
+    __syncthreads();
+    if (tid == 0) {
+        int32_t total = 0;
+        for (int k = 0; k < kEmitWarps; ++k) {
+            const int32_t c = s_warp[k];
+            s_warp[k] = total;
+            total += c;
+        }
+        s_base = take_rows(h, total, gridDim.x, max_groups, &s_lost, d_ngroups, status);
+    }
+    __syncthreads();
+    int64_t pos = s_base + s_warp[warp] + incl - fresh;
+    for (uint32_t b = word; b; b &= b - 1) {
+        const int64_t slot = w * 32 + __ffs(b) - 1;
+        const uint32_t had = h.row[slot];
+        const int64_t p = had ? had - 1 : pos++;
+        if (!had) h.row[slot] = static_cast<uint32_t>(p) + 1;
+        if (p >= max_groups) continue;
+        if (!had) write_group(sp, slot == h.slots ? ~0ull : ~h.key[slot], static_cast<int32_t>(p), out_seg);
+        for (int a = 0; a < sp.naggs; ++a)
+            sp.agg_out[a][p] = static_cast<int64_t>(h.acc[(static_cast<size_t>(slot) << h.shift) + a]);
+    }
+    if (word) h.touched[w] = 0;
+    if (s_lost)
+        hash_emit_lost<true>(sp, h, h.slots, gridDim.x, max_groups, out_seg, d_ngroups, status, sel, d_n, ncap, d_seg);
 }
 
 // How many slots the table of a large capacity uses: cleared and scanned whole it may cost
@@ -1743,11 +1820,11 @@ uint32_t gtable_slots(int64_t max_groups) {
 // now 308; 100,000 208 and 207; 30,000 200 and 206). Not fewer than kMinHashSlots, so that a
 // small capacity that is exceeded still gets a full count of a few thousand groups; as many
 // as 32-bit slot numbers hold.
-uint32_t htable_slots(int64_t max_groups, int naggs) {
+uint32_t htable_slots(int64_t max_groups, int naggs, bool stream) {
     const uint64_t m = static_cast<uint64_t>(max_groups);
-    uint64_t s = m + m / 2;
+    uint64_t s = stream ? m * 145 / 100 : m + m / 2;
     if (naggs <= 4) {
-        s = 2 * m + m / 2;
+        s = 2 * m + (stream ? m / 4 : m / 2);
         if (m <= 1 << 16) s = std::max<uint64_t>(s, gtable_slots(max_groups));
     }
     return static_cast<uint32_t>(std::min<uint64_t>(align_up(std::max(s, kMinHashSlots), kBucketSlots), 0xfffffff0u));
@@ -1763,15 +1840,25 @@ uint32_t cache_slots(int naggs) {
 // log2 of a table slot's accumulators, rounded up to a power of two.
 int acc_shift(int naggs) { return naggs <= 1 ? 0 : (naggs == 2 ? 1 : (naggs <= 4 ? 2 : 3)); }
 
-// The table of the hash mode: slots, and bytes with naggs accumulators each.
-size_t htable_bytes(uint32_t slots, int naggs) {
-    return align_up(8 * (static_cast<size_t>(slots) + 1), 256) + (8 * (static_cast<size_t>(slots) + 1) << acc_shift(naggs));
+// The table of the hash mode: the offsets of its parts from the keys on, and its bytes.
+struct HTableLayout {
+    size_t acc, row, touched, total;
+};
+HTableLayout htable_layout(uint32_t slots, int naggs, bool stream) {
+    const size_t n = static_cast<size_t>(slots) + 1;
+    HTableLayout L;
+    L.acc = align_up(8 * n, 256);
+    L.row = L.acc + align_up(8 * n << acc_shift(naggs), 256);
+    L.touched = L.row + (stream ? align_up(4 * n, 256) : 0);
+    L.total = L.touched + (stream ? align_up(cdiv(n, 32) * 4, 256) : 0);
+    return L;
 }
 // A table that takes more than this to clear is used as far as an estimate of the groups
 // says (with 3 aggregates from a capacity of about 1M on). The estimate and its kernels take
 // about as long as clearing and scanning 96 MB (10M rows in 100 groups: capacity 1M, without,
 // 117 us; capacity 10M, with it, 115).
 constexpr size_t kLooseBytes = 96 << 20;
+constexpr uint32_t kMarkedSlots = 1 << 19;  // see groupby_impl
 constexpr size_t kEmittedBytes = 256;  // HTable::emitted and done, before the table
 
 int num_sms() {
@@ -1827,10 +1914,10 @@ px_status launch_runs(const Spec& sp, size_t smem, const int64_t* d_n, int64_t n
     return check_launch("px_groupby_agg runs");
 }
 
-template <int NA, bool LOOSE>
+template <int NA, int MODE>
 px_status launch_hash(const Spec& sp, const int32_t* sel, const int64_t* d_n, int64_t ncap, const int64_t* d_seg,
                       const HTable& h, cudaStream_t st) {
-    auto kernel = groupby_hash_kernel<NA, LOOSE>;
+    auto kernel = groupby_hash_kernel<NA, MODE>;
     const uint32_t C = cache_slots(sp.naggs);
     const size_t smem = static_cast<size_t>(C) * (8 + 8 * static_cast<size_t>(sp.naggs));
     allow_smem(kernel, smem);
@@ -1869,7 +1956,9 @@ WsLayout ws_layout(int64_t max_groups) {
     L.gidx = L.key + align_up(8 * G, 256);
     L.total = L.gidx + align_up(4 * G, 256);
     for (int naggs : {4, PX_MAX_AGGS})
-        L.total = std::max(L.total, kWsScratch + kEmittedBytes + 32 + htable_bytes(htable_slots(max_groups, naggs), naggs));
+        for (bool stream : {false, true})
+            L.total = std::max(L.total, kWsScratch + kEmittedBytes + 32 +
+                                            htable_layout(htable_slots(max_groups, naggs, stream), naggs, stream).total);
     return L;
 }
 
@@ -2039,25 +2128,30 @@ static px_status groupby_impl(const px_batch* in, const int32_t* key_cols, int32
     if (!sp.dense) {
         // Hash mode. A stream of calls keeps one table, so its size must not depend on a
         // call's rows.
-        const uint32_t slots = htable_slots(streaming ? max_groups : std::min(max_groups, ncap), naggs);
+        const uint32_t slots = htable_slots(streaming ? max_groups : std::min(max_groups, ncap), naggs, streaming);
+        const HTableLayout T = htable_layout(slots, naggs, streaming);
         char* base = static_cast<char*>(d_ws) + kWsScratch;
+        // a bucket is one 32-byte load; the caller's workspace is only 16-byte aligned
+        char* keys = reinterpret_cast<char*>(align_up(reinterpret_cast<uintptr_t>(base) + kEmittedBytes, 32));
         HTable h;
         h.emitted = reinterpret_cast<unsigned long long*>(base);
         h.done = reinterpret_cast<uint32_t*>(base + 8);
-        // a bucket is one 32-byte load; the caller's workspace is only 16-byte aligned
-        char* keys = reinterpret_cast<char*>(align_up(reinterpret_cast<uintptr_t>(base) + kEmittedBytes, 32));
+        h.chosen = reinterpret_cast<uint32_t*>(base + 16);
         h.key = reinterpret_cast<unsigned long long*>(keys);
-        h.acc = reinterpret_cast<unsigned long long*>(keys + align_up(8 * (static_cast<size_t>(slots) + 1), 256));
+        h.acc = reinterpret_cast<unsigned long long*>(keys + T.acc);
+        h.row = streaming ? reinterpret_cast<uint32_t*>(keys + T.row) : nullptr;
+        h.touched = streaming ? reinterpret_cast<uint32_t*>(keys + T.touched) : nullptr;
         h.slots = slots;
         h.shift = acc_shift(naggs);
-        h.chosen = reinterpret_cast<uint32_t*>(base + 16);
-        const bool loose = !streaming && htable_bytes(slots, naggs) > kLooseBytes;
-        if (!accumulate)
-            cudaMemsetAsync(base, 0, kEmittedBytes + 32 + (loose ? kEstBytes : htable_bytes(slots, naggs)), st);
+        // A stream's call of few rows marks the groups that it touches; one of many, or into a
+        // small table, writes all groups out (10,000 rows: 281,000 slots 41 us marked, 36 all;
+        // 2.8M slots 41 and 63; 1M rows into 22.5M slots 208 and 308).
+        const int mode = !streaming ? (T.total > kLooseBytes ? kLoose : kWhole)
+                                    : (slots > kMarkedSlots && ncap < static_cast<int64_t>(slots) / 8 ? kMarked : kStream);
+        if (!accumulate) cudaMemsetAsync(base, 0, kEmittedBytes + 32 + (mode == kLoose ? kEstBytes : T.total), st);
         const int64_t* d_n = d_sel ? d_nsel : in->d_nrows;
         if (ncap > 0) {
-            const auto go = [&](auto launch) { return launch(sp, d_sel, d_n, ncap, d_seg, h, st); };
-            if (loose) {
+            if (mode == kLoose) {
                 const int64_t tiles = cdiv(cdiv(ncap, kEstTile), ncap >= kEstAll ? kEstRate : 1);
                 hash_estimate_kernel<<<static_cast<unsigned>(std::min<int64_t>(tiles, num_sms())), kEstThreads, 0, st>>>(
                     sp, d_sel, d_n, ncap, d_seg, h, reinterpret_cast<uint32_t*>(keys), h.done);
@@ -2065,19 +2159,29 @@ static px_status groupby_impl(const px_batch* in, const int32_t* key_cols, int32
                 launch_after(hash_clear_kernel, dim3(num_sms() * 8), dim3(256), 0, st, h);
                 note_launch();
             }
+            const auto go = [&](auto na) {
+                constexpr int NA = decltype(na)::value;
+                const auto launch = mode == kLoose ? launch_hash<NA, kLoose>
+                                                   : (mode == kMarked ? launch_hash<NA, kMarked> : launch_hash<NA, kWhole>);
+                return launch(sp, d_sel, d_n, ncap, d_seg, h, st);
+            };
             switch (naggs) {
-                case 0: s = loose ? go(launch_hash<0, true>) : go(launch_hash<0, false>); break;
-                case 1: s = loose ? go(launch_hash<1, true>) : go(launch_hash<1, false>); break;
-                case 2: s = loose ? go(launch_hash<2, true>) : go(launch_hash<2, false>); break;
-                case 3: s = loose ? go(launch_hash<3, true>) : go(launch_hash<3, false>); break;
-                case 4: s = loose ? go(launch_hash<4, true>) : go(launch_hash<4, false>); break;
-                default: s = loose ? go(launch_hash<PX_MAX_AGGS, true>) : go(launch_hash<PX_MAX_AGGS, false>); break;
+                case 0: s = go(std::integral_constant<int, 0>{}); break;
+                case 1: s = go(std::integral_constant<int, 1>{}); break;
+                case 2: s = go(std::integral_constant<int, 2>{}); break;
+                case 3: s = go(std::integral_constant<int, 3>{}); break;
+                case 4: s = go(std::integral_constant<int, 4>{}); break;
+                default: s = go(std::integral_constant<int, PX_MAX_AGGS>{}); break;
             }
             if (s != PX_OK) return s;
         }
-        const int64_t tiles = cdiv(static_cast<int64_t>(slots) + 1, kEmitTile);
-        const dim3 grid(static_cast<unsigned>(loose ? std::min<int64_t>(tiles, num_sms() * 4) : tiles));
-        const auto emit = loose ? hash_emit_kernel<true> : hash_emit_kernel<false>;
+        int64_t blocks = cdiv(static_cast<int64_t>(slots) + 1, mode == kMarked ? 32 * kEmitThreads : kEmitTile);
+        if (mode == kLoose) blocks = std::min<int64_t>(blocks, num_sms() * 4);
+        const auto emit = mode == kLoose    ? hash_emit_kernel<kLoose>
+                          : mode == kMarked ? hash_emit_marked_kernel
+                          : mode == kStream ? hash_emit_kernel<kStream>
+                                            : hash_emit_kernel<kWhole>;
+        const dim3 grid(static_cast<unsigned>(blocks));
         if (ncap > 0)  // launch_after only behind a kernel: with no rows the work before is a memset
             launch_after(emit, grid, dim3(kEmitThreads), 0, st, sp, h, max_groups, d_out_seg, d_ngroups, status, d_sel,
                          d_n, ncap, d_seg);
