@@ -191,8 +191,8 @@ px_status px_partition(const px_batch* in, int32_t key_col,
 
 /* Launch shape of px_partition: rows per thread in a tile of 256 threads (2, 4 or
  * 8, capped at the widest whose tile of every column fits the 48 KB staging
- * area; 0 = that widest, or the library's own tile where it does not stage tiles:
- * through a selection, whatever items says, and for many partitions) and the most
+ * area where tiles are staged; 0 = that widest, or the library's own tile where it
+ * does not stage them: through a selection, and for many partitions) and the most
  * resident scatter blocks per SM (0 = as many as fit). Every shape gives the same
  * result; they differ only in speed (an autotuner picks one per GPU and workload). */
 typedef struct {

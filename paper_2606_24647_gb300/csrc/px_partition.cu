@@ -786,16 +786,19 @@ px_status px_partition_tuned(const px_batch* in, int32_t key_col, const int32_t*
     // staging budget, else the widest that fits.
     const int fit = items_for(row_bytes);
     const int staged = items_req > 0 && items_req <= fit ? items_req : fit;
-    // The kernel without staging (see part_direct_kernel): through a selection; with many
-    // partitions, whose short runs make the writes the bound (20M rows, staged against
-    // not: fact columns at 256 partitions 274 and 266 us, at 1024 623 and 599; four 8-byte
-    // columns at 256 471 and 367, at 64 296 and 282, at 16 246 and 273; the six columns of
-    // the plain batch at 200 453 and 366, at 64 300 and 311). A caller's own shape is
-    // staged. Tiles of 1024 rows while 2048 would not give every SM two.
+    // The kernel without staging (see part_direct_kernel): through a selection, in the
+    // caller's rows per thread if given (98 % of 20M fact rows, 8 partitions, 8 rows 229 us, 4
+    // rows 256, 2 rows 294; two blocks per SM 280, staged 333); with many partitions, whose
+    // short runs make the writes the bound (20M rows, staged against not: fact columns at 256
+    // partitions 274 and 266 us, at 1024 623 and 599; four 8-byte columns at 256 471 and 367, at
+    // 64 296 and 282, at 16 246 and 273; the six columns of the plain batch at 200 453 and 366,
+    // at 64 300 and 311). A caller's own shape is staged there. Tiles of 1024 rows while 2048
+    // would not give every SM two.
     const bool shaped = items_req > 0 && items_req <= fit;
     const bool direct =
         d_sel || (!shaped && (nparts > 64 || (nparts > 32 && fit < 8 && static_cast<int>(row_bytes) >= 6 * in->ncols)));
-    const int items = direct ? (ncap >= 2 * 2048 * static_cast<int64_t>(sm_count()) ? 8 : 4) : staged;
+    const int own = ncap >= 2 * 2048 * static_cast<int64_t>(sm_count()) ? 8 : 4;
+    const int items = !direct ? staged : (d_sel && items_req > 0 ? items_req : own);
     const int64_t T = static_cast<int64_t>(kThreads) * items;
     uint32_t stage_bytes = 0;
     for (int c = 0; c < in->ncols; ++c) {
