@@ -212,8 +212,10 @@ def _stream(stream) -> int:
         return stream.cuda_stream
     # torch.cuda.current_stream().cuda_stream without building a Stream (2.8 us a call);
     # a private call, so not relied on
-    raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
-    return torch.cuda.current_stream().cuda_stream if raw is None else raw(torch.cuda.current_device())
+    try:
+        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+    except AttributeError:
+        return torch.cuda.current_stream().cuda_stream
 
 
 def _words(t: torch.Tensor) -> tuple:
