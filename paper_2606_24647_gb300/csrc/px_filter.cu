@@ -13,7 +13,7 @@
 // again.
 // Measured, 60M int32 rows, 30 % kept (312 MB): 154 us when the write pass read the
 // column again behind a one-block scan of the tile counts, now 77 us: the count is
-// DRAM bound (42 us, 5.8 TB/s; 2.8 TB/s when every block read a contiguous run of its
+// DRAM bound (47 us, 5.2 TB/s; 2.8 TB/s when every block read a contiguous run of its
 // own, 12 MB apart), the write issue bound (30 us, 2.8 instructions per cycle). 60M
 // int64 rows: 182 -> 123 us; 1M int32 rows 7.4 -> 4.8 us. Prefetching the next tiles
 // into L2 (up to 60 MB ahead) evicted lines before their use: int64 166 us.
@@ -29,7 +29,9 @@ namespace {
 
 constexpr int kThreads = 128;
 constexpr int kWarps = kThreads / 32;
-constexpr int kBlocksPerSm = 12;       // 1536 resident threads, 42 registers each
+// 1536 resident threads of 40 registers each: the 32-word kernels of int64 columns spill 72
+// bytes (count) and 64 (write), the count of int32 columns 16.
+constexpr int kBlocksPerSm = 12;
 // Words of 32 rows a warp takes per tile: 32, or 8 while one tile of 8 per block
 // holds the rows: a short column then spreads over more warps with fewer serial
 // loads each (10,000 int64 rows: 3.6 us, 7.9 us in 32-word tiles).

@@ -564,7 +564,8 @@ __device__ void aggregate_range_dense(const Spec& sp, const Smem& m, const int32
 // products and at most one COUNT. Each thread takes kItems consecutive rows of a tile aligned to
 // kTile with vector loads (rows outside [a0, a1) masked), so widths are looked at once
 // per column and thread instead of once per value. Issue bound (2.3 instructions per
-// cycle; the loads' latency next). Measured, 20M rows: two int8 keys, 3 sums and COUNT at
+// cycle; the loads' latency next; three sums under two keys spill 128 bytes of the 64
+// registers). Measured, 20M rows: two int8 keys, 3 sums and COUNT at
 // 30M rows 306 -> 189 us; 1000 groups, SUM + SUM_MUL + COUNT 152 -> 109; 2 sums without
 // COUNT, 100 groups 134 -> 104.
 template <int NS, int NK>
@@ -773,13 +774,14 @@ __device__ __forceinline__ uint32_t cache_claim(unsigned long long* c_key, uint3
 // the low bits a slot of the table in the workspace, where the rows the cache does not
 // hold are added with 64-bit reductions. NA: number of aggregates when known at compile
 // time (0..4), or PX_MAX_AGGS.
-// Bound by the 64-bit reductions' L2 traffic where most rows go to the table (L2 81 %
+// Bound by the 64-bit reductions' traffic where most rows go to the table (L1 72 %, L2 69 %
 // busy), else by the latency of the dependent steps at 1024 threads per SM. Measured,
-// 10M rows, int64 keys, SUM + SUM_MUL + COUNT (240 MB), against block tables of 4096
-// slots probed 8 deep in front of a claimed and published table: 100,000 groups 1465 ->
-// 207 us, Zipf(1.1) 1209 -> 153; 3000 groups 833 -> 152; 1M groups 1469 -> 353; 100
-// groups 97 -> 94. A cache slot pair is read with one 16-byte load and a bucket with
-// one 32-byte load; single-slot probing took 408 us at 100,000 groups.
+// whole calls, 10M rows, int64 keys, SUM + SUM_MUL + COUNT (240 MB), capacity a quarter
+// above the groups, against block tables of 4096 slots probed 8 deep in front of a claimed
+// and published table: 100,000 groups 1476 -> 207 us; 1M groups 1480 -> 330; 100 groups 98 ->
+// 97; Zipf(1.1), 100,000 groups (this kernel) 1209 -> 153. A cache slot pair is read with one
+// 16-byte load and a bucket with one 32-byte load; single-slot probing took 408 us at
+// 100,000 groups.
 // MODE: kWhole (for kStream too), kLoose or kMarked.
 template <int NA, int MODE>
 __global__ void __launch_bounds__(kHashThreads, kHashBlocksPerSm)

@@ -4,8 +4,8 @@
 //
 // Table: caller memory with the private layout of px_table.cuh (32-byte buckets
 // of 2 slots: keys, build rows, payload values; segment q owns n_q + 1 buckets, or
-// 2 n_q + 1 in a small table, so every segment runs at load factor < 1/2 or < 1/4
-// with no size known before the build). Linear probing over slots starts at the
+// 2 n_q + 1 or 4 n_q + 1 in smaller tables, so every segment runs at load factor < 1/2,
+// < 1/4 or < 1/8 with no size known before the build). Linear probing over slots starts at the
 // first slot of the key's home bucket: the multiply-shift reduction of the LOWER
 // 32 bits of fmix64(key) (the exchange uses the upper 32) onto the segment's
 // buckets. A lookup reads its home bucket's whole sector (keys, rows and payload
