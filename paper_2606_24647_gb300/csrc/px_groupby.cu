@@ -1224,9 +1224,9 @@ hash_emit_marked_kernel(const __grid_constant__ Spec sp, const __grid_constant__
 // distinct codes by HyperLogLog (Flajolet et al., 2007) in one row in eight, in two halves:
 // as a sample grows its distinct codes grow ever more slowly, so the whole has at most
 // d + 14 (d - h) of them, with d in the sample and h in half of it. A count that is too low
-// all the same (see hash_emit_lost) costs time, not rows.
-// 10M rows, 3 aggregates, capacity 10M: 100 groups 312 us, now 115; 100,000 groups 1004, now
-// 226; 1M groups 1055, now 718; 4.3M groups 1084 and 1096. The estimate itself takes 13 us
+// all the same (see hash_emit_lost) costs time, a block's work on all rows, but no rows.
+// 10M rows, 3 aggregates, capacity 10M: 100 groups 312 us, now 118; 100,000 groups 1004, now
+// 231; 1M groups 1055, now 730; 4.3M groups 1084 and 1088. The estimate itself takes 13 us
 // there, a chain of latencies.
 constexpr int kEstThreads = 1024;
 constexpr int kEstItems = 4;
@@ -1235,6 +1235,9 @@ constexpr int kEstRegs = 2048;       // registers of one count: standard error 2
 constexpr int kEstRate = 8;          // one tile in so many is read,
 constexpr int64_t kEstAll = 1 << 20; // but every one of fewer rows than this
 constexpr size_t kEstBytes = 2 * kEstRegs * 4;
+// Slots beside those asked for: up to 14 tiles in a row, 57,344 rows, go unread, and their codes
+// may occur nowhere else (6M rows, of one key but for 57,344: 66 ms with room for 8192, now 0.14).
+constexpr uint64_t kEstRoom = 1 << 18;
 
 __device__ __forceinline__ float hll_count(float sum, int zero) {
     constexpr float m = kEstRegs;
@@ -1321,7 +1324,7 @@ hash_estimate_kernel(const __grid_constant__ Spec sp, const int32_t* __restrict_
         const float half = 0.5f * (hll_count(s_sum[0], s_zero[0]) + hll_count(s_sum[1], s_zero[1]));
         float most = 1.1f * d;
         if (rate > 1) most = d + 14.0f * (fmaxf(d - half, 0.0f) + 0.04f * d);  // with two errors' room
-        const uint64_t want = static_cast<uint64_t>(2.5f * most) + kMinHashSlots;
+        const uint64_t want = static_cast<uint64_t>(2.5f * most) + kEstRoom;
         *h.chosen = static_cast<uint32_t>(want < h.slots ? want / kBucketSlots * kBucketSlots : h.slots);
     }
 }
@@ -1858,7 +1861,7 @@ HTableLayout htable_layout(uint32_t slots, int naggs, bool stream) {
 // A table that takes more than this to clear is used as far as an estimate of the groups
 // says (with 3 aggregates from a capacity of about 1M on). The estimate and its kernels take
 // about as long as clearing and scanning 96 MB (10M rows in 100 groups: capacity 1M, without,
-// 117 us; capacity 10M, with it, 115).
+// 117 us; capacity 10M, with it, 118).
 constexpr size_t kLooseBytes = 96 << 20;
 constexpr uint32_t kMarkedSlots = 1 << 19;  // see groupby_impl
 constexpr size_t kEmittedBytes = 256;  // HTable::emitted and done, before the table

@@ -93,3 +93,32 @@ def test_loose_capacity_costs_little(px):
             assert count(r["ngroups"]) == groups
         # the whole table cleared and scanned took 3 to 5 times as long
         assert us[n] < 1.7 * us[groups + groups // 4], us
+
+
+def test_codes_that_the_sample_does_not_see(px):
+    """One key in all rows but a stretch of distinct ones between two tiles that the estimate
+    reads: they find room, without the rows being gone through by one block (100 ms)."""
+    def read(t):  # the tile of the t-th eight that is read: MurmurHash3's finalizer of t
+        h, m = t, 2**64 - 1
+        h = (h ^ h >> 33) * 0xff51afd7ed558ccd & m
+        h = (h ^ h >> 33) * 0xc4ceb9fe1a85ec53 & m
+        return t * 8 + (h ^ h >> 33) % 8
+
+    tile, n = 4096, 6_000_000
+    gaps = [(read(t + 1) - read(t) - 1, read(t) + 1) for t in range(n // tile // 8 - 1)]
+    tiles, first = max(gaps)
+    assert tiles >= 9
+    us = {}
+    for burst in (False, True):
+        key = np.full(n, 5, np.int64)
+        if burst:
+            key[first * tile:(first + tiles) * tile] = 1000 + np.arange(tiles * tile)
+        val = np.arange(n, dtype=np.int64)
+        ws = px.Workspace(px.lib().px_groupby_ws_bytes(n, n))
+        out = [torch.empty(n, dtype=torch.int64, device="cuda") for _ in range(3)]
+        cols = [dev(key), dev(val)]
+        us[burst], r = _time(lambda: px.px_groupby_agg(cols, [0], [(px.PX_SUM, 1, None), (px.PX_COUNT, None, None)],
+                                                       max_groups=n, out=out, ws=ws))
+        assert ws.status() == px.PX_OK
+        assert_groups_equal(r, oracle.groupby([key], [(oracle.SUM, val, None), (oracle.COUNT, None, None)]), 1)
+    assert us[True] < 3 * us[False] + 0.1, us
