@@ -288,9 +288,11 @@ typedef struct {
  * `out`: nkeys key columns (same types as the input keys) then naggs PX_I64
  * columns, capacity out->nrows >= max_groups; groups come in an unspecified
  * order. *d_ngroups receives the number of groups; more than max_groups records
- * PX_ERR_CAPACITY. The sum of the key widths plus ceil(log2(nsegs)) bits must not
- * exceed 64 bits (PX_ERR_UNSUPPORTED otherwise). `range` (nullable) is the key
- * statistic described above. A Final merge of Partial results is another
+ * PX_ERR_CAPACITY (the number is exact when it is little above max_groups, else a
+ * lower bound of it that is above max_groups). The sum of the key widths plus
+ * ceil(log2(nsegs)) bits must not exceed 64 bits (PX_ERR_UNSUPPORTED otherwise).
+ * `range` (nullable) is the key statistic described above. A Final merge of
+ * Partial results is another
  * px_groupby_agg over them with PX_SUM of each partial aggregate. */
 px_status px_groupby_agg(const px_batch* in, const int32_t* key_cols, int32_t nkeys,
                          const px_agg* aggs, int32_t naggs,
